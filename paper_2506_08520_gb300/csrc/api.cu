@@ -134,7 +134,11 @@ int nystra_call(const void* q, const void* k, const void* v, void* out, int n_wi
         e = s16 ? nystra_host::launch_nystra_tc_n1024_s16(q, k, v, out, units, d_h, m, iters, pool, dtype, s, bp)
                 : nystra_host::launch_nystra_tc_n1024(q, k, v, out, units, d_h, m, iters, pool, dtype, s, bp);
     else
-        e = nystra_host::launch_nystra_generic(q, k, v, out, units, N, d_h, m, iters, pool, dtype, s, bias);
+        e = (m <= 8    ? nystra_host::launch_nystra_generic_m8
+             : m <= 16 ? nystra_host::launch_nystra_generic_m16
+             : m <= 32 ? nystra_host::launch_nystra_generic_m32
+                       : nystra_host::launch_nystra_generic_m64)(q, k, v, out, units, N, d_h, m, iters, pool, dtype, s,
+                                                                 bias);
     return e == cudaSuccess ? NYSTRA_OK : fail_cuda(e);
 }
 

@@ -86,9 +86,19 @@ cudaError_t persistent_grid(K kern, int threads, size_t smem, std::atomic<int> (
 // Each returns a cudaError_t of the launch.
 namespace nystra_host {
 // pool: landmark pooling, 0 = segments, 1 = square patches of a square window.
-cudaError_t launch_nystra_generic(const void* q, const void* k, const void* v, void* out,
-                                  long long n_units, int N, int d, int m, int iters, int pool, int dtype,
-                                  cudaStream_t stream, const nystra::NystraBias& bias = {});
+// Generic kernel (any shape), one translation unit per landmark bound.
+cudaError_t launch_nystra_generic_m8(const void* q, const void* k, const void* v, void* out, long long n_units, int N,
+                                     int d, int m, int iters, int pool, int dtype, cudaStream_t stream,
+                                     const nystra::NystraBias& bias);
+cudaError_t launch_nystra_generic_m16(const void* q, const void* k, const void* v, void* out, long long n_units, int N,
+                                      int d, int m, int iters, int pool, int dtype, cudaStream_t stream,
+                                      const nystra::NystraBias& bias);
+cudaError_t launch_nystra_generic_m32(const void* q, const void* k, const void* v, void* out, long long n_units, int N,
+                                      int d, int m, int iters, int pool, int dtype, cudaStream_t stream,
+                                      const nystra::NystraBias& bias);
+cudaError_t launch_nystra_generic_m64(const void* q, const void* k, const void* v, void* out, long long n_units, int N,
+                                      int d, int m, int iters, int pool, int dtype, cudaStream_t stream,
+                                      const nystra::NystraBias& bias);
 // Pools bias [n_bias, N, N] into its landmark blocks (bias.cu).
 cudaError_t launch_pool_bias(const float* bias, long long n_bias, int N, int m, int pool, float* bias_L,
                              float* bias_U, float* bias_A, cudaStream_t stream);

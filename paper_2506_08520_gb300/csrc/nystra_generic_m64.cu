@@ -1,0 +1,4 @@
+// Generic PnP-Nystra kernel (nystra_generic.cuh) for up to 64 landmarks.
+#include "nystra_generic.cuh"
+
+NYSTRA_GENERIC_DEFINE(64)
