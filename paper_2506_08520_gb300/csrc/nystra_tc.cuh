@@ -3,8 +3,9 @@
 // tokens (8x8, 16x16, 32x32), m in {8, 16, 32, 64}, even d_h <= 32, 16-bit
 // I/O (fp32 I/O through the operand policy Opnd<float>, used by the 8x8 pool
 // kernel).  Included by one translation unit per N (nystra_tc_n*.cu), which
-// also includes the kernel for its common case: nystra_pool.cuh (8x8, m <=
-// 16), nystra_team.cuh (16x16, m <= 32), nystra_stream.cuh (32x32, m <= 32).
+// also includes the kernels for its common cases: nystra_pool.cuh (8x8, m <=
+// 16), nystra_team.cuh (16x16, m <= 32), nystra_stream.cuh (32x32, m <= 32),
+// nystra_wide.cuh (8x8 and 16x16, m = 64).
 // Compile-time options of those kernels: square-patch landmarks (Pooling,
 // PW > 0) and an additive score bias (BIAS, m <= 16).
 //
@@ -23,14 +24,15 @@
 //   core     G_A^n = exp(Qbar Kbar^T - m_U), Z_0 = A^T/(||A||_1 ||A||_inf),
 //            `iters` steps Z <- Z(13I - X(15I - X(7I - X)))/4 with X = A Z
 //            (step 4), Y = Z W stored as a 16-bit B operand: core_warp (one
-//            warp, in registers, m <= 16) or dist_core (m/16 warps).
+//            warp, in registers, m <= 16), dist_core (m = 32, two warps) or
+//            vc_core (m = 64, four warps; nystra_vcore.cuh).
 //   output   O = (G_L^n Y_:d) / (G_L^n Y_d) (steps 5-7), staged row-major and
 //            written with one bulk store (rows of 60 bytes would otherwise be
 //            written as partial sectors); [P2] S_L and G_L^n recomputed from
 //            a still-resident Q.
 //
-// Grouped kernel (nystra_tc_kernel; every m = 32 or 64 the three kernels
-// above do not take).  A group of token warps owns one unit at a time, plus
+// Grouped kernel (nystra_tc_kernel; m = 32 at 8x8 windows and, with d_h = 32,
+// at 16x16; m = 64 at 32x32).  A group of token warps owns one unit at a time, plus
 // helper warps when the distributed core needs more warps than there are
 // token warps; a CTA holds GROUPS groups and the grid is persistent.  The
 // next unit's Q and K are copied after the combine ([P2]: K only, Q after the
@@ -95,7 +97,7 @@ __host__ __device__ constexpr int mrow() {
 }
 static_assert(row_step(30) == 4 && row_step(28) == 2 && row_step(32) == 1 && row_step(0) == 1, "row steps");
 
-// Shared scratch of the distributed core (m = 32, 64; see dist_core): two
+// Shared scratch of the distributed core (m = 32; see dist_core): two
 // matrices of fp16 pairs (hi plane, then lo plane; rows padded to m + 8
 // halves so ldmatrix is conflict-free) and an auxiliary float area.
 template <int M>
@@ -105,6 +107,21 @@ struct DistScratch {
     static constexpr size_t MAT = 2 * PLANE;
     static constexpr size_t AUX = ((size_t)CW * M * 4 + 4 * CW * 4 + 15) / 16 * 16;  // column sums, maxima
     static constexpr size_t BYTES = ((2 * MAT + AUX + 127) / 128) * 128;
+};
+
+// Shared scratch of the core that carries V (nystra_vcore.cuh): two matrices of fp16 pairs (hi plane, then lo plane; rows
+// padded to m + 8 halves so ldmatrix is conflict-free), V (m rows of 40
+// columns, likewise) and an auxiliary float area.
+template <int M>
+struct VcScratch {
+    static constexpr int CW = M / 16, SS = M + 8, VS = 40;
+    static constexpr size_t PLANE = (size_t)M * SS * 2;
+    static constexpr size_t MAT = 2 * PLANE;
+    static constexpr size_t VPLANE = (size_t)M * VS * 2;
+    static constexpr size_t VMAT = 2 * VPLANE;
+    // column sums of A, maxima, column maxima of V
+    static constexpr size_t AUX = ((size_t)CW * M * 4 + 4 * CW * 4 + CW * VS * 4 + 15) / 16 * 16;
+    static constexpr size_t BYTES = ((2 * MAT + VMAT + AUX + 127) / 128) * 128;  // mat0 | mat1 | V | aux
 };
 
 template <typename T, int M>
@@ -136,12 +153,11 @@ struct Layout {
     // stages (TPW >= 256), the first two token warps' K/V rows (consumed by
     // the combine before the core starts; the next unit's K and V are copied
     // after the core).
-    static constexpr bool SCR_IN_STAGE = (CW > 1) && (TPW >= 256);
+    static constexpr bool SCR_IN_STAGE = M == 64;
     static constexpr bool SCR_IN_GROUP = (CW > 1) && !SCR_IN_STAGE;
     static constexpr size_t SCR_BYTES = SCR_IN_GROUP ? DistScratch<(M > 16 ? M : 32)>::BYTES : 0;
-    static_assert(!SCR_IN_STAGE || (WPU >= 2 && DistScratch<(M > 16 ? M : 32)>::MAT +
-                                                       DistScratch<(M > 16 ? M : 32)>::AUX <=
-                                                   2 * (size_t)TPW * DS * 2),
+    static_assert(!SCR_IN_STAGE || (WPU >= 2 && CW == 4 &&
+                                    VcScratch<64>::MAT + VcScratch<64>::VMAT <= 2 * (size_t)TPW * DS * 2),
                   "scratch must fit in two warps' K/V rows");
     static constexpr size_t QB_BYTES = LmS<T>::bytes(MP);
     static constexpr size_t YT_BYTES = YtS<T, M>::bytes(NCOL);
@@ -1070,7 +1086,7 @@ __device__ __forceinline__ void core_warp(const T* qbar, const T* kbar, const fl
     }
 }
 
-// ---- distributed core for m = 32, 64: CW = m/16 warps, warp c owns rows 16c..16c+15 ----
+// ---- distributed core for m = 32: CW = m/16 warps, warp c owns rows 16c..16c+15 ----
 // The m x m operands no longer fit one warp's registers.  Each warp keeps the
 // A operands of its own rows (X and Z, fp16 pairs) and reads right-hand
 // factors from two shared-memory matrices (hi and lo planes, rows padded to
@@ -1447,6 +1463,14 @@ __device__ __forceinline__ void dist_core(const T* qbar, const T* kbar, const fl
     }
 }
 
+}  // namespace tc
+}  // namespace nystra
+
+#include "nystra_vcore.cuh"
+
+namespace nystra {
+namespace tc {
+
 // Output for one warp's NCH chunks: O = (G_L^n Y_:d) / (G_L^n Y_d) (steps
 // 5-7); G_L^n fragments come from glf (parked) or are recomputed from Qs and
 // Kbar; rows are written row-major to obase (N_w x d), each to its own token
@@ -1569,15 +1593,18 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
     // distributed-core scratch
     unsigned char* mat0 = nullptr;
     unsigned char* mat1 = nullptr;
+    unsigned char* vmat = nullptr;
     float* aux = nullptr;
     if constexpr (CW > 1) {
-        using DSc = DistScratch<(M > 16 ? M : 32)>;
         if constexpr (Lay::SCR_IN_STAGE) {
+            using VSc = VcScratch<64>;
             unsigned char* w0 = smem_raw + (size_t)GROUPS * Lay::GROUP_BYTES + (size_t)(grp * WPU) * Lay::WARP_BYTES;
             mat0 = w0 + Lay::WPART;
-            aux = reinterpret_cast<float*>(mat0 + DSc::MAT);
+            aux = reinterpret_cast<float*>(mat0 + VSc::MAT);
             mat1 = w0 + Lay::WARP_BYTES + Lay::WPART;
+            vmat = mat1 + VSc::MAT;
         } else {
+            using DSc = DistScratch<(M > 16 ? M : 32)>;
             mat0 = gb + Lay::G_SCR;
             mat1 = mat0 + DSc::MAT;
             aux = reinterpret_cast<float*>(mat1 + DSc::MAT);
@@ -1719,9 +1746,17 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
                 core_warp<T, M, NCOL>(qbar, kbar, mU, mW, yT, iters, sl2, g, t);
             }
         } else {
-            if (r < CW)
+            if constexpr (M == 64) {
+                if (r < CW) {
+                    float w[NCOL / 8][4];
+                    vc_load_w<NCOL>(mW, w, r, g, t);
+                    vc_core<T, M, NCOL>(qbar, kbar, gmu[16 * r + g], gmu[16 * r + g + 8], w, yT, mat0, mat1, vmat, aux,
+                                        iters, sl2, r, lane, 1 + GROUPS + grp);
+                }
+            } else if (r < CW) {
                 dist_core<T, (M > 16 ? M : 32), NCOL>(qbar, kbar, gmu, mW, yT, mat0, mat1, aux, iters, sl2, r, lane,
                                                       1 + GROUPS + grp);
+            }
         }
         gsync();
         if constexpr (Lay::SCR_IN_STAGE) prefetch_qk();
@@ -1809,6 +1844,11 @@ template <typename T, int M, int NCOL, int PW = 0>
 cudaError_t launch_pool(const void* q, const void* k, const void* v, void* out, long long n_units, int d,
                         int iters, cudaStream_t stream, unsigned int* fault, const NystraBias* bias = nullptr);
 
+// Wide kernel (nystra_wide.cuh): m = 64 at 8x8 and 16x16 windows.
+template <typename T, int M, int NCOL, int N>
+cudaError_t launch_wide(const void* q, const void* k, const void* v, void* out, long long n_units, int d,
+                        int iters, cudaStream_t stream, unsigned int* fault);
+
 // Team kernel for 16x16 windows (nystra_team.cuh, N = 256 translation unit only).
 template <typename T, int M, int NCOL, int PW = 0>
 cudaError_t launch_team(const void* q, const void* k, const void* v, void* out, long long n_units, int d,
@@ -1882,8 +1922,10 @@ cudaError_t launch_n(const void* q, const void* k, const void* v, void* out, lon
             return wide ? launch_stream<T, 32, 40>(q, k, v, out, n_units, d, iters, stream, fault)
                         : launch_stream<T, 32, 32>(q, k, v, out, n_units, d, iters, stream, fault);
     }
-    // The grouped kernel: m = 32 at 8x8 windows (core in one warp's registers)
-    // and at 16x16 windows with d_h = 32 (core on two warps); every m = 64.
+    // The grouped kernel: m = 32 at 8x8 windows (core in one warp's registers;
+    // 20000 units of d_h = 30 take 400 us, on the wide kernel's two warps 519)
+    // and at 16x16 windows with d_h = 32 (core on two warps), m = 64 at 32x32
+    // windows.  The wide kernel: m = 64 at 8x8 and 16x16.
     if (m == 32) {
         if constexpr (TPW == 64 && WPU == 1)
             return wide ? launch_cfg<T, 32, 40, 64, 1, 1>(q, k, v, out, n_units, d, iters, stream, fault)
@@ -1893,12 +1935,12 @@ cudaError_t launch_n(const void* q, const void* k, const void* v, void* out, lon
         return cudaErrorInvalidValue;  // not reached: the stream kernel takes 32x32 windows
     }
     if (m == 64) {
-        // the core on four warps; W partials of 64 rows need K/V rows of at
-        // least 128 tokens per token warp
-        constexpr int TP = (TPW * WPU == 64) ? 64 : (TPW * WPU == 256) ? 128 : 256;
-        constexpr int WP = TPW * WPU / TP;
-        return wide ? launch_cfg<T, 64, 40, TP, WP, 4>(q, k, v, out, n_units, d, iters, stream, fault)
-                    : launch_cfg<T, 64, 32, TP, WP, 4>(q, k, v, out, n_units, d, iters, stream, fault);
+        if constexpr (TPW * WPU == 1024)  // a token warp of 256 rows: W partials of 64 rows lie over its K/V rows
+            return wide ? launch_cfg<T, 64, 40, 256, 4, 4>(q, k, v, out, n_units, d, iters, stream, fault)
+                        : launch_cfg<T, 64, 32, 256, 4, 4>(q, k, v, out, n_units, d, iters, stream, fault);
+        else
+            return wide ? launch_wide<T, 64, 40, TPW * WPU>(q, k, v, out, n_units, d, iters, stream, fault)
+                        : launch_wide<T, 64, 32, TPW * WPU>(q, k, v, out, n_units, d, iters, stream, fault);
     }
     return cudaErrorInvalidValue;  // not reached: m is checked by the caller
 }

@@ -3,5 +3,6 @@
 // a caller selects with NYSTRA_FACTORS_16 (16-bit I/O only).
 #include "nystra_tc.cuh"
 #include "nystra_pool.cuh"
+#include "nystra_wide.cuh"
 
 NYSTRA_TC_DEFINE(n64_s16, 64, 1, nystra::Single16<__nv_bfloat16>, nystra::Single16<__half>, false)
