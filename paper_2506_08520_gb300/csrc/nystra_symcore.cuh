@@ -1,6 +1,6 @@
-// The m x m core of m = 64 on CW = m/16 = 4 warps, carrying V = Z W instead of
-// Z.  Included by nystra_tc.cuh after the other cores, whose fragment helpers
-// it uses.
+// The m x m core of m = 64 on CW = m/16 = 4 warps, with symmetric products.
+// Included by nystra_tc.cuh after the other cores, whose fragment helpers it
+// uses.
 #pragma once
 
 #include "ptx.cuh"
@@ -8,61 +8,62 @@
 namespace nystra {
 namespace tc {
 
-// Warp c owns rows 16c..16c+15.  Instead of Z (dist_core) the iteration
-// carries V_k = Z_k W and the symmetric X_k = Z_k A (V_0 = a A^T W, X_0 = a A^T A): with T3 = 13I - X(15I - X(7I - X)), Z_{k+1} = T3 Z_k / 4 (its
-// factors are polynomials in X_k and commute), so V_{k+1} = T3 V_k / 4 and
-// X_{k+1} = T3 X_k / 4, and Y = V at the end.  V has d_h + 1 columns instead of
-// m, needs no separate product with W, and all three m x m products of a step
-// are symmetric: of a warp's 2 CW tiles of 16 x 8 only one triangle's CW + 1
-// are computed (20 tile products per warp and step instead of 32) and mirrored, which removes antisymmetric round-off.
+// Warp c owns rows 16c..16c+15.  The arithmetic is dist_core's: X = A Z_k and
+// Z are carried, T2 = 15I - 7X + XX, T3 = 13I - X T2, Z <- Z T3/4, X <- X T3/4.
+// T2, T3 and X are polynomials in X_0 = a A A^T and symmetric: of a warp's
+// 2 CW tiles of 16 x 8 in each of their products only one triangle's CW + 1 are
+// computed, and mirrored, which also removes antisymmetric round-off (23 tile
+// products per warp and step instead of 32).  Z's own rows stay in registers
+// at a power of two per warp, so no step needs a maximum over the warps.
 //
 // A warp computes its diagonal block (two tiles), the block to its right,
 // cyclically (two tiles), and one tile of the blocks two apart, whose left
-// rows it keeps as a second A operand.  X's k-blocks are taken in the cyclic order of those columns, so the
-// registers that hold X's own entries of a tile have constant indexes.
+// rows it keeps as a second A operand.  X's k-blocks and Z's tiles are taken
+// in the cyclic order of those columns, so that register indexes are constant.
 //
 // Right factors are read from two shared-memory matrices (hi and lo planes,
 // rows padded to m + 8 halves so ldmatrix is conflict-free) that alternate
 // roles: X in one, -T2/4 in the other, T3/4 over X once every warp has used X,
 // the next X over -T2/4 once every warp has used it; three barriers per step.
-// V lies in its own matrix (m rows of 40 columns), split at a power of two per
-// column (V's columns, the features and the ones column, are independent
-// outputs of any scale) that puts its largest entry in [2^10, 2^11).
+// W waits for Y = Z W in its own matrix (m rows of 40 columns), split at a power
+// of two per column (the features and the ones column are independent outputs
+// of any scale) that puts its largest entry in [2^10, 2^11).
 //
 // What bounds it: the tensor pipe's mma.sync rate and, between two barriers,
 // a chain of 12 dependent MMAs with the split and store of their results.
 // Measured in the wide kernel (4096 units of 16x16 windows, d_h = 32, bf16):
-// 0.93 ms with Z carried and two groups per SM -> 0.51 ms, the tensor pipe
-// about half busy; 32x32 windows (1024 units, the grouped kernel) 0.50 -> 0.46.
-// At m = 32 (16x16 windows, two warps) carrying Z is the faster form, 352
-// against 395 us for 8192 units: a step's products are too short for the
-// column maxima and the mirrored stores to hide behind.
+// 0.93 ms with full products and two groups per SM -> 0.50 ms; in the grouped
+// kernel (1024 units of 32x32 windows) 0.50 -> 0.40 ms.  Carrying V = Z W
+// instead (V <- T3 V/4 with X = Z A: d_h + 1 columns instead of m, 20 tile
+// products a step, but V's column scales to agree on in every step) took 0.51
+// and 0.46 ms, and was less accurate: under sharp attention (logit std 4) its
+// error was up to twice as large, since Z T3 meets W's small parts exactly.
 
 template <int M>
-__device__ __forceinline__ void vc_store(unsigned char* mat, int row, int col, const H2Pair& p) {
-    constexpr int SS = VcScratch<M>::SS;
+__device__ __forceinline__ void sc_store(unsigned char* mat, int row, int col, const H2Pair& p) {
+    constexpr int SS = ScScratch<M>::SS;
     *reinterpret_cast<uint32_t*>(mat + ((size_t)row * SS + col) * 2) = p.hi;
-    *reinterpret_cast<uint32_t*>(mat + VcScratch<M>::PLANE + ((size_t)row * SS + col) * 2) = p.lo;
+    *reinterpret_cast<uint32_t*>(mat + ScScratch<M>::PLANE + ((size_t)row * SS + col) * 2) = p.lo;
 }
 
 // Own rows of acc (already scaled) into a scratch matrix.
 template <int M>
-__device__ __forceinline__ void vc_put(unsigned char* mat, const float (&acc)[M / 8][4], int c, int g, int t) {
+__device__ __forceinline__ void sc_put(unsigned char* mat, const float (&acc)[M / 8][4], int c, int g, int t) {
 #pragma unroll
     for (int n = 0; n < M / 8; ++n) {
-        vc_store<M>(mat, 16 * c + g, 8 * n + 2 * t, split_h2(acc[n][0], acc[n][1]));
-        vc_store<M>(mat, 16 * c + g + 8, 8 * n + 2 * t, split_h2(acc[n][2], acc[n][3]));
+        sc_store<M>(mat, 16 * c + g, 8 * n + 2 * t, split_h2(acc[n][0], acc[n][1]));
+        sc_store<M>(mat, 16 * c + g + 8, 8 * n + 2 * t, split_h2(acc[n][2], acc[n][3]));
     }
 }
 
 // The tiles of one warp (see above): columns 8 n(i) .. 8 n(i) + 7 of its own
 // rows for i < OWN, of row block r5 for the last.
 template <int M>
-struct VcTiles {
+struct ScTiles {
     static constexpr int CW = M / 16, N = CW + 1, OWN = N - 1;
     static_assert(CW == 4, "the cyclic split is that of four row blocks");
     int c, r5, b5, h5;  // own block; the last tile's row block, column block and half
-    __device__ __forceinline__ explicit VcTiles(int c_) : c(c_) {
+    __device__ __forceinline__ explicit ScTiles(int c_) : c(c_) {
         r5 = c & 1;
         b5 = r5 + 2;
         h5 = c >> 1;
@@ -73,10 +74,10 @@ struct VcTiles {
 
 // The symmetric matrix of which acc (scaled by s) holds this warp's tiles.
 template <int M>
-__device__ __forceinline__ void vc_put_sym(unsigned char* mat, const float (&acc)[M / 16 + 1][4], float s,
-                                             const VcTiles<M>& tl, int g, int t, uint32_t sel) {
+__device__ __forceinline__ void sc_put_sym(unsigned char* mat, const float (&acc)[M / 16 + 1][4], float s,
+                                             const ScTiles<M>& tl, int g, int t, uint32_t sel) {
 #pragma unroll
-    for (int i = 0; i < VcTiles<M>::N; ++i)
+    for (int i = 0; i < ScTiles<M>::N; ++i)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int R = 2 * tl.row(i) + h, n = tl.col(i);  // 8x8 block (R, n)
@@ -87,18 +88,18 @@ __device__ __forceinline__ void vc_put_sym(unsigned char* mat, const float (&acc
                 p.hi = prmt(p.hi, q.hi, sel);
                 p.lo = prmt(p.lo, q.lo, sel);
             } else {
-                vc_store<M>(mat, 8 * n + g, 8 * R + 2 * t, q);
+                sc_store<M>(mat, 8 * n + g, 8 * R + 2 * t, q);
             }
-            vc_store<M>(mat, 8 * R + g, 8 * n + 2 * t, p);
+            sc_store<M>(mat, 8 * R + g, 8 * n + 2 * t, p);
         }
 }
 
 // A operand of row block rb (TR: of the transpose's) from a scratch matrix,
 // k-step j = block (b0 + j) mod CW.
 template <int M, bool TR>
-__device__ __forceinline__ void vc_load_a(const unsigned char* mat, H2Pair (&a)[M / 16][4], int rb, int b0,
+__device__ __forceinline__ void sc_load_a(const unsigned char* mat, H2Pair (&a)[M / 16][4], int rb, int b0,
                                             int lane) {
-    constexpr int SS = VcScratch<M>::SS, CW = M / 16;
+    constexpr int SS = ScScratch<M>::SS, CW = M / 16;
     const int blk = lane >> 3, rr = lane & 7;
 #pragma unroll
     for (int j = 0; j < CW; ++j) {
@@ -109,10 +110,10 @@ __device__ __forceinline__ void vc_load_a(const unsigned char* mat, H2Pair (&a)[
         const unsigned char* ph = mat + ((size_t)row * SS + col) * 2;
         if (TR) {
             ldsm_x4_t(h, ph);
-            ldsm_x4_t(l, ph + VcScratch<M>::PLANE);
+            ldsm_x4_t(l, ph + ScScratch<M>::PLANE);
         } else {
             ldsm_x4(h, ph);
-            ldsm_x4(l, ph + VcScratch<M>::PLANE);
+            ldsm_x4(l, ph + ScScratch<M>::PLANE);
         }
 #pragma unroll
         for (int r = 0; r < 4; ++r) a[j][r] = H2Pair{h[r], l[r]};
@@ -122,7 +123,7 @@ __device__ __forceinline__ void vc_load_a(const unsigned char* mat, H2Pair (&a)[
 // D[i] += A_i B_i over the pair's significant products (lo hi, hi lo, hi hi),
 // tile by tile within each so that consecutive MMAs are independent.
 template <int NTL>
-__device__ __forceinline__ void vc_mma(float (*const (&D)[NTL])[4], const H2Pair (*const (&A)[NTL])[4],
+__device__ __forceinline__ void sc_mma(float (*const (&D)[NTL])[4], const H2Pair (*const (&A)[NTL])[4],
                                          const uint32_t (*const (&bh)[NTL]), const uint32_t (*const (&bl)[NTL])) {
     using H = Mma16<__half>;
 #pragma unroll
@@ -137,49 +138,31 @@ __device__ __forceinline__ void vc_mma(float (*const (&D)[NTL])[4], const H2Pair
         }
 }
 
-// This warp's tiles of A P^T (P symmetric, in mat) or, TR, of P^T P (P in mat,
-// A its transpose): acc += ...; Ao, A5: A operands of the own rows and of row
-// block r5, in the cyclic k order of vc_load_a from block c and b5.
-template <int M, bool TR>
-__device__ __forceinline__ void vc_sym_mm(const H2Pair (&Ao)[M / 16][4], const H2Pair (&A5)[M / 16][4],
-                                            const unsigned char* mat, float (&acc)[M / 16 + 1][4],
-                                            const VcTiles<M>& tl, int lane) {
-    constexpr int SS = VcScratch<M>::SS, CW = M / 16, OWN = CW;
-    constexpr size_t PL = VcScratch<M>::PLANE;
+// This warp's tiles of A P^T (P in mat): acc += ...; Ao, A5: A operands of the
+// own rows and of row block r5, in the cyclic k order of sc_load_a from block c
+// and b5.
+template <int M>
+__device__ __forceinline__ void sc_sym_mm(const H2Pair (&Ao)[M / 16][4], const H2Pair (&A5)[M / 16][4],
+                                          const unsigned char* mat, float (&acc)[M / 16 + 1][4],
+                                          const ScTiles<M>& tl, int lane) {
+    constexpr int SS = ScScratch<M>::SS, CW = M / 16, OWN = CW;
+    constexpr size_t PL = ScScratch<M>::PLANE;
     const int blk = lane >> 3, rr = lane & 7;
 #pragma unroll
     for (int j = 0; j < CW; ++j) {
-        // B fragments of the own tiles, two at a time (16 columns), and of the last tile for two k-steps
-        uint32_t bh[OWN / 2][4], bl[OWN / 2][4];
-        const int kk = (tl.c + j) % CW;
+        // B fragments of the own tiles, two at a time (16 columns), and of the last tile
+        uint32_t bh[OWN / 2][4], bl[OWN / 2][4], eh[2], el[2];
+        const int kk = (tl.c + j) % CW, k5 = (tl.b5 + j) % CW;
 #pragma unroll
         for (int p = 0; p < OWN / 2; ++p) {
             const int cb = (tl.c + p) % CW;
-            const unsigned char* ph =
-                TR ? mat + ((size_t)(16 * kk + 8 * (blk & 1) + rr) * SS + 16 * cb + 8 * (blk >> 1)) * 2
-                   : mat + ((size_t)(16 * cb + 8 * (blk >> 1) + rr) * SS + 16 * kk + 8 * (blk & 1)) * 2;
-            if (TR) {
-                ldsm_x4_t(bh[p], ph);
-                ldsm_x4_t(bl[p], ph + PL);
-            } else {
-                ldsm_x4(bh[p], ph);
-                ldsm_x4(bl[p], ph + PL);
-            }
+            const unsigned char* ph = mat + ((size_t)(16 * cb + 8 * (blk >> 1) + rr) * SS + 16 * kk + 8 * (blk & 1)) * 2;
+            ldsm_x4(bh[p], ph);
+            ldsm_x4(bl[p], ph + PL);
         }
-        uint32_t eh[2], el[2];
-        {
-            const int k5 = (tl.b5 + j) % CW, n5 = tl.col(OWN);
-            const int hb = blk & 1;  // 8x8 blocks k, k + 8 (x2: lanes 16..31 repeat them)
-            const unsigned char* ph = TR ? mat + ((size_t)(16 * k5 + 8 * hb + rr) * SS + 8 * n5) * 2
-                                         : mat + ((size_t)(8 * n5 + rr) * SS + 16 * k5 + 8 * hb) * 2;
-            if (TR) {
-                ldsm_x2_t(eh, ph);
-                ldsm_x2_t(el, ph + PL);
-            } else {
-                ldsm_x2(eh, ph);
-                ldsm_x2(el, ph + PL);
-            }
-        }
+        const unsigned char* p5 = mat + ((size_t)(8 * tl.col(OWN) + rr) * SS + 16 * k5 + 8 * (blk & 1)) * 2;
+        ldsm_x2(eh, p5);
+        ldsm_x2(el, p5 + PL);
         float(*D[OWN + 1])[4];
         const H2Pair(*A[OWN + 1])[4];
         const uint32_t *ph[OWN + 1], *pl[OWN + 1];
@@ -194,16 +177,55 @@ __device__ __forceinline__ void vc_sym_mm(const H2Pair (&Ao)[M / 16][4], const H
         A[OWN] = &A5[j];
         ph[OWN] = eh;
         pl[OWN] = el;
-        vc_mma<OWN + 1>(D, A, ph, pl);
+        sc_mma<OWN + 1>(D, A, ph, pl);
     }
 }
 
-// Own rows of A V (V in vmat): acc = A V, A in the k order of vc_load_a from block b0.
+// All tiles of the own rows of A P^T (P in mat), column block (c + i / 2) mod CW
+// in tiles i, i + 1: acc = A P^T; A in the cyclic k order from block c.
+template <int M>
+__device__ __forceinline__ void sc_row_mm(const H2Pair (&A)[M / 16][4], const unsigned char* mat,
+                                          float (&acc)[M / 8][4], int c, int lane) {
+    constexpr int SS = ScScratch<M>::SS, CW = M / 16, NT = M / 8;
+    constexpr size_t PL = ScScratch<M>::PLANE;
+    const int blk = lane >> 3, rr = lane & 7;
+#pragma unroll
+    for (int i = 0; i < NT; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+#pragma unroll
+    for (int j = 0; j < CW; ++j) {
+        const int kk = (c + j) % CW;
+#pragma unroll
+        for (int q = 0; q < CW; q += 2) {  // four tiles at a time
+            uint32_t bh[2][4], bl[2][4];
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                const int cb = (c + q + p) % CW;
+                const unsigned char* ph =
+                    mat + ((size_t)(16 * cb + 8 * (blk >> 1) + rr) * SS + 16 * kk + 8 * (blk & 1)) * 2;
+                ldsm_x4(bh[p], ph);
+                ldsm_x4(bl[p], ph + PL);
+            }
+            float(*D[4])[4];
+            const H2Pair(*Ap[4])[4];
+            const uint32_t *ph[4], *pl[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                D[i] = &acc[2 * q + i];
+                Ap[i] = &A[j];
+                ph[i] = bh[i / 2] + 2 * (i & 1);
+                pl[i] = bl[i / 2] + 2 * (i & 1);
+            }
+            sc_mma<4>(D, Ap, ph, pl);
+        }
+    }
+}
+
+// Own rows of A W (W in wmat): acc = A W, A in the k order of sc_load_a from block b0.
 template <int M, int NCOL>
-__device__ __forceinline__ void vc_v_mm(const H2Pair (&A)[M / 16][4], const unsigned char* vmat,
+__device__ __forceinline__ void sc_w_mm(const H2Pair (&A)[M / 16][4], const unsigned char* wmat,
                                           float (&acc)[NCOL / 8][4], int b0, int lane) {
-    constexpr int VS = VcScratch<M>::VS, CW = M / 16, NTO = NCOL / 8;
-    constexpr size_t PL = VcScratch<M>::VPLANE;
+    constexpr int WS = ScScratch<M>::WS, CW = M / 16, NTO = NCOL / 8;
+    constexpr size_t PL = ScScratch<M>::WPLANE;
     const int blk = lane >> 3, rr = lane & 7;
 #pragma unroll
     for (int n = 0; n < NTO; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
@@ -213,7 +235,7 @@ __device__ __forceinline__ void vc_v_mm(const H2Pair (&A)[M / 16][4], const unsi
         uint32_t bh[NTO][2], bl[NTO][2];
 #pragma unroll
         for (int n = 0; n < NTO; n += 2) {
-            const unsigned char* ph = vmat + ((size_t)(16 * kk + 8 * (blk & 1) + rr) * VS + 8 * (n + (blk >> 1))) * 2;
+            const unsigned char* ph = wmat + ((size_t)(16 * kk + 8 * (blk & 1) + rr) * WS + 8 * (n + (blk >> 1))) * 2;
             if (n + 1 < NTO) {
                 uint32_t x[4], y[4];
                 ldsm_x4_t(x, ph);
@@ -221,7 +243,7 @@ __device__ __forceinline__ void vc_v_mm(const H2Pair (&A)[M / 16][4], const unsi
                 bh[n][0] = x[0]; bh[n][1] = x[1]; bh[n + 1][0] = x[2]; bh[n + 1][1] = x[3];
                 bl[n][0] = y[0]; bl[n][1] = y[1]; bl[n + 1][0] = y[2]; bl[n + 1][1] = y[3];
             } else {
-                ph = vmat + ((size_t)(16 * kk + 8 * (blk & 1) + rr) * VS + 8 * n) * 2;
+                ph = wmat + ((size_t)(16 * kk + 8 * (blk & 1) + rr) * WS + 8 * n) * 2;
                 ldsm_x2_t(bh[n], ph);
                 ldsm_x2_t(bl[n], ph + PL);
             }
@@ -236,13 +258,13 @@ __device__ __forceinline__ void vc_v_mm(const H2Pair (&A)[M / 16][4], const unsi
             ph[n] = bh[n];
             pl[n] = bl[n];
         }
-        vc_mma<NTO>(D, Ap, ph, pl);
+        sc_mma<NTO>(D, Ap, ph, pl);
     }
 }
 
-// Column maxima of |v| over this warp's rows into slot[0 .. NCOL).
+// Column maxima of |w| over this warp's rows into slot[0 .. NCOL).
 template <int NCOL>
-__device__ __forceinline__ void vc_colmax(const float (&v)[NCOL / 8][4], float* slot, int g, int t) {
+__device__ __forceinline__ void sc_colmax(const float (&v)[NCOL / 8][4], float* slot, int g, int t) {
 #pragma unroll
     for (int n = 0; n < NCOL / 8; ++n)
 #pragma unroll
@@ -255,14 +277,13 @@ __device__ __forceinline__ void vc_colmax(const float (&v)[NCOL / 8][4], float* 
         }
 }
 
-// Own rows of V into vmat, column by column scaled by 2^e with e from the
-// column's largest entry (over the warps' slots); e is added to ev (per lane:
-// columns 8n + 2t, 8n + 2t + 1).  The total stays within +-120, so that both
-// powers of two are normal numbers.
+// Own rows of W into wmat, column by column scaled by 2^ev with ev from the
+// column's largest entry (over the warps' slots; per lane columns 8n + 2t,
+// 8n + 2t + 1), within +-120, so that both powers of two are normal numbers.
 template <int M, int NCOL>
-__device__ __forceinline__ void vc_put_v(unsigned char* vmat, const float (&v)[NCOL / 8][4], const float* slots,
-                                           int (&ev)[NCOL / 8][2], int c, int g, int t) {
-    constexpr int VS = VcScratch<M>::VS, CW = M / 16;
+__device__ __forceinline__ void sc_put_w(unsigned char* wmat, const float (&v)[NCOL / 8][4], const float* slots,
+                                         int (&ev)[NCOL / 8][2], int c, int g, int t) {
+    constexpr int WS = ScScratch<M>::WS, CW = M / 16;
 #pragma unroll
     for (int n = 0; n < NCOL / 8; ++n) {
         float s[2];
@@ -271,63 +292,58 @@ __device__ __forceinline__ void vc_put_v(unsigned char* vmat, const float (&v)[N
             float x = 0.f;
 #pragma unroll
             for (int w = 0; w < CW; ++w) x = fmaxf(x, slots[w * NCOL + 8 * n + 2 * t + e]);
-            int k = h2_exponent(x);
-            k = max(-120 - ev[n][e], min(120 - ev[n][e], k));
-            ev[n][e] += k;
-            s[e] = pow2i(k);
+            ev[n][e] = max(-120, min(120, h2_exponent(x)));
+            s[e] = pow2i(ev[n][e]);
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const H2Pair p = split_h2(s[0] * v[n][2 * h], s[1] * v[n][2 * h + 1]);
-            unsigned char* q = vmat + ((size_t)(16 * c + g + 8 * h) * VS + 8 * n + 2 * t) * 2;
+            unsigned char* q = wmat + ((size_t)(16 * c + g + 8 * h) * WS + 8 * n + 2 * t) * 2;
             *reinterpret_cast<uint32_t*>(q) = p.hi;
-            *reinterpret_cast<uint32_t*>(q + VcScratch<M>::VPLANE) = p.lo;
+            *reinterpret_cast<uint32_t*>(q + ScScratch<M>::WPLANE) = p.lo;
         }
     }
 }
 
 // Core on CW = M/16 warps (warp c of them calls with its index; bar_id is a
-// named barrier reserved for these warps; mat0, mat1, vmat, aux: VcScratch
+// named barrier reserved for these warps; mat0, mat1, wmat, aux: ScScratch
 // areas): G_A^n from the landmarks and the m_U of the own rows (mu0, mu1: rows
-// 16c + g and + 8, log2 domain), the iteration of step 4 on X and V (on entry
-// v: the own rows of W, C layout), Y = V stored as Y^T at yT, or where yT is
-// null over the scratch matrix that is free by then; returns its place.  vmat
-// may overlay Qbar (first written after every warp has read its rows).  As in
-// core_warp, A is split at 2^ea with its largest entry in
-// [2^10, 2^11); X, -T2/4 and T3/4 are split at the fixed scale 2^10 (their
-// entries stay within a few units, since X's eigenvalues lie in [0, 1]).
-// Scalar factors of V cancel in step 7 and are dropped; its columns' powers of
-// two are taken back before the store.
+// 16c + g and + 8, log2 domain), the iteration of step 4, Y = Z W (on entry w:
+// the own rows of W, C layout) stored as Y^T at yT, or where yT is null over
+// the scratch matrix that is free by then; returns its place.  wmat may overlay
+// Qbar (first written after every warp has read its rows).  As in core_warp, A
+// is split at 2^ea with its largest entry in [2^10, 2^11); X, -T2/4 and T3/4
+// are split at the fixed scale 2^10 (their entries stay within a few units,
+// since X's eigenvalues lie in [0, 1]).  Scalar factors of Z cancel in step 7
+// and are dropped; the warps' and columns' powers of two are taken back.
 template <typename T, int M, int NCOL>
-__device__ __forceinline__ T* vc_core(const T* qbar, const T* kbar, float mu0, float mu1, float (&v)[NCOL / 8][4],
-                                        T* yT, unsigned char* mat0, unsigned char* mat1, unsigned char* vmat,
-                                        float* aux, int iters, float sl2, int c, int lane, int bar_id) {
-    using S = VcScratch<M>;
+__device__ __forceinline__ T* sc_core(const T* qbar, const T* kbar, float mu0, float mu1, float (&w)[NCOL / 8][4],
+                                      T* yT, unsigned char* mat0, unsigned char* mat1, unsigned char* wmat, float* aux,
+                                      int iters, float sl2, int c, int lane, int bar_id) {
+    using S = ScScratch<M>;
     using O = Opnd<T>;
     using D = typename O::DReg;
-    constexpr int CW = S::CW, KT = M / 16, NT = M / 8, LS = LmS<T>::LS, LO = LmS<T>::LO,
-                  NTO = NCOL / 8, YS = YtS<T, M>::YS, YLO = YtS<T, M>::LO, NTL = VcTiles<M>::N;
-    static_assert(NCOL <= S::VS, "V's rows");
+    constexpr int CW = S::CW, KT = M / 16, NT = M / 8, LS = LmS<T>::LS, LO = LmS<T>::LO, NTO = NCOL / 8,
+                  YS = YtS<T, M>::YS, YLO = YtS<T, M>::LO, NTL = ScTiles<M>::N;
+    static_assert(NCOL <= S::WS, "W's rows");
     const int g = lane >> 2, t = lane & 3;
     unsigned char* cur = mat0;
     unsigned char* oth = mat1;
     float* cols = aux;                // [CW][M] column-sum partials
     float* slots = aux + CW * M;      // [4][CW] maxima
-    float* vslots = slots + 4 * CW;   // [CW][NCOL] column maxima of V
+    float* wslots = slots + 4 * CW;   // [CW][NCOL] column maxima of W
     auto csync = [&]() { named_barrier(bar_id, CW * 32); };
     const uint32_t sel = tril_selector(g, t);
-    const VcTiles<M> tl(c);
+    const ScTiles<M> tl(c);
     constexpr float kS = 1024.f, kS2 = 1048576.f;  // fixed scale 2^10 of X, -T2/4, T3/4 (and its square)
-    H2Pair Xa[KT][4], X5[KT][4];
+    H2Pair Xa[KT][4], X5[KT][4], Za[KT][4];
     float acc[NTL][4];
-    int ev[NTO][2];
-    float alpha;  // a A^T A = alpha (2^ea A)^T (2^ea A)
+    int ev[NTO][2], ez = 0;  // powers of two of W's columns and of Z's rows
+    float alpha;             // a A A^T = alpha (2^ea A)(2^ea A)^T
     {
         float a[NT][4];
         // ---- G_A^n's own rows ----
-#pragma unroll
-        for (int n = 0; n < NTO; ++n) ev[n][0] = ev[n][1] = 0;
-        vc_colmax<NCOL>(v, vslots + c * NCOL, g, t);
+        sc_colmax<NCOL>(w, wslots + c * NCOL, g, t);
         {
             D aq[2][4];
 #pragma unroll
@@ -365,7 +381,7 @@ __device__ __forceinline__ T* vc_core(const T* qbar, const T* kbar, float mu0, f
             csync();  // every warp has read its rows of Qbar
             float lmax = -INFINITY;
 #pragma unroll
-            for (int w = 0; w < CW; ++w) lmax = fmaxf(lmax, slots[3 * CW + w]);
+            for (int x = 0; x < CW; ++x) lmax = fmaxf(lmax, slots[3 * CW + x]);
             const float fa = (lmax > -INFINITY && lmax < INFINITY) ? (float)(10 - (int)floorf(lmax)) : 0.f;
 #pragma unroll
             for (int n = 0; n < NT; ++n)
@@ -397,16 +413,16 @@ __device__ __forceinline__ T* vc_core(const T* qbar, const T* kbar, float mu0, f
                     if (g == 0) cols[c * M + 8 * n + 2 * t + e] = cs;
                 }
         }
-        vc_put<M>(cur, a, c, g, t);  // 2^ea A
-        vc_put_v<M, NCOL>(vmat, v, vslots, ev, c, g, t);
+        sc_put<M>(cur, a, c, g, t);  // 2^ea A
+        sc_put_w<M, NCOL>(wmat, w, wslots, ev, c, g, t);
         csync();
         float rmax = 0.f, cmax = 0.f;
 #pragma unroll
-        for (int w = 0; w < CW; ++w) rmax = fmaxf(rmax, slots[w]);
+        for (int x = 0; x < CW; ++x) rmax = fmaxf(rmax, slots[x]);
         for (int col = lane; col < M; col += 32) {
             float cs = 0.f;
 #pragma unroll
-            for (int w = 0; w < CW; ++w) cs += cols[w * M + col];
+            for (int x = 0; x < CW; ++x) cs += cols[x * M + col];
             cmax = fmaxf(cmax, cs);
         }
         alpha = 1.f / (rmax * warp_max_nonneg(cmax));
@@ -415,8 +431,7 @@ __device__ __forceinline__ T* vc_core(const T* qbar, const T* kbar, float mu0, f
 #pragma unroll
         for (int i = 0; i < NTL; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
     };
-    // acc += s I + f (hi + lo of the tiles' own X entries)
-    auto add_diag = [&](float s) {
+    auto add_diag = [&](float s) {  // acc += s I
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -430,19 +445,15 @@ __device__ __forceinline__ T* vc_core(const T* qbar, const T* kbar, float mu0, f
         const float2 y = __half22float2(*reinterpret_cast<const __half2*>(&p.lo));
         return make_float2(x.x + y.x, x.y + y.y);
     };
-    // ---- V_0 = A^T W, X_0 = alpha A^T A ----
-    vc_load_a<M, true>(cur, Xa, c, c, lane);
-    vc_load_a<M, true>(cur, X5, tl.r5, tl.b5, lane);
+    // ---- Z_0 = (2^ea A)^T (a and 2^ea dropped), X_0 = alpha (2^ea A)(2^ea A)^T ----
+    sc_load_a<M, false>(cur, Xa, c, c, lane);
+    sc_load_a<M, false>(cur, X5, tl.r5, tl.b5, lane);
     zero();
-    vc_sym_mm<M, true>(Xa, X5, cur, acc, tl, lane);
-    vc_v_mm<M, NCOL>(Xa, vmat, v, c, lane);
-    vc_put_sym<M>(oth, acc, kS * alpha, tl, g, t, sel);  // kS X_0
-    vc_colmax<NCOL>(v, vslots + c * NCOL, g, t);
+    sc_sym_mm<M>(Xa, X5, cur, acc, tl, lane);
+    sc_load_a<M, true>(cur, Za, c, c, lane);
+    sc_put_sym<M>(oth, acc, kS * alpha, tl, g, t, sel);  // kS X_0
     csync();
-    if (iters > 0) {
-        vc_put_v<M, NCOL>(vmat, v, vslots, ev, c, g, t);
-        vc_load_a<M, false>(oth, Xa, c, c, lane);
-        vc_load_a<M, false>(oth, X5, tl.r5, tl.b5, lane);
+    {
         unsigned char* tmp = cur;
         cur = oth;
         oth = tmp;
@@ -450,6 +461,8 @@ __device__ __forceinline__ T* vc_core(const T* qbar, const T* kbar, float mu0, f
     // ---- iteration (step 4): X in cur ----
 #pragma unroll 1
     for (int it = 0; it < iters; ++it) {
+        sc_load_a<M, false>(cur, Xa, c, c, lane);
+        sc_load_a<M, false>(cur, X5, tl.r5, tl.b5, lane);
         // kS^2 T2 = kS^2 (15I - 7X + X X); X's entries of a tile are its k-step i / 2's (the last tile's: 0's)
 #pragma unroll
         for (int i = 0; i < NTL; ++i)
@@ -465,43 +478,56 @@ __device__ __forceinline__ T* vc_core(const T* qbar, const T* kbar, float mu0, f
                 acc[i][2 * h + 1] = -7.f * kS * x.y;
             }
         add_diag(15.f * kS2);
-        vc_sym_mm<M, false>(Xa, X5, cur, acc, tl, lane);
-        vc_put_sym<M>(oth, acc, -0.25f / kS, tl, g, t, sel);  // kS (-T2/4)
+        sc_sym_mm<M>(Xa, X5, cur, acc, tl, lane);
+        sc_put_sym<M>(oth, acc, -0.25f / kS, tl, g, t, sel);  // kS (-T2/4)
         csync();
         zero();
         add_diag(3.25f * kS2);
-        vc_sym_mm<M, false>(Xa, X5, oth, acc, tl, lane);     // kS^2 T3/4
-        vc_put_sym<M>(cur, acc, 1.f / kS, tl, g, t, sel);    // kS T3/4 (every warp is done with X)
+        sc_sym_mm<M>(Xa, X5, oth, acc, tl, lane);          // kS^2 T3/4
+        sc_put_sym<M>(cur, acc, 1.f / kS, tl, g, t, sel);  // kS T3/4 (every warp is done with X)
         csync();
         const bool more = it + 1 < iters;
         if (more) {
             zero();
-            vc_sym_mm<M, false>(Xa, X5, cur, acc, tl, lane);   // kS^2 X T3/4
-            vc_put_sym<M>(oth, acc, 1.f / kS, tl, g, t, sel);  // every warp is done with -T2/4
+            sc_sym_mm<M>(Xa, X5, cur, acc, tl, lane);          // kS^2 X T3/4
+            sc_put_sym<M>(oth, acc, 1.f / kS, tl, g, t, sel);  // every warp is done with -T2/4
         }
-        vc_load_a<M, false>(cur, Xa, c, c, lane);
-        vc_v_mm<M, NCOL>(Xa, vmat, v, c, lane);  // kS T3/4 V
+        {
+            float z[NT][4];
+            sc_row_mm<M>(Za, cur, z, c, lane);  // kS Z T3/4
+            float zm = 0.f;
 #pragma unroll
-        for (int n = 0; n < NTO; ++n)
+            for (int n = 0; n < NT; ++n)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) v[n][e] *= 1.f / kS;
+                for (int e = 0; e < 4; ++e) zm = fmaxf(zm, fabsf(z[n][e]));
+            const int e = h2_exponent(warp_max_nonneg(zm));
+            const float s = pow2i(e);
+            ez += e + 10;  // and kS
+#pragma unroll
+            for (int j = 0; j < KT; ++j)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int n = 2 * j + (r >> 1), x = 2 * (r & 1);
+                    Za[j][r] = split_h2(s * z[n][x], s * z[n][x + 1]);
+                }
+        }
         if (more) {
-            vc_colmax<NCOL>(v, vslots + c * NCOL, g, t);
             csync();
-            vc_put_v<M, NCOL>(vmat, v, vslots, ev, c, g, t);  // every warp is done with V
-            vc_load_a<M, false>(oth, Xa, c, c, lane);
-            vc_load_a<M, false>(oth, X5, tl.r5, tl.b5, lane);
             unsigned char* tmp = cur;
             cur = oth;
             oth = tmp;
         }
     }
-    // ---- Y = V, own rows, without the columns' powers of two, stored as Y^T ----
+    // ---- Y = Z W, own rows, without the powers of two, stored as Y^T ----
+    sc_w_mm<M, NCOL>(Za, wmat, w, c, lane);
+    const float sz = pow2i(-ez);
 #pragma unroll
     for (int n = 0; n < NTO; ++n) {
         const float s0 = pow2i(-ev[n][0]), s1 = pow2i(-ev[n][1]);
-        v[n][0] *= s0; v[n][2] *= s0;
-        v[n][1] *= s1; v[n][3] *= s1;
+        w[n][0] = sz * w[n][0] * s0;
+        w[n][2] = sz * w[n][2] * s0;
+        w[n][1] = sz * w[n][1] * s1;
+        w[n][3] = sz * w[n][3] * s1;
     }
     float scale = 1.f;
     if (O::kNarrowRange) {
@@ -509,33 +535,33 @@ __device__ __forceinline__ T* vc_core(const T* qbar, const T* kbar, float mu0, f
 #pragma unroll
         for (int j = 0; j < NTO; ++j)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) ym = fmaxf(ym, fabsf(v[j][e]));
+            for (int e = 0; e < 4; ++e) ym = fmaxf(ym, fabsf(w[j][e]));
         ym = warp_max_nonneg(ym);
         if (lane == 0) slots[2 * CW + c] = ym;
         csync();
         float ymax = 0.f;
 #pragma unroll
-        for (int w = 0; w < CW; ++w) ymax = fmaxf(ymax, slots[2 * CW + w]);
+        for (int x = 0; x < CW; ++x) ymax = fmaxf(ymax, slots[2 * CW + x]);
         if (ymax > 0.f && ymax < INFINITY) scale = pow2i(14 - ilogbf(ymax));
     }
     // free: after the last step -T2/4's matrix (its readers have passed a
-    // barrier since), without steps X_0's
+    // barrier since), without steps A's
     if (!yT) yT = reinterpret_cast<T*>(oth);
     static_assert(YtS<T, M>::bytes(NCOL) <= S::MAT, "Y^T must fit over a scratch matrix");
 #pragma unroll
     for (int j = 0; j < NTO; ++j) {
         const int rr = 16 * c + g, cc = 8 * j + 2 * t;
-        DSt<T>::put(yT + cc * YS + rr, YLO, v[j][0] * scale);
-        DSt<T>::put(yT + (cc + 1) * YS + rr, YLO, v[j][1] * scale);
-        DSt<T>::put(yT + cc * YS + rr + 8, YLO, v[j][2] * scale);
-        DSt<T>::put(yT + (cc + 1) * YS + rr + 8, YLO, v[j][3] * scale);
+        DSt<T>::put(yT + cc * YS + rr, YLO, w[j][0] * scale);
+        DSt<T>::put(yT + (cc + 1) * YS + rr, YLO, w[j][1] * scale);
+        DSt<T>::put(yT + cc * YS + rr + 8, YLO, w[j][2] * scale);
+        DSt<T>::put(yT + (cc + 1) * YS + rr + 8, YLO, w[j][3] * scale);
     }
     return yT;
 }
 
-// The own rows of W (fp32, row stride NCOL + 4 at mW) as vc_core takes them.
+// The own rows of W (fp32, row stride NCOL + 4 at mW) as sc_core takes them.
 template <int NCOL>
-__device__ __forceinline__ void vc_load_w(const float* mW, float (&v)[NCOL / 8][4], int c, int g, int t) {
+__device__ __forceinline__ void sc_load_w(const float* mW, float (&v)[NCOL / 8][4], int c, int g, int t) {
     constexpr int WS = NCOL + 4;
 #pragma unroll
     for (int n = 0; n < NCOL / 8; ++n) {

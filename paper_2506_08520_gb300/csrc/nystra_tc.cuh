@@ -25,7 +25,7 @@
 //            `iters` steps Z <- Z(13I - X(15I - X(7I - X)))/4 with X = A Z
 //            (step 4), Y = Z W stored as a 16-bit B operand: core_warp (one
 //            warp, in registers, m <= 16), dist_core (m = 32, two warps) or
-//            vc_core (m = 64, four warps; nystra_vcore.cuh).
+//            sc_core (m = 64, four warps; nystra_symcore.cuh).
 //   output   O = (G_L^n Y_:d) / (G_L^n Y_d) (steps 5-7), staged row-major and
 //            written with one bulk store (rows of 60 bytes would otherwise be
 //            written as partial sectors); [P2] S_L and G_L^n recomputed from
@@ -109,19 +109,20 @@ struct DistScratch {
     static constexpr size_t BYTES = ((2 * MAT + AUX + 127) / 128) * 128;
 };
 
-// Shared scratch of the core that carries V (nystra_vcore.cuh): two matrices of fp16 pairs (hi plane, then lo plane; rows
-// padded to m + 8 halves so ldmatrix is conflict-free), V (m rows of 40
+// Shared scratch of the core with symmetric products (nystra_symcore.cuh): two
+// matrices of fp16 pairs (hi plane, then lo plane; rows
+// padded to m + 8 halves so ldmatrix is conflict-free), W (m rows of 40
 // columns, likewise) and an auxiliary float area.
 template <int M>
-struct VcScratch {
-    static constexpr int CW = M / 16, SS = M + 8, VS = 40;
+struct ScScratch {
+    static constexpr int CW = M / 16, SS = M + 8, WS = 40;
     static constexpr size_t PLANE = (size_t)M * SS * 2;
     static constexpr size_t MAT = 2 * PLANE;
-    static constexpr size_t VPLANE = (size_t)M * VS * 2;
-    static constexpr size_t VMAT = 2 * VPLANE;
-    // column sums of A, maxima, column maxima of V
-    static constexpr size_t AUX = ((size_t)CW * M * 4 + 4 * CW * 4 + CW * VS * 4 + 15) / 16 * 16;
-    static constexpr size_t BYTES = ((2 * MAT + VMAT + AUX + 127) / 128) * 128;  // mat0 | mat1 | V | aux
+    static constexpr size_t WPLANE = (size_t)M * WS * 2;
+    static constexpr size_t WMAT = 2 * WPLANE;
+    // column sums of A, maxima, column maxima of W
+    static constexpr size_t AUX = ((size_t)CW * M * 4 + 4 * CW * 4 + CW * WS * 4 + 15) / 16 * 16;
+    static constexpr size_t BYTES = ((2 * MAT + WMAT + AUX + 127) / 128) * 128;  // mat0 | mat1 | W | aux
 };
 
 template <typename T, int M>
@@ -157,7 +158,7 @@ struct Layout {
     static constexpr bool SCR_IN_GROUP = (CW > 1) && !SCR_IN_STAGE;
     static constexpr size_t SCR_BYTES = SCR_IN_GROUP ? DistScratch<(M > 16 ? M : 32)>::BYTES : 0;
     static_assert(!SCR_IN_STAGE || (WPU >= 2 && CW == 4 &&
-                                    VcScratch<64>::MAT + VcScratch<64>::VMAT <= 2 * (size_t)TPW * DS * 2),
+                                    ScScratch<64>::MAT + ScScratch<64>::WMAT <= 2 * (size_t)TPW * DS * 2),
                   "scratch must fit in two warps' K/V rows");
     static constexpr size_t QB_BYTES = LmS<T>::bytes(MP);
     static constexpr size_t YT_BYTES = YtS<T, M>::bytes(NCOL);
@@ -1466,7 +1467,7 @@ __device__ __forceinline__ void dist_core(const T* qbar, const T* kbar, const fl
 }  // namespace tc
 }  // namespace nystra
 
-#include "nystra_vcore.cuh"
+#include "nystra_symcore.cuh"
 
 namespace nystra {
 namespace tc {
@@ -1593,16 +1594,16 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
     // distributed-core scratch
     unsigned char* mat0 = nullptr;
     unsigned char* mat1 = nullptr;
-    unsigned char* vmat = nullptr;
+    unsigned char* wmat = nullptr;
     float* aux = nullptr;
     if constexpr (CW > 1) {
         if constexpr (Lay::SCR_IN_STAGE) {
-            using VSc = VcScratch<64>;
+            using SSc = ScScratch<64>;
             unsigned char* w0 = smem_raw + (size_t)GROUPS * Lay::GROUP_BYTES + (size_t)(grp * WPU) * Lay::WARP_BYTES;
             mat0 = w0 + Lay::WPART;
-            aux = reinterpret_cast<float*>(mat0 + VSc::MAT);
+            aux = reinterpret_cast<float*>(mat0 + SSc::MAT);
             mat1 = w0 + Lay::WARP_BYTES + Lay::WPART;
-            vmat = mat1 + VSc::MAT;
+            wmat = mat1 + SSc::MAT;
         } else {
             using DSc = DistScratch<(M > 16 ? M : 32)>;
             mat0 = gb + Lay::G_SCR;
@@ -1749,8 +1750,8 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
             if constexpr (M == 64) {
                 if (r < CW) {
                     float w[NCOL / 8][4];
-                    vc_load_w<NCOL>(mW, w, r, g, t);
-                    vc_core<T, M, NCOL>(qbar, kbar, gmu[16 * r + g], gmu[16 * r + g + 8], w, yT, mat0, mat1, vmat, aux,
+                    sc_load_w<NCOL>(mW, w, r, g, t);
+                    sc_core<T, M, NCOL>(qbar, kbar, gmu[16 * r + g], gmu[16 * r + g + 8], w, yT, mat0, mat1, wmat, aux,
                                         iters, sl2, r, lane, 1 + GROUPS + grp);
                 }
             } else if (r < CW) {

@@ -8,7 +8,7 @@
 //   front    landmark means, every warp a share; [sync]; warp c: S_U of its 16
 //            landmarks against all tokens, its rows of W stay in registers in
 //            the very layout the core takes (no partial W, no combine);
-//   core     vc_core; its scratch overlays K, V and Qbar, Y^T one of its
+//   core     sc_core; its scratch overlays K, V and Qbar, Y^T one of its
 //            matrices; [sync]
 //   output   every warp a share of the 16-token tiles: S_L, G_L^n from the
 //            resident Q, O in place over Q; [sync]; one bulk store.
@@ -16,8 +16,8 @@
 // a group per SM, and the SM's other groups fill the wait.  Three groups of
 // four warps run per SM (73 KB each at N = 256), against two groups with 108 KB
 // and two token warps each on the grouped kernel.
-// Measured (bf16): 4096 units of 16x16 windows, d_h = 32: 0.93 -> 0.51 ms;
-// 8640 units of 8x8 windows, d_h = 30: 1.45 -> 0.79 ms.
+// Measured (bf16): 4096 units of 16x16 windows, d_h = 32: 0.93 -> 0.50 ms;
+// 8640 units of 8x8 windows, d_h = 30: 1.45 -> 0.78 ms.
 //
 // Every wait on an mbarrier is bounded; the warps of a group share its
 // barriers, and a wait that gives up is agreed on at the next one.
@@ -30,15 +30,15 @@ namespace tc {
 
 template <typename T, int M, int NCOL, int N>
 struct WideLayout {
-    using Sc = VcScratch<M>;
+    using Sc = ScScratch<M>;
     static constexpr int CW = Sc::CW;
     static constexpr int DS = (NCOL == 32) ? 30 : 32;
     static constexpr size_t ROWS = (size_t)N * DS * 2;
     static constexpr size_t G_Q = 0;
     static constexpr size_t G_KV = ROWS;  // K, V; the core's two matrices
     static constexpr size_t KV = ((2 * ROWS > 2 * Sc::MAT ? 2 * ROWS : 2 * Sc::MAT) + 15) / 16 * 16;
-    static constexpr size_t G_QV = G_KV + KV;  // Qbar; the core's V
-    static constexpr size_t QV = LmS<T>::bytes(M) > Sc::VMAT ? LmS<T>::bytes(M) : Sc::VMAT;
+    static constexpr size_t G_QV = G_KV + KV;  // Qbar; the core's W
+    static constexpr size_t QV = LmS<T>::bytes(M) > Sc::WMAT ? LmS<T>::bytes(M) : Sc::WMAT;
     static constexpr size_t G_KBAR = G_QV + QV;
     static constexpr size_t G_AUX = G_KBAR + LmS<T>::bytes(M);
     static constexpr size_t G_BAR = G_AUX + Sc::AUX;  // Q and K rows; V rows
@@ -254,7 +254,7 @@ nystra_wide_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
         }
         // ---------------- core ----------------
         // (its first write to the K and V rows comes after a barrier of its own)
-        const T* yT = vc_core<T, M, NCOL>(qbar, kbar, run0, run1, w, nullptr, gb + Lay::G_KV,
+        const T* yT = sc_core<T, M, NCOL>(qbar, kbar, run0, run1, w, nullptr, gb + Lay::G_KV,
                                           gb + Lay::G_KV + Sc::MAT, gb + Lay::G_QV,
                                           reinterpret_cast<float*>(gb + Lay::G_AUX), iters, sl2, c, lane, bar);
         gsync();

@@ -1,6 +1,6 @@
-"""The wide-landmark kernel (m = 64 at 8x8 and 16x16 windows) and its core,
-which carries V = Z W column by column: one group up to many, no steps to many,
-the narrowest and widest heads, and columns of V of very different scales."""
+"""The wide-landmark kernel (m = 64 at 8x8 and 16x16 windows) and its core of
+symmetric products: one group up to many, no steps to many, the narrowest and
+widest heads, and columns of V of very different scales."""
 import numpy as np
 import pytest
 import torch
