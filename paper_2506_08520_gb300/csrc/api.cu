@@ -373,13 +373,13 @@ unsigned int take_fault_words(cudaStream_t stream, cudaError_t* err) {
     *err = cudaStreamSynchronize(stream);
     if (*err != cudaSuccess) return 0u;
     unsigned int w = 0;
-    unsigned int (*const take[17])(cudaError_t*) = {
+    unsigned int (*const take[16])(cudaError_t*) = {
         take_fault_word_tc_n64,       take_fault_word_tc_n256,       take_fault_word_tc_n1024,
         take_fault_word_tc_n64_s16,   take_fault_word_tc_n256_s16,   take_fault_word_tc_n1024_s16,
-        take_fault_word_exact_tc,     take_fault_word_debug,         take_fault_word_qkv_bf16,
-        take_fault_word_qkv_f16,      take_fault_word_qkv_bf16_s16,  take_fault_word_qkv_f16_s16,
-        take_fault_word_qkvs_bf16,    take_fault_word_qkvs_f16,      take_fault_word_qkvs_bf16_s16,
-        take_fault_word_qkvs_f16_s16, take_fault_word_proj};
+        take_fault_word_debug,        take_fault_word_qkv_bf16,      take_fault_word_qkv_f16,
+        take_fault_word_qkv_bf16_s16, take_fault_word_qkv_f16_s16,   take_fault_word_qkvs_bf16,
+        take_fault_word_qkvs_f16,     take_fault_word_qkvs_bf16_s16, take_fault_word_qkvs_f16_s16,
+        take_fault_word_proj};
     for (auto f : take) {
         w |= f(err);
         if (*err != cudaSuccess) return w;

@@ -138,7 +138,6 @@ unsigned int take_fault_word_tc_n1024_s16(cudaError_t* err);
 bool exact_tc_supports(int N, int d, int dtype);
 cudaError_t launch_exact_tc(const void* q, const void* k, const void* v, void* out, long long n_units, int N,
                             int d, int dtype, cudaStream_t stream);
-unsigned int take_fault_word_exact_tc(cudaError_t* err);
 // Device-side fault words (bit 0: a bounded wait gave up) of the translation
 // units whose kernels wait on barriers: OR-ed together, then cleared.
 unsigned int take_fault_words(cudaStream_t stream, cudaError_t* err);

@@ -2,226 +2,303 @@
 // even d_h <= 32; 16-bit I/O for windows of N = 64, 256 or 1024 tokens, fp32
 // I/O (split bf16 operands, three MMAs per product) for N = 64 and 256.
 //
-// A group of WPU = N/64 warps processes one (window, head) unit; warp r
-// bulk-copies rows [64r, 64r+64) of Q, K and V into its private stage (one
-// mbarrier, bounded wait), and after a group barrier every warp reads all of
-// the group's K and V.  Warp r computes the output rows it staged, one
-// 16-row tile at a time, streaming the keys in 64-token chunks with the
-// online (running-max) softmax: S = Q K_c^T (mma.sync, fp32 accumulate),
-// P = exp(S - m) in registers fed directly as the A operand of P [V_c | 1],
-// whose last column accumulates the row sums of the same rounded P.  Scores
-// are scaled by log2(e)/sqrt(d_h) so each exponential is one FFMA and one ex2.
-// This is the computation PnP-Nystra replaces; it is the in-library
-// comparator.
+// A group of WPU = N/64 warps processes one (window, head) unit.  Its K and V
+// are laid out in shared memory in rows of 40 16-bit values (fp32: a hi and a
+// lo plane), padded with zeros and, in V, a ones column, so that every B
+// fragment comes from ldmatrix without bank conflicts (rows of 60 bytes, as
+// they lie in HBM, take a 4-byte load and, for V, an 8x8 transpose per
+// register, with two-way conflicts).  Warp r computes output rows 64r .. 64r +
+// 63, 32 at a time so that a fragment serves two 16-row tiles, streaming the
+// keys in chunks of 32 with the online (running-max) softmax: S = Q K_c^T
+// (mma.sync, fp32 accumulate), P = exp(S - m) in registers fed directly as the
+// A operand of P [V_c | 1], whose last column accumulates the row sums of the
+// same rounded P.  Scores are scaled by log2(e)/sqrt(d_h) so each exponential
+// is half a packed FMA and one ex2.  This is the computation PnP-Nystra
+// replaces; it is the in-library comparator.
+//
+// What bounds it: at 32x32 windows the tensor pipe, 69% busy (32 MMAs and 32
+// ex2 per warp for 32 rows and 32 keys); at 16x16 windows also laying out K and
+// V, at 8x8 windows HBM.  The next unit's rows are brought to L2 meanwhile.
+// Measured (d_h = 30, bf16) against fragments loaded from 60-byte rows by one
+// 16-row tile: 5520 units of 32x32 windows 3.33 -> 1.98 ms, 6144 of 16x16
+// 0.27 -> 0.19 ms, 86400 of 8x8 266 -> 253 us; fp32, 2000 units of 16x16: 0.50 ->
+// 0.16 ms.
 #include "common.cuh"
 #include "ptx.cuh"
 
 namespace nystra {
-
-__device__ unsigned int g_fault_exact_tc;  // bit 0: a bounded wait gave up
-
 namespace {
 
-constexpr uint64_t kWaitNs = 2000000000ull;
 constexpr size_t kSmemLimit = 232448;
+constexpr int kRow = 40;  // 16-bit values per staged row: 80 bytes, an odd number of granules
 
-template <typename T, int NCOL, int WPU>
-struct ExactLayout {
-    static constexpr int DS = (NCOL == 32) ? 30 : 32;
-    static constexpr size_t STAGE = 3 * 64 * (size_t)DS * sizeof(T);
-    static constexpr size_t WARP_BYTES = ((STAGE + 127) / 128) * 128;
-    static constexpr size_t GROUP_BYTES = ((8 * WPU + 16 + 127) / 128) * 128;  // mbarriers + flag
-    static constexpr size_t PER_GROUP = GROUP_BYTES + WPU * WARP_BYTES;
+template <typename T>
+struct ExactOp {  // 16-bit I/O: one plane
+    using E = T;
+    static constexpr int NP = 1;
+    // per SM, with two key chunks unrolled: at N = 64 twelve warps of up to 168
+    // registers beat sixteen (86400 units: 253 against 267 us), elsewhere not
+    static constexpr int warps(int wpu) { return wpu == 1 ? 12 : 16; }
+};
+template <>
+struct ExactOp<float> {
+    using E = __nv_bfloat16;
+    static constexpr int NP = 2;
+    static constexpr int warps(int) { return 8; }
 };
 
-template <typename T, int NCOL, int WPU, int GROUPS>
-__global__ void __launch_bounds__(GROUPS * WPU * 32, 1)
-exact_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-                T* __restrict__ out, long long n_units, int d, float sl2, unsigned int* fault) {
-    using Lay = ExactLayout<T, NCOL, WPU>;
+template <typename T, int WPU>
+struct ExactLayout {
+    static constexpr int N = 64 * WPU;
+    static constexpr size_t PLANE = (size_t)N * kRow * 2;
+    static constexpr size_t GROUP = 2 * ExactOp<T>::NP * PLANE;  // K, then V
+    static constexpr int by_smem = (int)(kSmemLimit / GROUP);
+    static constexpr int by_warps = ExactOp<T>::warps(WPU) / WPU;
+    static constexpr int GROUPS = by_smem < by_warps ? by_smem : by_warps;
+    static_assert(GROUPS >= 1, "does not fit");
+};
+
+// Two elements at p as an operand register (fp32: a split pair).
+__device__ __forceinline__ uint32_t ld_global2(const __nv_bfloat16* p) { return __ldg(reinterpret_cast<const unsigned*>(p)); }
+__device__ __forceinline__ uint32_t ld_global2(const __half* p) { return __ldg(reinterpret_cast<const unsigned*>(p)); }
+__device__ __forceinline__ RegPair ld_global2(const float* p) {
+    const float2 x = __ldg(reinterpret_cast<const float2*>(p));
+    return Opnd<float>::pk(x.x, x.y);
+}
+// Four elements at p, and their operand registers 0 and 1.
+__device__ __forceinline__ uint2 ld_global4(const __nv_bfloat16* p) { return __ldg(reinterpret_cast<const uint2*>(p)); }
+__device__ __forceinline__ uint2 ld_global4(const __half* p) { return __ldg(reinterpret_cast<const uint2*>(p)); }
+__device__ __forceinline__ float4 ld_global4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ uint32_t word(uint2 x, int i) { return i ? x.y : x.x; }
+__device__ __forceinline__ RegPair word(float4 x, int i) { return i ? Opnd<float>::pk(x.z, x.w) : Opnd<float>::pk(x.x, x.y); }
+__device__ __forceinline__ void st_plane(unsigned char* p, size_t, uint32_t x) { *reinterpret_cast<uint32_t*>(p) = x; }
+__device__ __forceinline__ void st_plane(unsigned char* p, size_t plane, RegPair x) {
+    *reinterpret_cast<uint32_t*>(p) = x.hi;
+    *reinterpret_cast<uint32_t*>(p + plane) = x.lo;
+}
+
+// ldmatrix x4 (TR: transposed) as operand registers.
+template <bool TR>
+__device__ __forceinline__ void ld_frag(uint32_t (&r)[4], const unsigned char* p, size_t) {
+    if (TR) ldsm_x4_t(r, p);
+    else ldsm_x4(r, p);
+}
+template <bool TR>
+__device__ __forceinline__ void ld_frag(RegPair (&r)[4], const unsigned char* p, size_t plane) {
+    uint32_t h[4], l[4];
+    ld_frag<TR>(h, p, 0);
+    ld_frag<TR>(l, p + plane, 0);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r[i] = {h[i], l[i]};
+}
+
+template <typename T, int NCOL, int WPU, int DC>
+__global__ void __launch_bounds__(ExactLayout<T, WPU>::GROUPS * WPU * 32, 1)
+exact_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ out,
+                long long n_units, int d_in, float sl2) {
+    using Lay = ExactLayout<T, WPU>;
     using O = Opnd<T>;
     using R = typename O::Reg;
-    constexpr int N = 64 * WPU, NTO = NCOL / 8;
+    constexpr int N = Lay::N, NTO = NCOL / 8, GROUPS = Lay::GROUPS;
+    constexpr size_t PL = Lay::PLANE;
+    const int d = DC ? DC : d_in, h = d >> 1;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int grp = warp / WPU, r = warp - grp * WPU;
+    const int grp = warp / WPU, r = warp - grp * WPU, id = r * 32 + lane;
     const int g = lane >> 2, t = lane & 3;
-    unsigned char* gb = smem_raw + (size_t)grp * Lay::GROUP_BYTES;
-    unsigned char* wbase0 = smem_raw + (size_t)GROUPS * Lay::GROUP_BYTES + (size_t)(grp * WPU) * Lay::WARP_BYTES;
-    const int td = 64 * d;
-    auto stage_q = [&](int s) { return reinterpret_cast<T*>(wbase0 + (size_t)s * Lay::WARP_BYTES); };
-    T* Qs = stage_q(r);
-    uint64_t* bar = reinterpret_cast<uint64_t*>(gb) + r;
-    volatile unsigned int* gflag = reinterpret_cast<volatile unsigned int*>(gb + 8 * WPU);
-
+    unsigned char* Ks = smem_raw + (size_t)grp * Lay::GROUP;
+    unsigned char* Vs = Ks + ExactOp<T>::NP * PL;
     auto gsync = [&]() {
         if constexpr (WPU == 1) __syncwarp();
         else named_barrier(1 + grp, WPU * 32);
     };
-    const long long stride = (long long)gridDim.x * GROUPS;
-    long long u = (long long)blockIdx.x * GROUPS + grp;
-    const uint32_t tile_bytes = (uint32_t)(td * sizeof(T));
-    auto issue = [&](long long unit) {
-        const size_t off = (size_t)unit * N * d + (size_t)r * td;
-        mbar_arrive_expect_tx(bar, 3u * tile_bytes);
-        bulk_g2s(Qs, q + off, tile_bytes, bar);
-        bulk_g2s(Qs + td, k + off, tile_bytes, bar);
-        bulk_g2s(Qs + 2 * td, v + off, tile_bytes, bar);
-    };
-    if (lane == 0) {
-        mbar_init(bar, 1);
-        fence_mbar_init();
-        if (r == 0) *gflag = 0u;
+    // columns d .. 31: zeros, in V a ones column first (d = 32 has it as a constant fragment)
+    for (int i = id; i < N * (kRow / 2 - h); i += WPU * 32) {
+        const int row = i / (kRow / 2 - h), c = h + i - row * (kRow / 2 - h);
+        st_plane(Ks + (row * kRow + 2 * c) * 2, PL, O::zero());
+        st_plane(Vs + (row * kRow + 2 * c) * 2, PL, c == h ? O::one() : O::zero());
     }
-    gsync();
-    if (u < n_units && lane == 0) issue(u);
-    uint32_t phase = 0;
-    const int jd = d >> 3, tdn = (d & 7) >> 1, src = (lane & ~3) | tdn;
+    // fragment addresses: rows 8 (lane / 8) .. of an ldmatrix x4
+    const unsigned char* kf = Ks + ((lane & 7) * kRow + 8 * (lane >> 3)) * 2;                              // 8 keys x 32
+    const unsigned char* vf = Vs + (((lane & 7) + 8 * ((lane >> 3) & 1)) * kRow + 8 * (lane >> 4)) * 2;  // 16 keys x 16
+    R one0;  // B fragment of the ones column at d = 32: column 0 (lanes g = 0) is 1
+    if constexpr (NCOL > 32) one0 = g == 0 ? O::pk(1.f, 1.f) : O::zero();
+    const int jd = d >> 3, src = (lane & ~3) | ((d & 7) >> 1);
 
-    for (; u < n_units; u += stride) {
-        const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, phase, kWaitNs));
-        if (!ok && lane == 0) {
-            atomicOr(fault, 1u);
-            *gflag = 1u;
+    for (long long u = (long long)blockIdx.x * GROUPS + grp; u < n_units; u += (long long)gridDim.x * GROUPS) {
+        const size_t base = (size_t)u * N * d;
+        const long long un = u + (long long)gridDim.x * GROUPS;
+        if (id == 0 && un < n_units) {  // the next unit's rows on their way to L2
+            const size_t nb = (size_t)un * N * d;
+            const uint32_t bytes = (uint32_t)(N * d * sizeof(T));
+            bulk_prefetch_l2(k + nb, bytes);
+            bulk_prefetch_l2(v + nb, bytes);
+            bulk_prefetch_l2(q + nb, bytes);
         }
-        phase ^= 1u;
-        gsync();  // every warp's K and V rows are in place
-        if (*gflag != 0u) break;
-
-        T* obase = out + (size_t)u * N * d + (size_t)r * td;
-#pragma unroll 1
-        for (int tm = 0; tm < 4; ++tm) {
-            R aq[2][4];
-            const T* q0 = Qs + (16 * tm + g) * d;
-            const T* q1 = q0 + 8 * d;
+        gsync();  // every warp is done with the previous unit's K and V
+        {
+            // four elements (two words) a load; word i of the unit belongs to row i / h, 20 words long here
+            const T* ku = k + base;
+            const T* vu = v + base;
+            constexpr int U = 4;
+            const int n = N * h / 2;
+            for (int i0 = id; i0 < n; i0 += U * WPU * 32) {
+                decltype(ld_global4(ku)) x[U], y[U];
 #pragma unroll
-            for (int kk = 0; kk < 2; ++kk) {
-                const int c0 = 16 * kk + 2 * t, c1 = c0 + 8;
-                aq[kk][0] = c0 < d ? O::ld(q0 + c0) : O::zero();
-                aq[kk][1] = c0 < d ? O::ld(q1 + c0) : O::zero();
-                aq[kk][2] = c1 < d ? O::ld(q0 + c1) : O::zero();
-                aq[kk][3] = c1 < d ? O::ld(q1 + c1) : O::zero();
+                for (int e = 0; e < U; ++e) {
+                    const int i = min(i0 + e * WPU * 32, n - 1);
+                    x[e] = ld_global4(ku + 4 * i);
+                    y[e] = ld_global4(vu + 4 * i);
+                }
+#pragma unroll
+                for (int e = 0; e < U; ++e) {
+                    const int i = 2 * min(i0 + e * WPU * 32, n - 1);  // the last words may be written twice
+                    const int a0 = 4 * i + (i / h) * (2 * kRow - 4 * h), a1 = 4 * (i + 1) + ((i + 1) / h) * (2 * kRow - 4 * h);
+                    st_plane(Ks + a0, PL, word(x[e], 0));
+                    st_plane(Ks + a1, PL, word(x[e], 1));
+                    st_plane(Vs + a0, PL, word(y[e], 0));
+                    st_plane(Vs + a1, PL, word(y[e], 1));
+                }
             }
-            float o[NTO][4];
-#pragma unroll
-            for (int j = 0; j < NTO; ++j) o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
-            float run0 = -INFINITY, run1 = -INFINITY;
+        }
+        gsync();
 #pragma unroll 1
-            for (int c = 0; c < WPU; ++c) {
-                const T* Kc = stage_q(c) + td;
-                const T* Vc = stage_q(c) + 2 * td;
-                float s[8][4];
+        for (int blk = 0; blk < 2; ++blk) {
+            const T* q0 = q + base + (size_t)(64 * r + 32 * blk + g) * d;
+            R aq[2][2][4];
 #pragma unroll
-                for (int nt = 0; nt < 8; ++nt) {
-                    s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
-                    const T* kr = Kc + (8 * nt + g) * d;
+            for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-                    for (int kk = 0; kk < 2; ++kk) {
-                        const int c0 = 16 * kk + 2 * t, c1 = c0 + 8;
-                        O::mma(s[nt], aq[kk], c0 < d ? O::ld(kr + c0) : O::zero(),
-                               c1 < d ? O::ld(kr + c1) : O::zero());
+                for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int c = 16 * kk + 8 * (e >> 1) + 2 * t;
+                        aq[mt][kk][e] = c < d ? ld_global2(q0 + (16 * mt + 8 * (e & 1)) * d + c) : O::zero();
+                    }
+            float o[2][NTO][4], run[2][2];
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+                run[mt][0] = run[mt][1] = -INFINITY;
+#pragma unroll
+                for (int j = 0; j < NTO; ++j) o[mt][j][0] = o[mt][j][1] = o[mt][j][2] = o[mt][j][3] = 0.f;
+            }
+#pragma unroll 2
+            for (int c = 0; c < N; c += 32) {
+                float s[2][4][4];
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) {
+                    R b[4];
+                    ld_frag<false>(b, kf + (c + 8 * nt) * kRow * 2, PL);
+#pragma unroll
+                    for (int mt = 0; mt < 2; ++mt) {
+                        O::mmaz(s[mt][nt], aq[mt][0], b[0], b[1]);
+                        O::mma(s[mt][nt], aq[mt][1], b[2], b[3]);
                     }
                 }
-                float mx0 = run0, mx1 = run1;
+                // running maxima; the accumulators are rescaled
 #pragma unroll
-                for (int nt = 0; nt < 8; ++nt) {
-                    mx0 = fmaxf(mx0, fmaxf(s[nt][0], s[nt][1]) * sl2);
-                    mx1 = fmaxf(mx1, fmaxf(s[nt][2], s[nt][3]) * sl2);
+                for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        float m = fmaxf(s[mt][0][2 * e], s[mt][0][2 * e + 1]);
+#pragma unroll
+                        for (int nt = 1; nt < 4; ++nt) m = fmaxf(m, fmaxf(s[mt][nt][2 * e], s[mt][nt][2 * e + 1]));
+                        m = fmaxf(run[mt][e], quad_max(m) * sl2);
+                        const float f = ex2(run[mt][e] - m);
+                        run[mt][e] = m;
+#pragma unroll
+                        for (int j = 0; j < NTO; ++j) mul_x2(o[mt][j][2 * e], o[mt][j][2 * e + 1], f);
+                    }
+#pragma unroll
+                for (int kt = 0; kt < 2; ++kt) {
+                    R a[2][4];
+#pragma unroll
+                    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const float* x = s[mt][2 * kt + (e >> 1)] + 2 * (e & 1);
+                            const float m = -run[mt][e & 1];
+                            float p0, p1;
+                            fma_x2(p0, p1, x[0], x[1], sl2, sl2, m, m);
+                            a[mt][e] = O::pk(ex2(p0), ex2(p1));
+                        }
+#pragma unroll
+                    for (int j = 0; j < 4; j += 2) {
+                        R b[4];
+                        ld_frag<true>(b, vf + ((c + 16 * kt) * kRow + 8 * j) * 2, PL);
+#pragma unroll
+                        for (int mt = 0; mt < 2; ++mt) {
+                            O::mma(o[mt][j], a[mt], b[0], b[1]);
+                            O::mma(o[mt][j + 1], a[mt], b[2], b[3]);
+                        }
+                    }
+                    if constexpr (NCOL > 32) {
+#pragma unroll
+                        for (int mt = 0; mt < 2; ++mt) O::mma(o[mt][4], a[mt], one0, one0);
+                    }
                 }
-                mx0 = quad_max(mx0);
-                mx1 = quad_max(mx1);
-                const float f0 = ex2(run0 - mx0), f1 = ex2(run1 - mx1);
+            }
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+                float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+                for (int j = 0; j < NTO; ++j)
+                    if (j == jd) {
+                        d0 = o[mt][j][0];
+                        d1 = o[mt][j][2];
+                    }
+                const float i0 = __fdividef(1.f, __shfl_sync(0xffffffffu, d0, src));
+                const float i1 = __fdividef(1.f, __shfl_sync(0xffffffffu, d1, src));
+                T* o0 = out + base + (size_t)(64 * r + 32 * blk + 16 * mt + g) * d;
+                T* o1 = o0 + 8 * d;
 #pragma unroll
                 for (int j = 0; j < NTO; ++j) {
-                    o[j][0] *= f0; o[j][1] *= f0; o[j][2] *= f1; o[j][3] *= f1;
-                }
-                run0 = mx0;
-                run1 = mx1;
-#pragma unroll
-                for (int kt = 0; kt < 4; ++kt) {
-                    R a[4];
-                    a[0] = O::pk(ex2(fmaf(s[2 * kt][0], sl2, -mx0)), ex2(fmaf(s[2 * kt][1], sl2, -mx0)));
-                    a[1] = O::pk(ex2(fmaf(s[2 * kt][2], sl2, -mx1)), ex2(fmaf(s[2 * kt][3], sl2, -mx1)));
-                    a[2] = O::pk(ex2(fmaf(s[2 * kt + 1][0], sl2, -mx0)), ex2(fmaf(s[2 * kt + 1][1], sl2, -mx0)));
-                    a[3] = O::pk(ex2(fmaf(s[2 * kt + 1][2], sl2, -mx1)), ex2(fmaf(s[2 * kt + 1][3], sl2, -mx1)));
-#pragma unroll
-                    for (int j = 0; j < NTO; ++j) {
-                        const int c0 = 8 * j + 2 * t;
-                        const R x0 = c0 < d ? O::ld(Vc + (16 * kt + g) * d + c0) : (c0 == d ? O::one() : O::zero());
-                        const R x1 =
-                            c0 < d ? O::ld(Vc + (16 * kt + 8 + g) * d + c0) : (c0 == d ? O::one() : O::zero());
-                        O::mma(o[j], a, O::tr(x0), O::tr(x1));
+                    const int c = 8 * j + 2 * t;
+                    if (c < d) {
+                        O::st2(o0 + c, o[mt][j][0] * i0, o[mt][j][1] * i0);
+                        O::st2(o1 + c, o[mt][j][2] * i1, o[mt][j][3] * i1);
                     }
                 }
             }
-            float d0 = 0.f, d1 = 0.f;
-#pragma unroll
-            for (int j = 0; j < NTO; ++j)
-                if (j == jd) {
-                    d0 = o[j][0];
-                    d1 = o[j][2];
-                }
-            const float i0 = __fdividef(1.f, __shfl_sync(0xffffffffu, d0, src));
-            const float i1 = __fdividef(1.f, __shfl_sync(0xffffffffu, d1, src));
-            T* o0 = obase + (16 * tm + g) * d;
-            T* o1 = o0 + 8 * d;
-#pragma unroll
-            for (int j = 0; j < NTO; ++j) {
-                const int c = 8 * j + 2 * t;
-                if (c < d) {
-                    O::st2(o0 + c, o[j][0] * i0, o[j][1] * i0);
-                    O::st2(o1 + c, o[j][2] * i1, o[j][3] * i1);
-                }
-            }
-        }
-        gsync();  // no warp reads another warp's stage any more
-        const long long un = u + stride;
-        if (un < n_units && lane == 0) {
-            fence_proxy_async_smem();
-            issue(un);
         }
     }
 }
 
-template <typename T, int NCOL, int WPU>
-cudaError_t launch_cfg(const void* q, const void* k, const void* v, void* out, long long n_units, int d,
-                       cudaStream_t stream, unsigned int* fault) {
-    using Lay = ExactLayout<T, NCOL, WPU>;
-    constexpr int by_smem = (int)(kSmemLimit / Lay::PER_GROUP);
-    // at most 512 threads (registers stay <= 128), 256 with split fp32 operands
-    constexpr int by_threads = (sizeof(T) == 4 ? 8 : 16) / WPU;
-    constexpr int kGroups = by_smem < by_threads ? by_smem : by_threads;
-    static_assert(kGroups >= 1, "does not fit");
-    auto kern = exact_tc_kernel<T, NCOL, WPU, kGroups>;
-    const size_t smem = (size_t)kGroups * Lay::PER_GROUP;
+template <typename T, int NCOL, int WPU, int DC>
+cudaError_t launch_dc(const void* q, const void* k, const void* v, void* out, long long n_units, int d,
+                      cudaStream_t stream) {
+    using Lay = ExactLayout<T, WPU>;
+    constexpr int kThreads = Lay::GROUPS * WPU * 32;
+    auto kern = exact_tc_kernel<T, NCOL, WPU, DC>;
+    const size_t smem = (size_t)Lay::GROUPS * Lay::GROUP;
     static std::atomic<int> s_blocks[kMaxDevices];  // persistent grid size per device
     int blocks = 0;
-    if (cudaError_t e = persistent_grid(kern, kGroups * WPU * 32, smem, s_blocks, &blocks); e != cudaSuccess)
-        return e;
-    const long long want = (n_units + kGroups - 1) / kGroups;
+    if (cudaError_t e = persistent_grid(kern, kThreads, smem, s_blocks, &blocks); e != cudaSuccess) return e;
+    const long long want = (n_units + Lay::GROUPS - 1) / Lay::GROUPS;
     const long long grid = want < blocks ? want : blocks;
     const float sl2 = 1.4426950408889634f / sqrtf((float)d);
-    kern<<<(unsigned)grid, kGroups * WPU * 32, smem, stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)out,
-                                                              n_units, d, sl2, fault);
+    kern<<<(unsigned)grid, kThreads, smem, stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)out, n_units, d, sl2);
     return cudaGetLastError();
+}
+
+// The common head widths get kernels with d_h as a compile-time constant.
+template <typename T, int WPU>
+cudaError_t launch_n(const void* q, const void* k, const void* v, void* out, long long n_units, int d,
+                     cudaStream_t stream) {
+    if (d == 32) return launch_dc<T, 40, WPU, 32>(q, k, v, out, n_units, d, stream);
+    if (d == 30) return launch_dc<T, 32, WPU, 30>(q, k, v, out, n_units, d, stream);
+    return launch_dc<T, 32, WPU, 0>(q, k, v, out, n_units, d, stream);
 }
 
 template <typename T>
 cudaError_t launch_t(const void* q, const void* k, const void* v, void* out, long long n_units, int N, int d,
-                     cudaStream_t stream, unsigned int* fault) {
-    const bool wide = d > 30;
+                     cudaStream_t stream) {
     switch (N) {
-        case 64:
-            return wide ? launch_cfg<T, 40, 1>(q, k, v, out, n_units, d, stream, fault)
-                        : launch_cfg<T, 32, 1>(q, k, v, out, n_units, d, stream, fault);
-        case 256:
-            return wide ? launch_cfg<T, 40, 4>(q, k, v, out, n_units, d, stream, fault)
-                        : launch_cfg<T, 32, 4>(q, k, v, out, n_units, d, stream, fault);
+        case 64: return launch_n<T, 1>(q, k, v, out, n_units, d, stream);
+        case 256: return launch_n<T, 4>(q, k, v, out, n_units, d, stream);
         default:
             if constexpr (sizeof(T) == 4) return cudaErrorInvalidValue;  // not offered (see supports)
-            else
-                return wide ? launch_cfg<T, 40, 16>(q, k, v, out, n_units, d, stream, fault)
-                            : launch_cfg<T, 32, 16>(q, k, v, out, n_units, d, stream, fault);
+            else return launch_n<T, 16>(q, k, v, out, n_units, d, stream);
     }
 }
 
@@ -237,25 +314,8 @@ bool exact_tc_supports(int N, int d, int dtype) {
 
 cudaError_t launch_exact_tc(const void* q, const void* k, const void* v, void* out, long long n_units, int N,
                             int d, int dtype, cudaStream_t stream) {
-    static unsigned int* s_fault[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!s_fault[dev]) {
-        e = cudaGetSymbolAddress((void**)&s_fault[dev], nystra::g_fault_exact_tc);
-        if (e != cudaSuccess) return e;
-    }
-    if (dtype == 0) return nystra::launch_t<float>(q, k, v, out, n_units, N, d, stream, s_fault[dev]);
-    if (dtype == 1)
-        return nystra::launch_t<__nv_bfloat16>(q, k, v, out, n_units, N, d, stream, s_fault[dev]);
-    return nystra::launch_t<__half>(q, k, v, out, n_units, N, d, stream, s_fault[dev]);
-}
-
-unsigned int take_fault_word_exact_tc(cudaError_t* err) {
-    unsigned int w = 0, zero = 0;
-    *err = cudaMemcpyFromSymbol(&w, nystra::g_fault_exact_tc, sizeof(w));
-    if (*err == cudaSuccess && w != 0) *err = cudaMemcpyToSymbol(nystra::g_fault_exact_tc, &zero, sizeof(zero));
-    return w;
+    if (dtype == 0) return nystra::launch_t<float>(q, k, v, out, n_units, N, d, stream);
+    if (dtype == 1) return nystra::launch_t<__nv_bfloat16>(q, k, v, out, n_units, N, d, stream);
+    return nystra::launch_t<__half>(q, k, v, out, n_units, N, d, stream);
 }
 }  // namespace nystra_host

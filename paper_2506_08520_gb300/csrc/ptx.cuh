@@ -71,6 +71,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
         : "memory");
 }
 
+// Brings bytes (16-byte aligned, a multiple of 16) of global memory to L2.
+__device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
 // Named barrier over `nthreads` threads (a multiple of 32); id 0 is the one
 // __syncthreads uses, so groups of warps take ids 1..15.
 __device__ __forceinline__ void named_barrier(int id, int nthreads) {
@@ -137,6 +142,19 @@ __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+// Packed fp32 pairs: one instruction for both.
+__device__ __forceinline__ void fma_x2(float& d0, float& d1, float a0, float a1, float b0, float b1, float c0, float c1) {
+    asm("{\n .reg .b64 a, b, c;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mov.b64 c, {%6, %7};\n"
+        " fma.rn.f32x2 a, a, b, c;\n mov.b64 {%0, %1}, a;\n}\n"
+        : "=f"(d0), "=f"(d1)
+        : "f"(a0), "f"(a1), "f"(b0), "f"(b1), "f"(c0), "f"(c1));
+}
+__device__ __forceinline__ void mul_x2(float& d0, float& d1, float b) {
+    asm("{\n .reg .b64 a, b;\n mov.b64 a, {%0, %1};\n mov.b64 b, {%2, %2};\n mul.rn.f32x2 a, a, b;\n"
+        " mov.b64 {%0, %1}, a;\n}\n"
+        : "+f"(d0), "+f"(d1)
+        : "f"(b));
 }
 // Transpose of an 8x8 matrix of 16-bit elements held one row pair per lane
 // (lane 4r + c holds row r, columns 2c and 2c+1).
@@ -225,6 +243,13 @@ __device__ __forceinline__ H2Pair split_h2(float x0, float x1) {
 template <typename T> struct Mma16;
 
 template <> struct Mma16<__nv_bfloat16> {
+    // c = a b (no zeroed accumulator to set up)
+    static __device__ __forceinline__ void k16z(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+            "{%10,%10,%10,%10};"
+            : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+    }
     static __device__ __forceinline__ void k16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
         asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
             "{%0,%1,%2,%3};"
@@ -248,6 +273,13 @@ template <> struct Mma16<__nv_bfloat16> {
 };
 
 template <> struct Mma16<__half> {
+    // c = a b (no zeroed accumulator to set up)
+    static __device__ __forceinline__ void k16z(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+            "{%10,%10,%10,%10};"
+            : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+    }
     static __device__ __forceinline__ void k16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
         asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
             "{%0,%1,%2,%3};"
@@ -299,6 +331,9 @@ struct Opnd {
     static __device__ __forceinline__ Reg one() { return Op::kOne; }  // the pair (1, 0)
     static __device__ __forceinline__ void mma(float (&c)[4], const Reg (&a)[4], Reg b0, Reg b1) {
         Op::k16(c, a, b0, b1);
+    }
+    static __device__ __forceinline__ void mmaz(float (&c)[4], const Reg (&a)[4], Reg b0, Reg b1) {  // c = a b
+        Op::k16z(c, a, b0, b1);
     }
     static __device__ __forceinline__ void mma8(float (&c)[4], Reg a0, Reg a1, Reg b0) { Op::k8(c, a0, a1, b0); }
     static __device__ __forceinline__ void st2(T* p, float a, float b) {
@@ -360,6 +395,13 @@ struct Opnd<float> {
         const uint32_t ah[4] = {a[0].hi, a[1].hi, a[2].hi, a[3].hi};
         const uint32_t al[4] = {a[0].lo, a[1].lo, a[2].lo, a[3].lo};
         Op::k16(c, al, b0.hi, b1.hi);
+        Op::k16(c, ah, b0.lo, b1.lo);
+        Op::k16(c, ah, b0.hi, b1.hi);
+    }
+    static __device__ __forceinline__ void mmaz(float (&c)[4], const Reg (&a)[4], Reg b0, Reg b1) {  // c = a b
+        const uint32_t ah[4] = {a[0].hi, a[1].hi, a[2].hi, a[3].hi};
+        const uint32_t al[4] = {a[0].lo, a[1].lo, a[2].lo, a[3].lo};
+        Op::k16z(c, al, b0.hi, b1.hi);
         Op::k16(c, ah, b0.lo, b1.lo);
         Op::k16(c, ah, b0.hi, b1.hi);
     }

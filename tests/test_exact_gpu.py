@@ -1,0 +1,49 @@
+"""The tensor-core exact attention at the edges of its layout: every window
+size it takes, the narrowest and widest heads (padding columns, the ones column
+inside and beyond them), one unit up to several rounds of groups, fp32's split
+planes, and rows whose scores differ by far more than the exponential's range."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2506_08520_gb300 import binding, workloads
+from tests.parity import TOL, per_unit_rel, units_view
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2506_08520_gb300 import build
+    build.build()
+
+
+def _check(q, k, v, tol):
+    out = binding.exact(q.cuda(), k.cuda(), v.cuda())
+    torch.cuda.synchronize()
+    err = per_unit_rel(units_view(out.cpu()).double().numpy(), oracle.exact_attention(q, k, v))
+    assert err.max() <= tol, f"{err.max():.3e} at unit {int(np.argmax(err))}"
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
+@pytest.mark.parametrize("units,N,d", [(1, 64, 2), (1825, 64, 30), (3, 64, 32), (2, 64, 24), (1, 256, 2),
+                                       (609, 256, 30), (2, 256, 32), (3, 256, 18), (1, 1024, 30), (2, 1024, 32),
+                                       (3, 1024, 8)])
+def test_units_and_widths(units, N, d, dtype):
+    if N == 1024 and dtype == "f32":
+        pytest.skip("32x32 windows in fp32 take the generic kernel")
+    q, k, v = workloads.random_qkv(units, N, d, dtype, seed=units + N + d)
+    _check(q, k, v, TOL[dtype])
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
+@pytest.mark.parametrize("N", [64, 256])
+def test_late_maximum(N, dtype):
+    # the row maximum sits in the last key chunk and exceeds every earlier
+    # score by about 50: the accumulated rows are rescaled to nothing
+    q, k, v = workloads.random_qkv(2, N, 30, "f32", seed=N)
+    T = workloads.DTYPES[dtype]
+    k[:, -1] = 0.0
+    q[..., 0], k[..., 0] = 4.0, torch.linspace(-30, 30, N)
+    _check(q.to(T), k.to(T), v.to(T), TOL[dtype])
