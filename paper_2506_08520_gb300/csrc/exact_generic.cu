@@ -1,97 +1,183 @@
-// Generic exact window attention, Eq. (1): O = softmax(Q K^T / sqrt(d_h)) V.
+// Generic exact window attention, Eq. (1): O = softmax(Q K^T / sqrt(d_h)) V,
+// for any N <= 1024 and d_h <= 64, fp32 arithmetic with expf.
 //
-// One CTA (256 threads) per (window, head) unit; one thread per query row.
-// Keys and values are staged through shared memory in chunks of 32 tokens;
-// each thread keeps its query row and output accumulator in registers and
-// applies the online (running-max) form of the row softmax, which equals the
-// max-shifted Eq. (2) up to rounding.  fp32 arithmetic, correctly rounded expf.
-// Always available for any N <= 1024 and d_h <= 64.
-#include "common.cuh"
+// One CTA (256 threads) per block of 64 query rows of a (window, head) unit.
+// Keys and values are staged in chunks of 64 tokens; a thread computes a 4 x 4
+// tile of the chunk's scores and keeps it in registers through the row maximum
+// (shuffles over the 16 lanes of a row) and the exponentials, P is stored once,
+// and P V accumulates in 4 x 4 register tiles across the chunks, rescaled as
+// the running maxima grow: the online form of the row softmax, which equals
+// the max-shifted Eq. (2) up to rounding.  Products as in nystra_generic.cuh:
+// packed FMAs on rows contiguous along the contraction (V transposed), row
+// strides of an odd number of 16-byte granules.
+//
+// What bounds it: instruction issue (about a third of them packed FMAs).
+// Measured against one thread per query row with the scores in shared memory:
+// 600 units of 32x32 windows, d_h = 30, fp32 11.4 -> 3.5 ms; 3000 units of 12x12,
+// bf16 1.9 -> 0.65 ms; 108 units of 10x10, d_h = 33, fp32 203 -> 27 us.
+#include "simt.cuh"
 
 namespace nystra {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kChunk = 32;
+using namespace simt;
 
-template <typename T, int DMAX>
-__global__ void __launch_bounds__(kThreads)
-exact_generic_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-                     T* __restrict__ out, long long n_units, int N, int d, float scale) {
-    __shared__ float kb[kChunk * DMAX];
-    __shared__ float vb[kChunk * DMAX];
-    __shared__ float sc[kChunk * kThreads];
-    const int tid = threadIdx.x;
-    for (long long u = blockIdx.x; u < n_units; u += gridDim.x) {
+constexpr int kThreads = 256;
+constexpr int kRows = 64;           // query rows per CTA, keys per chunk
+constexpr int kNS = kRows + 4;      // row stride of anything with key columns
+constexpr int kG = kRows / 4;       // tile groups per row and column of the scores: 16 x 16 threads
+static_assert(kG * kG == kThreads && (kNS / 4) % 2 == 1, "one score tile per thread");
+
+// DS: row stride of d_h columns; c4: groups of four columns (at most kG, so that
+// every thread has at most one tile of O).
+template <int DS>
+struct Shape {
+    int c4;
+    __host__ __device__ explicit Shape(int d) : c4((d + 3) / 4) {}
+    __host__ __device__ size_t bytes() const {
+        // Q rows | K rows or V^T | P | row factors
+        const int kv = kRows * DS > 4 * c4 * kNS ? kRows * DS : 4 * c4 * kNS;
+        return sizeof(float) * (size_t)(kRows * DS + kv + kRows * kNS + kRows);
+    }
+};
+
+template <int DS, typename T>
+__device__ __forceinline__ void run(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
+                                    T* __restrict__ out, long long n_units, int N, int d, float scale, float* sm) {
+    const Shape<DS> G(d);
+    const int tid = threadIdx.x, c4 = G.c4, pl = 4 * c4 <= 16 ? 3 : (4 * c4 <= 32 ? 4 : 5);
+    float* Qs = sm;                                                           // kRows rows
+    float* KV = Qs + kRows * DS;                                              // K rows, then V^T
+    float* P = KV + (kRows * DS > 4 * c4 * kNS ? kRows * DS : 4 * c4 * kNS);  // [row][key]
+    float* fac = P + kRows * kNS;                                             // rescale factors, then 1 / denominators
+    const int j0 = tid % kG, t0 = tid / kG;  // score tile: keys j0 + kG j, rows t0 + kG i
+    // O tile: columns oc + c4 j (oc < c4), rows t0 + kG i; narrow heads leave
+    // lanes over, which take a half or a quarter of the keys each
+    const int wd = c4 <= 4 ? 4 : (c4 <= 8 ? 8 : kG), oc = j0 % wd, g0 = (j0 / wd) * wd;
+    const int blocks = (N + kRows - 1) / kRows;
+
+    for (long long w = blockIdx.x; w < n_units * blocks; w += gridDim.x) {
+        const long long u = w / blocks;
+        const int r0 = (int)(w - u * blocks) * kRows, nr = min(kRows, N - r0);
         const size_t base = (size_t)u * N * d;
-        for (int r0 = 0; r0 < N; r0 += kThreads) {
-            const int row = r0 + tid;
-            const bool active = row < N;
-            float qr[DMAX], acc[DMAX];
+        load_rows<T>(q + base + (size_t)r0 * d, nr, kG, d, 4 * c4, pl,
+                     [&](int r, int c, float2 x) { *reinterpret_cast<float2*>(Qs + r * DS + c) = x; });
+        float run_max[4], den[4], o[4][4];
 #pragma unroll
-            for (int c = 0; c < DMAX; ++c) {
-                qr[c] = (active && c < d) ? scale * ldg_f32(q + base + (size_t)row * d + c) : 0.f;
-                acc[c] = 0.f;
-            }
-            float mx = -INFINITY, den = 0.f;
-            for (int t0 = 0; t0 < N; t0 += kChunk) {
-                const int nt = min(kChunk, N - t0);
-                __syncthreads();
-                for (int idx = tid; idx < nt * d; idx += blockDim.x) {
-                    const int t = idx / d, c = idx - (idx / d) * d;
-                    kb[t * DMAX + c] = ldg_f32(k + base + (size_t)t0 * d + idx);
-                    vb[t * DMAX + c] = ldg_f32(v + base + (size_t)t0 * d + idx);
-                }
-                __syncthreads();
-                if (!active) continue;
-                // this thread's scores for the chunk, kept in shared memory
-                float* s = sc + tid;
-                float cmx = -INFINITY;
-#pragma unroll 2
-                for (int t = 0; t < nt; ++t) {
-                    float a = 0.f;
+        for (int i = 0; i < 4; ++i) {
+            run_max[i] = -INFINITY;
+            den[i] = 0.f;
 #pragma unroll
-                    for (int c = 0; c < DMAX; ++c)
-                        if (c < d) a = fmaf(qr[c], kb[t * DMAX + c], a);
-                    s[t * kThreads] = a;
-                    cmx = fmaxf(cmx, a);
-                }
-                const float nmx = fmaxf(mx, cmx);
-                const float r = (mx == -INFINITY) ? 0.f : expf(mx - nmx);
-                den *= r;
-#pragma unroll
-                for (int c = 0; c < DMAX; ++c) acc[c] *= r;
-                mx = nmx;
-#pragma unroll 2
-                for (int t = 0; t < nt; ++t) {
-                    const float p = expf(s[t * kThreads] - mx);
-                    den += p;
-#pragma unroll
-                    for (int c = 0; c < DMAX; ++c)
-                        if (c < d) acc[c] = fmaf(p, vb[t * DMAX + c], acc[c]);
-                }
-            }
-            if (active) {
-                const float inv = 1.f / den;
-#pragma unroll
-                for (int c = 0; c < DMAX; ++c)
-                    if (c < d) out[base + (size_t)row * d + c] = from_f32<T>(acc[c] * inv);
-            }
+            for (int j = 0; j < 4; ++j) o[i][j] = 0.f;
         }
+        for (int k0 = 0; k0 < N; k0 += kRows) {
+            const int nt = min(kRows, N - k0);
+            load_rows<T>(k + base + (size_t)k0 * d, nt, kG, d, 4 * c4, pl,
+                         [&](int r, int c, float2 x) { *reinterpret_cast<float2*>(KV + r * DS + c) = x; });
+            __syncthreads();
+            f32x2 acc[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+            tile_nt<4, 4>(Qs + t0 * DS, kG * DS, KV + j0 * DS, kG * DS, c4, acc);
+            float s[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float mx = run_max[i];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    s[i][j] = j0 + kG * j < nt ? scale * sum2(acc[i][j]) : -INFINITY;
+                    mx = fmaxf(mx, s[i][j]);
+                }
+#pragma unroll
+                for (int x = kG / 2; x > 0; x >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+                const float f = run_max[i] == -INFINITY ? 0.f : expf(run_max[i] - mx);
+                run_max[i] = mx;
+                den[i] *= f;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float p = j0 + kG * j < nt ? expf(s[i][j] - mx) : 0.f;
+                    den[i] += p;
+                    P[(t0 + kG * i) * kNS + j0 + kG * j] = p;
+                }
+                if (j0 == 0) fac[t0 + kG * i] = f;
+            }
+            __syncthreads();  // K has been read: V takes its place
+            load_rows<T>(v + base + (size_t)k0 * d, nt, kG, d, 4 * c4, pl, [&](int r, int c, float2 x) {
+                KV[c * kNS + r] = x.x;
+                KV[(c + 1) * kNS + r] = x.y;
+            });
+            __syncthreads();
+            if (oc < c4) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float f = fac[t0 + kG * i];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[i][j] = __float_as_uint(o[i][j] * f);  // (o f, 0)
+                }
+                tile_nt<4, 4>(P + t0 * kNS + 4 * g0, kG * kNS, KV + oc * kNS + 4 * g0, c4 * kNS, wd, acc);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) o[i][j] = sum2(acc[i][j]);
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+#pragma unroll
+            for (int x = kG / 2; x > 0; x >>= 1) den[i] += __shfl_xor_sync(0xffffffffu, den[i], x);
+            if (j0 == 0) fac[t0 + kG * i] = 1.f / den[i];
+        }
+        __syncthreads();
+        for (int x = wd; x < kG; x <<= 1)  // the splits' sums
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) o[i][j] += __shfl_xor_sync(0xffffffffu, o[i][j], x);
+        if (oc < c4 && g0 == 0) {  // O over the Q rows, then out in row order
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    Qs[(t0 + kG * i) * DS + oc + c4 * j] = o[i][j] * fac[t0 + kG * i];
+        }
+        __syncthreads();
+        {
+            const int c = 2 * (tid & ((1 << pl) - 1));
+            if (c < d)
+                for (int r = tid >> pl; r < nr; r += kThreads >> pl)
+                    st_pair<T>(out + base + (size_t)(r0 + r) * d, c, d, Qs[r * DS + c], Qs[r * DS + c + 1]);
+        }
+        __syncthreads();
     }
 }
 
-template <typename T>
-cudaError_t launch_t(const void* q, const void* k, const void* v, void* out, long long n_units, int N,
-                     int d, cudaStream_t stream) {
-    const long long grid = n_units < (1LL << 30) ? n_units : (1LL << 30);
-    const float scale = 1.0f / sqrtf((float)d);
-    if (d <= 32)
-        exact_generic_kernel<T, 32><<<(unsigned)grid, kThreads, 0, stream>>>(
-            (const T*)q, (const T*)k, (const T*)v, (T*)out, n_units, N, d, scale);
+template <int DS>
+__global__ void __launch_bounds__(kThreads, 2)
+exact_generic_kernel(const void* q, const void* k, const void* v, void* out, long long n_units, int N, int d,
+                     int dtype, float scale) {
+    extern __shared__ __align__(16) float sm[];
+    if (dtype == 0)
+        run<DS, float>((const float*)q, (const float*)k, (const float*)v, (float*)out, n_units, N, d, scale, sm);
+    else if (dtype == 1)
+        run<DS, __nv_bfloat16>((const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,
+                               (__nv_bfloat16*)out, n_units, N, d, scale, sm);
     else
-        exact_generic_kernel<T, 64><<<(unsigned)grid, kThreads, 0, stream>>>(
-            (const T*)q, (const T*)k, (const T*)v, (T*)out, n_units, N, d, scale);
+        run<DS, __half>((const __half*)q, (const __half*)k, (const __half*)v, (__half*)out, n_units, N, d, scale, sm);
+}
+
+template <int DS>
+cudaError_t launch_ds(const void* q, const void* k, const void* v, void* out, long long n_units, int N, int d,
+                      int dtype, cudaStream_t stream) {
+    static std::atomic<int> s_ready[kMaxDevices];
+    auto kern = exact_generic_kernel<DS>;
+    if (cudaError_t e = opt_in_smem(kern, s_ready); e != cudaSuccess) return e;
+    const long long want = n_units * ((N + kRows - 1) / kRows);
+    const long long grid = want < (1LL << 30) ? want : (1LL << 30);
+    kern<<<(unsigned)grid, kThreads, Shape<DS>(d).bytes(), stream>>>(q, k, v, out, n_units, N, d, dtype,
+                                                                      1.0f / sqrtf((float)d));
     return cudaGetLastError();
 }
 
@@ -99,13 +185,12 @@ cudaError_t launch_t(const void* q, const void* k, const void* v, void* out, lon
 }  // namespace nystra
 
 namespace nystra_host {
-cudaError_t launch_exact_generic(const void* q, const void* k, const void* v, void* out,
-                                 long long n_units, int N, int d, int dtype, cudaStream_t stream) {
+// Row strides: d_h columns padded to whole granules, an odd number of them.
+cudaError_t launch_exact_generic(const void* q, const void* k, const void* v, void* out, long long n_units, int N,
+                                 int d, int dtype, cudaStream_t stream) {
     using namespace nystra;
-    switch (dtype) {
-        case 0: return launch_t<float>(q, k, v, out, n_units, N, d, stream);
-        case 1: return launch_t<__nv_bfloat16>(q, k, v, out, n_units, N, d, stream);
-        default: return launch_t<__half>(q, k, v, out, n_units, N, d, stream);
-    }
+    if (d <= 20) return launch_ds<20>(q, k, v, out, n_units, N, d, dtype, stream);
+    if (d <= 36) return launch_ds<36>(q, k, v, out, n_units, N, d, dtype, stream);
+    return launch_ds<68>(q, k, v, out, n_units, N, d, dtype, stream);
 }
 }  // namespace nystra_host
