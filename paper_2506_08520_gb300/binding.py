@@ -6,6 +6,7 @@ There is no CPU fallback: if the library is missing, every call raises.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 
@@ -293,10 +294,13 @@ def nystra_biased(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, pooled, m: 
 def nystra_qkv(x: torch.Tensor, w_qkv: torch.Tensor, heads: int, m: int = 16, iters: int = 6,
                b_qkv: torch.Tensor | None = None, pooled=None, out: torch.Tensor | None = None, stream=None,
                landmarks: str = "segments", factors: str = "pairs") -> torch.Tensor:
-    """Fused projection + PnP-Nystra: tokens ``x`` ``[n_windows, N, C]``, weights
+    """Projection + PnP-Nystra: tokens ``x`` ``[n_windows, N, C]``, weights
     ``w_qkv`` ``[3C, C]`` (a linear layer's weight: Q rows, then K, then V),
     optional fp32 bias ``b_qkv`` ``[3C]`` and pooled score bias (as for
-    ``nystra_biased``).  Returns ``[n_windows, heads, N, C / heads]``."""
+    ``nystra_biased``).  Returns ``[n_windows, heads, N, C / heads]``.  Runs as
+    one fused kernel (nystra_attention_qkv) or, where that is faster, as the
+    projection and the attention by turns over a workspace of up to
+    ``QKV_WORKSPACE`` bytes (`_two_pass`)."""
     if x.dim() != 3 or w_qkv.dim() != 2:
         raise ValueError("expected x [n_windows, N, C] and w_qkv [3C, C]")
     nw, N, C = x.shape
@@ -323,12 +327,83 @@ def nystra_qkv(x: torch.Tensor, w_qkv: torch.Tensor, heads: int, m: int = 16, it
     if pooled is not None:
         bL, bU, bA = (t.data_ptr() for t in pooled)
         bw = pooled[0].numel() // (heads * N * m)
+    lm, dt = _lm(landmarks, factors), _DTYPE_CODE[x.dtype]
     with torch.cuda.device(x.device):
-        rc = nystra_attention_qkv(x.data_ptr(), w_qkv.data_ptr(), bp, out.data_ptr(), nw, heads, N, d, m, iters,
-                                  _lm(landmarks, factors), bL, bU, bA, bw, _DTYPE_CODE[x.dtype], _stream_ptr(stream))
+        two = _two_pass(nw, N, heads, d, m, iters, landmarks, x, w_qkv, b_qkv, pooled, bw, out, stream)
+        rc = _qkv_two_pass(x, w_qkv, bp, out, nw, heads, N, d, m, iters, lm, bL, bU, bA, bw, dt, stream) if two else None
+        if rc is None:
+            rc = nystra_attention_qkv(x.data_ptr(), w_qkv.data_ptr(), bp, out.data_ptr(), nw, heads, N, d, m, iters,
+                                      lm, bL, bU, bA, bw, dt, _stream_ptr(stream))
     if rc != NYSTRA_OK:
         raise NystraError(rc, "nystra_attention_qkv")
     return out
+
+
+# The two-pass form of nystra_qkv: the tcgen05 projection into a workspace of
+# at most QKV_WORKSPACE bytes, then the attention on it, window chunk by window
+# chunk.  Q, K and V are rounded to the I/O type in both forms.
+QKV_WORKSPACE = 256 << 20
+
+
+def _disjoint(out: torch.Tensor, t: torch.Tensor | None) -> bool:
+    if t is None:
+        return True
+    a, b = out.data_ptr(), t.data_ptr()
+    return a >= b + t.numel() * t.element_size() or b >= a + out.numel() * out.element_size()
+
+
+def _two_pass(nw, N, heads, d, m, iters, landmarks, x, w_qkv, b_qkv, pooled, bw, out, stream) -> bool:
+    """Whether nystra_qkv takes the two-pass form: where it is the faster one,
+    for calls that nystra_attention_qkv accepts (it refuses the others) on a
+    stream the workspace can be allocated for.
+
+    The lines, from GPU times of both forms (m = 16, fused / two-pass, us), where
+    the second call's 10 us of host time are to be hidden too: 32x32 windows
+    everywhere (1 x 16 features, 2048 tokens 48/33; 6 x 30, 262144 tokens
+    706/240); 16x16 windows from 128 token features on (4 x 32, 2048 tokens 49/34;
+    6 x 30, 262144 tokens 579/241) or 64 and 65536 tokens (2 x 32: 62/53; but 1 x
+    32: 28/33, and at 2048 tokens 4 x 24: 33/27); 8x8 windows from 80 features and
+    65536 tokens on (3 x 28: 54/49; 6 x 30: 125/84; but 2 x 32: 43/50, and at 32768
+    tokens 4 x 24: 35/41)."""
+    C, T = heads * d, nw * N
+    if not (N == 1024 or (N == 256 and (C >= 128 or (C >= 64 and T >= 65536)))
+            or (N == 64 and C >= 80 and T >= 65536)):
+        return False
+    inputs = (x, w_qkv, b_qkv) + (tuple(pooled) if pooled is not None else ())
+    return (x.dtype in (torch.bfloat16, torch.float16)
+            and (stream is None or isinstance(stream, torch.cuda.Stream))
+            and d % 2 == 0 and 2 <= d <= 32 and heads * d <= QKV_MAX_C and 0 <= iters <= 12
+            and (m in (8, 16) or (m == 32 and N == 1024 and pooled is None)) and (landmarks == "segments" or m == 16)
+            and (pooled is None or bw in (1, nw))
+            and all(t is None or (t.data_ptr() % 16 == 0 and _disjoint(out, t)) for t in inputs)
+            and out.data_ptr() % 16 == 0)
+
+
+def _qkv_two_pass(x, w_qkv, bp, out, nw, heads, N, d, m, iters, lm, bL, bU, bA, bw, dt, stream):
+    """The status code, or None if there is no memory for the workspace."""
+    win = heads * N * d * 2  # bytes of one window's Q (as of its tokens and its output)
+    per = max(1, min(nw, QKV_WORKSPACE // (3 * win)))
+    per = -(-nw // (-(-nw // per)))  # chunks of equal length
+    try:
+        # from the pool of the stream it is used on: safe to reuse in stream order once freed
+        with contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
+            ws = torch.empty(3 * per * win, dtype=torch.uint8, device=x.device)
+    except torch.OutOfMemoryError:
+        return None
+    q, k, v = (ws.data_ptr() + i * per * win for i in range(3))
+    xp, op, wp, st = x.data_ptr(), out.data_ptr(), w_qkv.data_ptr(), _stream_ptr(stream)
+    for i in range(0, nw, per):
+        n = min(per, nw - i)
+        rc = nystra_project_qkv(xp + i * win, wp, bp, q, k, v, n, heads, N, d, dt, st)
+        if rc == NYSTRA_OK and bL == 0:
+            rc = nystra_attention_ex(q, k, v, op + i * win, n, heads, N, d, m, iters, lm, dt, st)
+        elif rc == NYSTRA_OK:
+            u = i * heads * 4 if bw != 1 else 0  # per-window blocks: this chunk's first
+            rc = nystra_attention_bias(q, k, v, op + i * win, n, heads, N, d, m, iters, lm, bL + u * N * m,
+                                       bU + u * N * m, bA + u * m * m, n if bw != 1 else 1, dt, st)
+        if rc != NYSTRA_OK:
+            return rc
+    return NYSTRA_OK
 
 
 def project_qkv(x: torch.Tensor, w_qkv: torch.Tensor, heads: int, b_qkv: torch.Tensor | None = None,

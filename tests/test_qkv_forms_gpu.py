@@ -1,0 +1,98 @@
+"""nystra_qkv's two forms: the fused kernel (the C entry point) and the
+projection and attention by turns over a workspace, in one chunk and in several
+(a ragged last one, per-window score biases, streams), and the calls at the
+edges of the rule that picks between them."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2506_08520_gb300 import binding, workloads
+from tests.parity import TOL, per_unit_rel
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2506_08520_gb300 import build
+    build.build()
+
+
+def _fused(x, w, heads, m, iters, b, pooled, lm):
+    nw, N, C = x.shape
+    out = torch.empty((nw, heads, N, C // heads), dtype=x.dtype, device=x.device)
+    bl = [t.data_ptr() for t in pooled] if pooled is not None else [0, 0, 0]
+    bw = pooled[0].numel() // (heads * N * m) if pooled is not None else 0
+    rc = binding.nystra_attention_qkv(x.data_ptr(), w.data_ptr(), b.data_ptr(), out.data_ptr(), nw, heads, N,
+                                      C // heads, m, iters, binding.LANDMARKS[lm], *bl, bw,
+                                      binding._DTYPE_CODE[x.dtype], torch.cuda.current_stream().cuda_stream)
+    assert rc == binding.NYSTRA_OK
+    return out
+
+
+CASES = [  # windows, heads, N, d, m, pooling, bias (None, "heads", "windows"), dtype
+    (5, 2, 1024, 16, 8, "segments", None, "bf16"), (3, 1, 1024, 32, 32, "segments", None, "f16"),
+    (4, 2, 1024, 30, 16, "patches", "heads", "bf16"), (7, 4, 256, 32, 16, "segments", "windows", "bf16"),
+    (5, 6, 256, 30, 16, "patches", "windows", "f16"), (1027, 3, 64, 30, 16, "segments", "heads", "bf16"),
+    (1025, 4, 64, 20, 8, "segments", "windows", "f16"),
+]
+
+
+@pytest.mark.parametrize("nw,heads,N,d,m,lm,kind,dtype", CASES)
+def test_both_forms_match_the_oracle(nw, heads, N, d, m, lm, kind, dtype, monkeypatch):
+    x, w, b = workloads.random_x_wqkv(nw, N, heads, d, dtype, seed=N + m + d)
+    rng = np.random.default_rng(N)
+    bias = None if kind is None else torch.from_numpy(
+        0.3 * rng.standard_normal(((nw, heads) if kind == "windows" else (heads,)) + (N, N))).float()
+    xd, wd, bd = x.cuda(), w.cuda(), b.cuda()
+    pooled = None if bias is None else binding.pool_bias(bias.cuda(), m, lm)
+    assert binding._two_pass(nw, N, heads, d, m, 5, lm, xd, wd, bd, pooled, nw if kind == "windows" else 1,
+                             torch.empty_like(xd), None)
+    one = binding.nystra_qkv(xd, wd, heads, m, 5, b_qkv=bd, pooled=pooled, landmarks=lm)
+    fused = _fused(xd, wd, heads, m, 5, bd, pooled, lm)
+    monkeypatch.setattr(binding, "QKV_WORKSPACE", 3 * (nw // 2) * heads * N * d * 2)  # two or three chunks
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    some = binding.nystra_qkv(xd, wd, heads, m, 5, b_qkv=bd, pooled=pooled, landmarks=lm, stream=s)
+    s.synchronize()
+    torch.cuda.synchronize()
+    assert binding.status() == binding.NYSTRA_OK
+    assert torch.equal(one, some)  # every window on its own, whatever the chunks
+    idx = np.unique(np.linspace(0, nw - 1, 6).astype(int))
+    q, k, v = oracle.project_qkv(x[idx], w, b, heads)
+    bb = None if bias is None else bias.double().numpy()[idx] if kind == "windows" else bias.double().numpy()[None]
+    ref = oracle.nystra_attention(q, k, v, m, 5, lm, bb).reshape(-1, N, d)
+    for out in (one, fused):
+        err = per_unit_rel(out.cpu()[idx].double().numpy(), ref)
+        assert err.max() <= TOL[dtype], err.max()
+
+
+def test_what_was_refused_stays_refused():
+    x, w, b = (t.cuda() for t in workloads.random_x_wqkv(4, 256, 4, 32, "bf16", seed=1))
+    for kw in ({"m": 32}, {"m": 64}, {"m": 16, "iters": 13}, {"m": 8, "landmarks": "patches"}):
+        with pytest.raises(binding.NystraError):
+            binding.nystra_qkv(x, w, 4, **kw)
+    with pytest.raises(binding.NystraError):  # out over the tokens
+        binding.nystra_qkv(x, w, 4, 16, 6, out=x.view(4, 4, 256, 32))
+    big = torch.zeros(4 * 256 * 128 + 8, dtype=torch.bfloat16, device="cuda")
+    with pytest.raises(binding.NystraError):  # tokens not 16-byte aligned
+        binding.nystra_qkv(big[4:4 + 4 * 256 * 128].view(4, 256, 128), w, 4, 16, 6)
+    with pytest.raises(binding.NystraError):
+        binding.nystra_qkv(x.float(), w.float(), 4, 16, 6)
+    torch.cuda.synchronize()
+    assert binding.status() == binding.NYSTRA_OK
+
+
+def test_without_memory_and_under_capture(monkeypatch):
+    x, w, b = (t.cuda() for t in workloads.random_x_wqkv(6, 1024, 2, 32, "bf16", seed=2))
+    ref = binding.nystra_qkv(x, w, 2, 16, 6, b_qkv=b)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        out = binding.nystra_qkv(x, w, 2, 16, 6, b_qkv=b)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref)
+    monkeypatch.setattr(binding, "_qkv_two_pass", lambda *a: None)  # no memory: the fused kernel
+    out = binding.nystra_qkv(x, w, 2, 16, 6, b_qkv=b)
+    assert torch.equal(out, _fused(x, w, 2, 16, 6, b, None, "segments"))
