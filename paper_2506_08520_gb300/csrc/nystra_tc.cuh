@@ -442,12 +442,9 @@ __device__ __forceinline__ void gl_tile(const T* q0, const T* kbar, int d, int g
     float sl[NTL][4];
 #pragma unroll
     for (int j = 0; j < NTL; ++j) {
-        sl[j][0] = sl[j][1] = sl[j][2] = sl[j][3] = 0.f;
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-            const T* kr = kbar + (8 * j + g) * LS + 16 * kk + 2 * t;
-            O::mma(sl[j], a[kk], DSt<T>::ld(kr, LO), DSt<T>::ld(kr + 8, LO));
-        }
+        const T* kr = kbar + (8 * j + g) * LS + 2 * t;
+        O::mmaz(sl[j], a[0], DSt<T>::ld(kr, LO), DSt<T>::ld(kr + 8, LO));
+        O::mma(sl[j], a[1], DSt<T>::ld(kr + 16, LO), DSt<T>::ld(kr + 24, LO));
     }
     if constexpr (BIAS) {  // scores in the log2 domain, bias included: e0/e1 below take them as they are
 #pragma unroll
@@ -469,19 +466,21 @@ __device__ __forceinline__ void gl_tile(const T* q0, const T* kbar, int d, int g
     const float ssl = BIAS ? 1.f : sl2;
     mx0 = quad_max(mx0) * ssl;
     mx1 = quad_max(mx1) * ssl;
-    auto e0 = [&](float x) { return ex2(fmaf(x, ssl, -mx0)); };
-    auto e1 = [&](float x) { return ex2(fmaf(x, ssl, -mx1)); };
+    auto e = [&](float x, float y, float m) {
+        const float2 p = ex2_pair(x, y, ssl, m);
+        return O::dpk(p.x, p.y);
+    };
     if constexpr (M >= 16) {
 #pragma unroll
         for (int kk = 0; kk < KTL; ++kk) {
-            f[kk][0] = O::dpk(e0(sl[2 * kk][0]), e0(sl[2 * kk][1]));
-            f[kk][1] = O::dpk(e1(sl[2 * kk][2]), e1(sl[2 * kk][3]));
-            f[kk][2] = O::dpk(e0(sl[2 * kk + 1][0]), e0(sl[2 * kk + 1][1]));
-            f[kk][3] = O::dpk(e1(sl[2 * kk + 1][2]), e1(sl[2 * kk + 1][3]));
+            f[kk][0] = e(sl[2 * kk][0], sl[2 * kk][1], mx0);
+            f[kk][1] = e(sl[2 * kk][2], sl[2 * kk][3], mx1);
+            f[kk][2] = e(sl[2 * kk + 1][0], sl[2 * kk + 1][1], mx0);
+            f[kk][3] = e(sl[2 * kk + 1][2], sl[2 * kk + 1][3], mx1);
         }
     } else {
-        f[0][0] = O::dpk(e0(sl[0][0]), e0(sl[0][1]));
-        f[0][1] = O::dpk(e1(sl[0][2]), e1(sl[0][3]));
+        f[0][0] = e(sl[0][0], sl[0][1], mx0);
+        f[0][1] = e(sl[0][2], sl[0][3], mx1);
         f[0][2] = f[0][3] = O::dzero();
     }
 }
@@ -672,14 +671,14 @@ __device__ __forceinline__ void su_w_chunk(const typename Opnd<T>::DReg (&aq)[2]
     float s[8][4];
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-        s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
         const T* kr = Kc + ctok<RS>(nt, g) * d;
 #pragma unroll
         for (int kk = 0; kk < 2; ++kk) {
             const int c0 = 16 * kk + 2 * t, c1 = c0 + 8;
             const R b0 = c0 < d ? O::ld(kr + c0) : O::zero();
             const R b1 = c1 < d ? O::ld(kr + c1) : O::zero();
-            O::mma(s[nt], aq[kk], b0, b1);
+            if (kk == 0) O::mmaz(s[nt], aq[kk], b0, b1);
+            else O::mma(s[nt], aq[kk], b0, b1);
         }
     }
     if constexpr (BIAS) {  // scores in the log2 domain, bias included (rows beyond m stay unbiased)
@@ -699,32 +698,35 @@ __device__ __forceinline__ void su_w_chunk(const typename Opnd<T>::DReg (&aq)[2]
         }
     }
     const float ssl = BIAS ? 1.f : sl2;
-    float mx0 = run0, mx1 = run1;
+    float mx0 = fmaxf(s[0][0], s[0][1]), mx1 = fmaxf(s[0][2], s[0][3]);
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        mx0 = fmaxf(mx0, fmaxf(s[nt][0], s[nt][1]) * ssl);
-        mx1 = fmaxf(mx1, fmaxf(s[nt][2], s[nt][3]) * ssl);
+    for (int nt = 1; nt < 8; ++nt) {
+        mx0 = fmaxf(mx0, fmaxf(s[nt][0], s[nt][1]));
+        mx1 = fmaxf(mx1, fmaxf(s[nt][2], s[nt][3]));
     }
-    mx0 = quad_max(mx0);
-    mx1 = quad_max(mx1);
+    mx0 = fmaxf(run0, quad_max(mx0) * ssl);  // (ssl > 0; run0, run1 are the quad's)
+    mx1 = fmaxf(run1, quad_max(mx1) * ssl);
     if (rescale) {  // online rescaling of the accumulated rows
         const float f0 = ex2(run0 - mx0), f1 = ex2(run1 - mx1);
 #pragma unroll
         for (int j = 0; j < NTO; ++j) {
-            w[j][0] *= f0; w[j][1] *= f0; w[j][2] *= f1; w[j][3] *= f1;
+            mul_x2(w[j][0], w[j][1], f0);
+            mul_x2(w[j][2], w[j][3], f1);
         }
     }
     run0 = mx0;
     run1 = mx1;
-    auto e0 = [&](float x) { return ex2(fmaf(x, ssl, -mx0)); };
-    auto e1 = [&](float x) { return ex2(fmaf(x, ssl, -mx1)); };
+    auto e = [&](float x, float y, float m) {
+        const float2 p = ex2_pair(x, y, ssl, m);
+        return O::dpk(p.x, p.y);
+    };
 #pragma unroll
     for (int kt = 0; kt < 4; ++kt) {
         typename O::DReg a[4];
-        a[0] = v0 ? O::dpk(e0(s[2 * kt][0]), e0(s[2 * kt][1])) : O::dzero();
-        a[1] = v1 ? O::dpk(e1(s[2 * kt][2]), e1(s[2 * kt][3])) : O::dzero();
-        a[2] = v0 ? O::dpk(e0(s[2 * kt + 1][0]), e0(s[2 * kt + 1][1])) : O::dzero();
-        a[3] = v1 ? O::dpk(e1(s[2 * kt + 1][2]), e1(s[2 * kt + 1][3])) : O::dzero();
+        a[0] = v0 ? e(s[2 * kt][0], s[2 * kt][1], mx0) : O::dzero();
+        a[1] = v1 ? e(s[2 * kt][2], s[2 * kt][3], mx1) : O::dzero();
+        a[2] = v0 ? e(s[2 * kt + 1][0], s[2 * kt + 1][1], mx0) : O::dzero();
+        a[3] = v1 ? e(s[2 * kt + 1][2], s[2 * kt + 1][3], mx1) : O::dzero();
 #pragma unroll
         for (int j = 0; j < NTO; ++j) {
             const int c0 = 8 * j + 2 * t;
@@ -1509,16 +1511,20 @@ __device__ __forceinline__ void output_rows(const uint32_t* glf, const T* Qs, co
                                              BIAS ? bl + (size_t)(ch * 64 + mtok<RS>(tm, g)) * M : nullptr);
             }
             float o[NTO][4];
-#pragma unroll
-            for (int j = 0; j < NTO; ++j) o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
             if constexpr (M >= 16) {
 #pragma unroll
                 for (int kk = 0; kk < KTL; ++kk)
 #pragma unroll
-                    for (int j = 0; j < NTO; ++j) O::mma(o[j], f[kk], by[kk][j][0], by[kk][j][1]);
+                    for (int j = 0; j < NTO; ++j) {
+                        if (kk == 0) O::mmaz(o[j], f[kk], by[kk][j][0], by[kk][j][1]);
+                        else O::mma(o[j], f[kk], by[kk][j][0], by[kk][j][1]);
+                    }
             } else {
 #pragma unroll
-                for (int j = 0; j < NTO; ++j) O::mma8(o[j], f[0][0], f[0][1], by[0][j][0]);
+                for (int j = 0; j < NTO; ++j) {
+                    o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
+                    O::mma8(o[j], f[0][0], f[0][1], by[0][j][0]);
+                }
             }
             float d0 = 0.f, d1 = 0.f;
 #pragma unroll

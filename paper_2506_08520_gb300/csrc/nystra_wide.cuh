@@ -114,11 +114,10 @@ __device__ __forceinline__ void wide_output_tile(T* q0, const T* kbar, const T* 
     float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
     for (int j = 0; j < NTL; ++j) {
-        sl[j][0] = sl[j][1] = sl[j][2] = sl[j][3] = 0.f;
         D b[2][2];
         wide_b_k32<T>(kbar + 8 * j * LS, LS, LO, lane, b);
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) O::mma(sl[j], a[kk], b[kk][0], b[kk][1]);
+        O::mmaz(sl[j], a[0], b[0][0], b[0][1]);
+        O::mma(sl[j], a[1], b[1][0], b[1][1]);
     }
 #pragma unroll
     for (int j = 0; j < NTL; ++j) {

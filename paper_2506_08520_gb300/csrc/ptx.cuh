@@ -156,6 +156,12 @@ __device__ __forceinline__ void mul_x2(float& d0, float& d1, float b) {
         : "+f"(d0), "+f"(d1)
         : "f"(b));
 }
+// 2^(s x0 - m), 2^(s x1 - m).
+__device__ __forceinline__ float2 ex2_pair(float x0, float x1, float s, float m) {
+    float p0, p1;
+    fma_x2(p0, p1, x0, x1, s, s, -m, -m);
+    return make_float2(ex2(p0), ex2(p1));
+}
 // Transpose of an 8x8 matrix of 16-bit elements held one row pair per lane
 // (lane 4r + c holds row r, columns 2c and 2c+1).
 __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
@@ -343,7 +349,9 @@ struct Opnd {
     static __device__ __forceinline__ DReg dpk(float a, float b) {
         const uint32_t h = Op::pack(a, b);
         const float2 hf = Op::unpack(h);
-        return {h, Op::pack(a - hf.x, b - hf.y)};
+        float r0, r1;  // a - hf.x, b - hf.y
+        fma_x2(r0, r1, hf.x, hf.y, -1.f, -1.f, a, b);
+        return {h, Op::pack(r0, r1)};
     }
     static __device__ __forceinline__ DReg dzero() { return {0u, 0u}; }
     static __device__ __forceinline__ DReg dtr(DReg r) { return {movmatrix_trans(r.hi), movmatrix_trans(r.lo)}; }
@@ -364,6 +372,24 @@ struct Opnd {
         const uint32_t ah[4] = {a[0].hi, a[1].hi, a[2].hi, a[3].hi};
         const uint32_t al[4] = {a[0].lo, a[1].lo, a[2].lo, a[3].lo};
         Op::k16(c, al, b0.hi, b1.hi);
+        Op::k16(c, ah, b0.lo, b1.lo);
+        Op::k16(c, ah, b0.hi, b1.hi);
+    }
+    // the same products with c = instead of c +=
+    static __device__ __forceinline__ void mmaz(float (&c)[4], const Reg (&a)[4], DReg b0, DReg b1) {
+        Op::k16z(c, a, b0.lo, b1.lo);
+        Op::k16(c, a, b0.hi, b1.hi);
+    }
+    static __device__ __forceinline__ void mmaz(float (&c)[4], const DReg (&a)[4], Reg b0, Reg b1) {
+        const uint32_t ah[4] = {a[0].hi, a[1].hi, a[2].hi, a[3].hi};
+        const uint32_t al[4] = {a[0].lo, a[1].lo, a[2].lo, a[3].lo};
+        Op::k16z(c, al, b0, b1);
+        Op::k16(c, ah, b0, b1);
+    }
+    static __device__ __forceinline__ void mmaz(float (&c)[4], const DReg (&a)[4], DReg b0, DReg b1) {
+        const uint32_t ah[4] = {a[0].hi, a[1].hi, a[2].hi, a[3].hi};
+        const uint32_t al[4] = {a[0].lo, a[1].lo, a[2].lo, a[3].lo};
+        Op::k16z(c, al, b0.hi, b1.hi);
         Op::k16(c, ah, b0.lo, b1.lo);
         Op::k16(c, ah, b0.hi, b1.hi);
     }
@@ -435,6 +461,9 @@ struct Opnd<Single16<T>> {
     static __device__ __forceinline__ Reg one() { return Op::kOne; }
     static __device__ __forceinline__ void mma(float (&c)[4], const Reg (&a)[4], Reg b0, Reg b1) {
         Op::k16(c, a, b0, b1);
+    }
+    static __device__ __forceinline__ void mmaz(float (&c)[4], const Reg (&a)[4], Reg b0, Reg b1) {  // c = a b
+        Op::k16z(c, a, b0, b1);
     }
     static __device__ __forceinline__ void mma8(float (&c)[4], Reg a0, Reg a1, Reg b0) { Op::k8(c, a0, a1, b0); }
     static __device__ __forceinline__ void st2(Single16<T>* p, float a, float b) {
