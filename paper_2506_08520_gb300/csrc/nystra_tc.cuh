@@ -429,6 +429,14 @@ __device__ __forceinline__ void gl_tile(const T* q0, const T* kbar, int d, int g
     using O = Opnd<T>;
     using R = typename O::Reg;
     constexpr int NTL = M / 8, LS = LmS<T>::LS, LO = LmS<T>::LO;
+    float2 b0[BIAS ? NTL : 1], b1[BIAS ? NTL : 1];  // on their way from L2 during the products
+    if constexpr (BIAS) {
+#pragma unroll
+        for (int j = 0; j < NTL; ++j) {
+            b0[j] = __ldg(reinterpret_cast<const float2*>(bl + 8 * j + 2 * t));
+            b1[j] = __ldg(reinterpret_cast<const float2*>(bl + mrow<RS>() * M + 8 * j + 2 * t));
+        }
+    }
     R a[2][4];
     const T* q1 = q0 + mrow<RS>() * d;
 #pragma unroll
@@ -446,15 +454,13 @@ __device__ __forceinline__ void gl_tile(const T* q0, const T* kbar, int d, int g
         O::mmaz(sl[j], a[0], DSt<T>::ld(kr, LO), DSt<T>::ld(kr + 8, LO));
         O::mma(sl[j], a[1], DSt<T>::ld(kr + 16, LO), DSt<T>::ld(kr + 24, LO));
     }
-    if constexpr (BIAS) {  // scores in the log2 domain, bias included: e0/e1 below take them as they are
+    if constexpr (BIAS) {  // scores in the log2 domain, bias included: e below takes them as they are
 #pragma unroll
         for (int j = 0; j < NTL; ++j) {
-            const float2 b0 = __ldg(reinterpret_cast<const float2*>(bl + 8 * j + 2 * t));
-            const float2 b1 = __ldg(reinterpret_cast<const float2*>(bl + mrow<RS>() * M + 8 * j + 2 * t));
-            sl[j][0] = fmaf(sl[j][0], sl2, kLog2e * b0.x);
-            sl[j][1] = fmaf(sl[j][1], sl2, kLog2e * b0.y);
-            sl[j][2] = fmaf(sl[j][2], sl2, kLog2e * b1.x);
-            sl[j][3] = fmaf(sl[j][3], sl2, kLog2e * b1.y);
+            mul_x2(b0[j].x, b0[j].y, kLog2e);
+            mul_x2(b1[j].x, b1[j].y, kLog2e);
+            fma_x2(sl[j][0], sl[j][1], sl[j][0], sl[j][1], sl2, sl2, b0[j].x, b0[j].y);
+            fma_x2(sl[j][2], sl[j][3], sl[j][2], sl[j][3], sl2, sl2, b1[j].x, b1[j].y);
         }
     }
     float mx0 = -INFINITY, mx1 = -INFINITY;
@@ -668,6 +674,39 @@ __device__ __forceinline__ void su_w_chunk(const typename Opnd<T>::DReg (&aq)[2]
     using O = Opnd<T>;
     using R = typename O::Reg;
     constexpr int NTO = NCOL / 8;
+    // BIAS: the entries of keys 2t, 2t + 1 (in row order) of each n-tile, rows g
+    // and g + 8, on their way from L2 during the products.  In the RS = 4 order
+    // those of four n-tiles are eight consecutive keys: two 16-byte loads.  With 32
+    // 4-byte loads after the products instead, the bias cost 103 us on 21600
+    // units of 16x16 windows (421 against 318 us); so it costs 43 (360).
+    float2 b0[BIAS ? 8 : 1], b1[BIAS ? 8 : 1];
+    if constexpr (BIAS) {
+        auto load = [&](const float* p, bool real, float2(&b)[8]) {
+            if constexpr (RS == 4) {
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                    const float4 x = real ? __ldg(reinterpret_cast<const float4*>(p + 32 * q + 8 * t)) : z;
+                    const float4 y = real ? __ldg(reinterpret_cast<const float4*>(p + 32 * q + 8 * t + 4)) : z;
+                    b[4 * q] = make_float2(x.x, y.x);
+                    b[4 * q + 1] = make_float2(x.y, y.y);
+                    b[4 * q + 2] = make_float2(x.z, y.z);
+                    b[4 * q + 3] = make_float2(x.w, y.w);
+                }
+            } else {
+#pragma unroll
+                for (int nt = 0; nt < 8; ++nt) {
+                    if constexpr (RS == 1)
+                        b[nt] = real ? __ldg(reinterpret_cast<const float2*>(p + 8 * nt + 2 * t)) : make_float2(0.f, 0.f);
+                    else
+                        b[nt] = real ? make_float2(__ldg(p + ctok<RS>(nt, 2 * t)), __ldg(p + ctok<RS>(nt, 2 * t + 1)))
+                                     : make_float2(0.f, 0.f);
+                }
+            }
+        };
+        load(bu, v0, b0);
+        load(bu + 8 * bn, v1, b1);
+    }
     float s[8][4];
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
@@ -684,17 +723,10 @@ __device__ __forceinline__ void su_w_chunk(const typename Opnd<T>::DReg (&aq)[2]
     if constexpr (BIAS) {  // scores in the log2 domain, bias included (rows beyond m stay unbiased)
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
-            // keys of columns 2t, 2t + 1 of n-tile nt
-            auto ld2 = [&](const float* p) -> float2 {
-                if constexpr (RS == 1) return __ldg(reinterpret_cast<const float2*>(p + 8 * nt + 2 * t));
-                else return make_float2(__ldg(p + ctok<RS>(nt, 2 * t)), __ldg(p + ctok<RS>(nt, 2 * t + 1)));
-            };
-            const float2 b0 = v0 ? ld2(bu) : make_float2(0.f, 0.f);
-            const float2 b1 = v1 ? ld2(bu + 8 * bn) : make_float2(0.f, 0.f);
-            s[nt][0] = fmaf(s[nt][0], sl2, kLog2e * b0.x);
-            s[nt][1] = fmaf(s[nt][1], sl2, kLog2e * b0.y);
-            s[nt][2] = fmaf(s[nt][2], sl2, kLog2e * b1.x);
-            s[nt][3] = fmaf(s[nt][3], sl2, kLog2e * b1.y);
+            mul_x2(b0[nt].x, b0[nt].y, kLog2e);
+            mul_x2(b1[nt].x, b1[nt].y, kLog2e);
+            fma_x2(s[nt][0], s[nt][1], s[nt][0], s[nt][1], sl2, sl2, b0[nt].x, b0[nt].y);
+            fma_x2(s[nt][2], s[nt][3], s[nt][2], s[nt][3], sl2, sl2, b1[nt].x, b1[nt].y);
         }
     }
     const float ssl = BIAS ? 1.f : sl2;
