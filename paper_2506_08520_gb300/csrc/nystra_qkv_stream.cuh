@@ -109,7 +109,7 @@ __device__ __forceinline__ void project_chunk(const T* __restrict__ xr, const ui
 template <typename T, int M, int NCOL, int TPW>
 struct QsLayout {
     static constexpr int NT = 4, N = NT * TPW, CH = 64, NCHK = TPW / CH;  // token warps, chunks per warp
-    static constexpr int CWN = M > 16 ? M / 16 : 1;  // core warps (m = 32: distributed core)
+    static constexpr int CWN = M > 16 ? M / 16 : 1;  // core warps (m = 32: sc_core)
     static constexpr int MT = (M + 15) / 16, MP = MT * 16, WS = NCOL + 4;
     static constexpr int DS = (NCOL == 32) ? 30 : 32;
     static constexpr int L = N / M, LPW = TPW / L;  // tokens per segment, segments per token warp
@@ -125,7 +125,7 @@ struct QsLayout {
     static constexpr size_t B_YT = B_QB;
     static constexpr size_t BUF = ((B_KB + LmS<T>::bytes(MP) + 127) / 128) * 128;
     static_assert(YtS<T, M>::bytes(NCOL) <= B_KB, "Y^T must fit over Qbar, W and m_U");
-    static constexpr size_t SCR = CWN > 1 ? DistScratch<(M > 16 ? M : 32)>::BYTES : 0;
+    static constexpr size_t SCR = CWN > 1 ? ScScratch<(M > 16 ? M : 32)>::BYTES : 0;
     static constexpr size_t T_BUF = NT * SLOT;
     static constexpr size_t T_BAR = T_BUF + 2 * BUF;  // F[2], C[2]
     static constexpr size_t T_SCR = ((T_BAR + 4 * 8 + 127) / 128) * 128;
@@ -242,13 +242,15 @@ nystra_qkv_stream_kernel(const T* __restrict__ x, const T* __restrict__ wqkv, co
                                                    reinterpret_cast<T*>(bb + Lay::B_YT), iters, sl2, g, t, nullptr,
                                                    bAu);
             } else {
-                using DSc = DistScratch<(M > 16 ? M : 32)>;
+                using Sc = ScScratch<(M > 16 ? M : 32)>;
                 unsigned char* scr = tb + Lay::T_SCR;
-                dist_core<T, (M > 16 ? M : 32), NCOL>(
-                    reinterpret_cast<const T*>(bb + Lay::B_QB), reinterpret_cast<const T*>(bb + Lay::B_KB), gmu,
-                    reinterpret_cast<const float*>(bb + Lay::B_W), reinterpret_cast<T*>(bb + Lay::B_YT), scr,
-                    scr + DSc::MAT, reinterpret_cast<float*>(scr + 2 * DSc::MAT), iters, sl2, c, lane,
-                    1 + TEAMS + team);
+                float wr[NCOL / 8][4];
+                sc_load_w<NCOL>(reinterpret_cast<const float*>(bb + Lay::B_W), wr, c, g, t);
+                sc_core<T, (M > 16 ? M : 32), NCOL>(
+                    reinterpret_cast<const T*>(bb + Lay::B_QB), reinterpret_cast<const T*>(bb + Lay::B_KB),
+                    gmu[16 * c + g], gmu[16 * c + g + 8], wr, reinterpret_cast<T*>(bb + Lay::B_YT), scr,
+                    scr + Sc::MAT, scr + 2 * Sc::MAT, reinterpret_cast<float*>(scr + 2 * Sc::MAT + Sc::WMAT), iters,
+                    sl2, c, lane, 1 + TEAMS + team);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(barC + b);

@@ -1,5 +1,5 @@
 // Streaming team kernel for 32x32 windows (N = 1024 tokens), m <= 32, even
-// d_h <= 32, 16-bit I/O (m = 32: the core runs on two warps, dist_core).  Included by the N = 1024 translation unit after
+// d_h <= 32, 16-bit I/O (m = 32: the core runs on two warps, sc_core).  Included by the N = 1024 translation unit after
 // nystra_tc.cuh, whose per-phase device functions it reuses.
 //
 // A whole 32x32 unit (Q, K, V: 184 KB at d_h = 30) fills an SM, so staging
@@ -36,7 +36,7 @@ namespace tc {
 template <typename T, int M, int NCOL>
 struct StreamLayout {
     static constexpr int NT = 4, TPW = 256, N = NT * TPW, CH = 64, NCHK = TPW / CH;
-    static constexpr int CWN = M > 16 ? M / 16 : 1;  // core warps (m = 32: distributed core)
+    static constexpr int CWN = M > 16 ? M / 16 : 1;  // core warps (m = 32: sc_core)
     static constexpr int MT = (M + 15) / 16;         // landmark m-tiles
     static constexpr int DS = (NCOL == 32) ? 30 : 32;
     static constexpr int MP = MT * 16, LS = LmS<T>::LS, WS = NCOL + 4;
@@ -56,7 +56,7 @@ struct StreamLayout {
     static constexpr size_t B_YT = B_QB;
     static constexpr size_t BUF = ((B_KB + LmS<T>::bytes(MP) + 127) / 128) * 128;
     static_assert(YtS<T, M>::bytes(NCOL) <= B_KB, "Y^T must fit over Qbar, W and m_U");
-    static constexpr size_t SCR = CWN > 1 ? DistScratch<(M > 16 ? M : 32)>::BYTES : 0;
+    static constexpr size_t SCR = CWN > 1 ? ScScratch<(M > 16 ? M : 32)>::BYTES : 0;
     template <int S>
     struct Team {
         static constexpr size_t WARP = S * SLOT;  // a token warp's ring of chunk buffers
@@ -84,7 +84,7 @@ struct StreamLayout {
 // then for k >= 1 Q(k), OUT(k - 1), KV(k), finally OUT(count - 1): a unit's Q
 // rows are read again two blocks after their first read, while they are
 // still in L2, and the core of unit k runs during Q(k + 1).  Otherwise (the
-// slower distributed core of m = 32): Q(k), KV(k), OUT(k - 1) for each k,
+// slower core of m = 32): Q(k), KV(k), OUT(k - 1) for each k,
 // finally OUT(count - 1), so the core has two blocks to finish.
 struct StreamTask {
     int k, type, c;  // unit (team-local), 0 = Q, 1 = KV, 2 = OUT, chunk
@@ -189,13 +189,15 @@ nystra_stream_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
                                                    reinterpret_cast<T*>(bb + Lay::B_YT), iters, sl2, g, t, nullptr,
                                                    bAu);
             } else {
-                using DSc = DistScratch<(M > 16 ? M : 32)>;
+                using Sc = ScScratch<(M > 16 ? M : 32)>;
                 unsigned char* scr = tb + TL::T_SCR;
-                dist_core<T, (M > 16 ? M : 32), NCOL>(
-                    reinterpret_cast<const T*>(bb + Lay::B_QB), reinterpret_cast<const T*>(bb + Lay::B_KB), gmu,
-                    reinterpret_cast<const float*>(bb + Lay::B_W), reinterpret_cast<T*>(bb + Lay::B_YT), scr,
-                    scr + DSc::MAT, reinterpret_cast<float*>(scr + 2 * DSc::MAT), iters, sl2, c, lane,
-                    1 + Lay::TEAMS + team);
+                float wr[NCOL / 8][4];
+                sc_load_w<NCOL>(reinterpret_cast<const float*>(bb + Lay::B_W), wr, c, g, t);
+                sc_core<T, (M > 16 ? M : 32), NCOL>(
+                    reinterpret_cast<const T*>(bb + Lay::B_QB), reinterpret_cast<const T*>(bb + Lay::B_KB),
+                    gmu[16 * c + g], gmu[16 * c + g + 8], wr, reinterpret_cast<T*>(bb + Lay::B_YT), scr,
+                    scr + Sc::MAT, scr + 2 * Sc::MAT, reinterpret_cast<float*>(scr + 2 * Sc::MAT + Sc::WMAT), iters,
+                    sl2, c, lane, 1 + Lay::TEAMS + team);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(barC + b);

@@ -1,5 +1,5 @@
-// The m x m core of m = 64 on CW = m/16 = 4 warps, with symmetric products.
-// Included by nystra_tc.cuh after the other cores, whose fragment helpers it
+// The m x m core of m = 32 and 64 on CW = m/16 warps, with symmetric products.
+// Included by nystra_tc.cuh after the one-warp core, whose fragment helpers it
 // uses.
 #pragma once
 
@@ -8,18 +8,21 @@
 namespace nystra {
 namespace tc {
 
-// Warp c owns rows 16c..16c+15.  The arithmetic is dist_core's: X = A Z_k and
-// Z are carried, T2 = 15I - 7X + XX, T3 = 13I - X T2, Z <- Z T3/4, X <- X T3/4.
-// T2, T3 and X are polynomials in X_0 = a A A^T and symmetric: of a warp's
-// 2 CW tiles of 16 x 8 in each of their products only one triangle's CW + 1 are
-// computed, and mirrored, which also removes antisymmetric round-off (23 tile
-// products per warp and step instead of 32).  Z's own rows stay in registers
-// at a power of two per warp, so no step needs a maximum over the warps.
+// The m x m operands no longer fit one warp's registers: warp c owns rows 16c ..
+// 16c + 15.  The arithmetic is core_warp's: X = A Z_k and Z are carried, T2 = 15I -
+// 7X + XX, T3 = 13I - X T2, Z <- Z T3/4, X <- X T3/4.  T2, T3 and X are
+// polynomials in X_0 = a A A^T and symmetric: of a warp's 2 CW tiles of 16 x 8 in
+// each of their products only one triangle's CW + 1 are computed, and mirrored,
+// which also removes antisymmetric round-off (m = 64: 23 tile products per warp
+// and step instead of 32; m = 32: 13 instead of 16).  Z's own rows stay in
+// registers at a power of two per warp, so no step needs a maximum over the
+// warps.
 //
-// A warp computes its diagonal block (two tiles), the block to its right,
-// cyclically (two tiles), and one tile of the blocks two apart, whose left
-// rows it keeps as a second A operand.  X's k-blocks and Z's tiles are taken
-// in the cyclic order of those columns, so that register indexes are constant.
+// A warp computes its diagonal block (two tiles), m = 64: the block to its right,
+// cyclically (two tiles), and one tile of the blocks two apart (m = 32: of the
+// only off-diagonal block), whose left rows it keeps as a second A operand.  X's
+// k-blocks and Z's tiles are taken in the cyclic order of those columns, so that
+// register indexes are constant.
 //
 // Right factors are read from two shared-memory matrices (hi and lo planes,
 // rows padded to m + 8 halves so ldmatrix is conflict-free) that alternate
@@ -30,13 +33,16 @@ namespace tc {
 // of any scale) that puts its largest entry in [2^10, 2^11).
 //
 // What bounds it: the tensor pipe's mma.sync rate and, between two barriers,
-// a chain of 12 dependent MMAs with the split and store of their results.
-// Measured in the wide kernel (4096 units of 16x16 windows, d_h = 32, bf16):
-// 0.93 ms with full products and two groups per SM -> 0.50 ms; in the grouped
-// kernel (1024 units of 32x32 windows) 0.50 -> 0.40 ms.  Carrying V = Z W
+// a chain of 6 or 12 dependent MMAs with the split and store of their results.
+// Measured (bf16) against full products and scales agreed on over the warps:
+// m = 64, 4096 units of 16x16 windows, d_h = 32, 0.93 -> 0.50 ms (in the wide
+// kernel, with three groups per SM instead of two), 1024 of 32x32 0.50 -> 0.37;
+// m = 32, 8192 units of 16x16, d_h = 30, 353 -> 290 us (d_h = 32 now in the team
+// kernel too: 557 -> 345); 1024 units of 32x32, d_h = 32, not bound by the core,
+// 144 us as before.  At m = 64, carrying V = Z W
 // instead (V <- T3 V/4 with X = Z A: d_h + 1 columns instead of m, 20 tile
-// products a step, but V's column scales to agree on in every step) took 0.51
-// and 0.46 ms, and was less accurate: under sharp attention (logit std 4) its
+// products a step, but V's column scales to agree on in every step) took 0.51 and
+// 0.46 ms, and was less accurate: under sharp attention (logit std 4) its
 // error was up to twice as large, since Z T3 meets W's small parts exactly.
 
 template <int M>
@@ -61,12 +67,12 @@ __device__ __forceinline__ void sc_put(unsigned char* mat, const float (&acc)[M 
 template <int M>
 struct ScTiles {
     static constexpr int CW = M / 16, N = CW + 1, OWN = N - 1;
-    static_assert(CW == 4, "the cyclic split is that of four row blocks");
+    static_assert(CW == 4 || CW == 2, "the splits are those of four and two row blocks");
     int c, r5, b5, h5;  // own block; the last tile's row block, column block and half
     __device__ __forceinline__ explicit ScTiles(int c_) : c(c_) {
-        r5 = c & 1;
-        b5 = r5 + 2;
-        h5 = c >> 1;
+        r5 = CW == 4 ? (c & 1) : 0;
+        b5 = CW == 4 ? r5 + 2 : 1;
+        h5 = CW == 4 ? (c >> 1) : c;
     }
     __device__ __forceinline__ int row(int i) const { return i < OWN ? c : r5; }
     __device__ __forceinline__ int col(int i) const { return i < OWN ? 2 * ((c + i / 2) % CW) + (i & 1) : 2 * b5 + h5; }
@@ -546,8 +552,8 @@ __device__ __forceinline__ T* sc_core(const T* qbar, const T* kbar, float mu0, f
     }
     // free: after the last step -T2/4's matrix (its readers have passed a
     // barrier since), without steps A's
-    if (!yT) yT = reinterpret_cast<T*>(oth);
-    static_assert(YtS<T, M>::bytes(NCOL) <= S::MAT, "Y^T must fit over a scratch matrix");
+    if constexpr (YtS<T, M>::bytes(NCOL) <= S::MAT)  // (m = 32: the caller has a place)
+        if (!yT) yT = reinterpret_cast<T*>(oth);
 #pragma unroll
     for (int j = 0; j < NTO; ++j) {
         const int rr = 16 * c + g, cc = 8 * j + 2 * t;

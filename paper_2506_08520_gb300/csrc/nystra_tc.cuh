@@ -24,16 +24,15 @@
 //   core     G_A^n = exp(Qbar Kbar^T - m_U), Z_0 = A^T/(||A||_1 ||A||_inf),
 //            `iters` steps Z <- Z(13I - X(15I - X(7I - X)))/4 with X = A Z
 //            (step 4), Y = Z W stored as a 16-bit B operand: core_warp (one
-//            warp, in registers, m <= 16), dist_core (m = 32, two warps) or
-//            sc_core (m = 64, four warps; nystra_symcore.cuh).
+//            warp, in registers; m = 32 at 8x8 windows too) or sc_core (m/16
+//            warps, m = 32 and 64; nystra_symcore.cuh).
 //   output   O = (G_L^n Y_:d) / (G_L^n Y_d) (steps 5-7), staged row-major and
 //            written with one bulk store (rows of 60 bytes would otherwise be
 //            written as partial sectors); [P2] S_L and G_L^n recomputed from
 //            a still-resident Q.
 //
-// Grouped kernel (nystra_tc_kernel; m = 32 at 8x8 windows and, with d_h = 32,
-// at 16x16; m = 64 at 32x32).  A group of token warps owns one unit at a time, plus
-// helper warps when the distributed core needs more warps than there are
+// Grouped kernel (nystra_tc_kernel; m = 32 at 8x8 windows, m = 64 at 32x32).  A group of token warps owns one unit at a time, plus
+// helper warps when the core needs more warps than there are
 // token warps; a CTA holds GROUPS groups and the grid is persistent.  The
 // next unit's Q and K are copied after the combine ([P2]: K only, Q after the
 // output), V once the output store has read its staging.  P1 ("G_L parked")
@@ -97,22 +96,10 @@ __host__ __device__ constexpr int mrow() {
 }
 static_assert(row_step(30) == 4 && row_step(28) == 2 && row_step(32) == 1 && row_step(0) == 1, "row steps");
 
-// Shared scratch of the distributed core (m = 32; see dist_core): two
-// matrices of fp16 pairs (hi plane, then lo plane; rows padded to m + 8
-// halves so ldmatrix is conflict-free) and an auxiliary float area.
-template <int M>
-struct DistScratch {
-    static constexpr int CW = M / 16, SS = M + 8;
-    static constexpr size_t PLANE = (size_t)M * SS * 2;
-    static constexpr size_t MAT = 2 * PLANE;
-    static constexpr size_t AUX = ((size_t)CW * M * 4 + 4 * CW * 4 + 15) / 16 * 16;  // column sums, maxima
-    static constexpr size_t BYTES = ((2 * MAT + AUX + 127) / 128) * 128;
-};
-
 // Shared scratch of the core with symmetric products (nystra_symcore.cuh): two
-// matrices of fp16 pairs (hi plane, then lo plane; rows
-// padded to m + 8 halves so ldmatrix is conflict-free), W (m rows of 40
-// columns, likewise) and an auxiliary float area.
+// matrices of fp16 pairs (hi plane, then lo plane; rows padded to m + 8 halves
+// so ldmatrix is conflict-free), W (m rows of 40 columns, likewise) and an
+// auxiliary float area.
 template <int M>
 struct ScScratch {
     static constexpr int CW = M / 16, SS = M + 8, WS = 40;
@@ -150,42 +137,31 @@ struct Layout {
     static constexpr size_t WPART = (size_t)TPW * DS * 2;
     static_assert(WPU == 1 || (size_t)MP * WS * 4 + MP * 4 <= 2 * (size_t)TPW * DS * 2,
                   "W partial must fit in K+V");
-    // Distributed core (CW > 1): its scratch is group memory, or, with long
-    // stages (TPW >= 256), the first two token warps' K/V rows (consumed by
-    // the combine before the core starts; the next unit's K and V are copied
-    // after the core).
-    static constexpr bool SCR_IN_STAGE = M == 64;
-    static constexpr bool SCR_IN_GROUP = (CW > 1) && !SCR_IN_STAGE;
-    static constexpr size_t SCR_BYTES = SCR_IN_GROUP ? DistScratch<(M > 16 ? M : 32)>::BYTES : 0;
-    static_assert(!SCR_IN_STAGE || (WPU >= 2 && CW == 4 &&
-                                    ScScratch<64>::MAT + ScScratch<64>::WMAT <= 2 * (size_t)TPW * DS * 2),
+    // The core on several warps (CW > 1, m = 64) has its scratch in the first two
+    // token warps' K/V rows (consumed by the combine before the core starts; the
+    // next unit's K and V are copied after the core).
+    static_assert(CW == 1 || (M == 64 && CW == 4 && WPU >= 2 &&
+                              ScScratch<64>::MAT + ScScratch<64>::WMAT <= 2 * (size_t)TPW * DS * 2),
                   "scratch must fit in two warps' K/V rows");
     static constexpr size_t QB_BYTES = LmS<T>::bytes(MP);
     static constexpr size_t YT_BYTES = YtS<T, M>::bytes(NCOL);
-    // Per-group shared memory.  Y^T is written by the core once it has read
-    // Qbar, W and m_U for the last time, so it overlays them when no warp can
-    // write the next unit's landmarks or W while another still reads Y^T:
-    // with one warp per unit, or when G_L^n is recomputed (the output is
-    // followed by a group barrier before the next unit's Q lands); with the
-    // distributed core, whose scratch starts after every core warp has read
-    // its Qbar rows, the scratch overlays Qbar and Y^T overlays W and m_U.
-    //   one-warp core:     Qbar | W | m_U | Kbar (| Y^T) | bars
-    //   distributed core:  W | m_U | Kbar | bars | Qbar (inside the scratch)
-    static constexpr bool YT_OVERLAY = SCR_IN_GROUP || (WPU == 1) || !GLS;
-    static constexpr size_t G_W = SCR_IN_GROUP ? 0 : QB_BYTES;  // fp32 MP x WS
-    static constexpr size_t G_MU = G_W + MP * WS * 4;           // m_U, log2 domain
+    // Per-group shared memory: Qbar | W | m_U | Kbar (| Y^T) | bars.  Y^T is
+    // written by the core once every core warp has read Qbar, W and m_U for the
+    // last time, so it overlays them when no warp can write the next unit's
+    // landmarks or W while another still reads Y^T: with one warp per unit, or
+    // when G_L^n is recomputed (the output is followed by a group barrier before
+    // the next unit's Q lands).
+    static constexpr bool YT_OVERLAY = (WPU == 1) || !GLS;
+    static constexpr size_t G_QBAR = 0;
+    static constexpr size_t G_W = QB_BYTES;            // fp32 MP x WS
+    static constexpr size_t G_MU = G_W + MP * WS * 4;  // m_U, log2 domain
     static constexpr size_t G_KBAR = ((G_MU + MP * 4 + 15) / 16) * 16;
-    static constexpr size_t G_BAR = SCR_IN_GROUP ? ((G_KBAR + QB_BYTES + 15) / 16) * 16
-                                                 : (((YT_OVERLAY ? G_KBAR + QB_BYTES : G_KBAR + QB_BYTES + YT_BYTES) +
-                                                     15) / 16) * 16;
+    static constexpr size_t G_BAR =
+        (((YT_OVERLAY ? G_KBAR + QB_BYTES : G_KBAR + QB_BYTES + YT_BYTES) + 15) / 16) * 16;
     static constexpr size_t G_BAR_END = G_BAR + 16 * WPU;  // two mbarriers per token warp
-    static constexpr size_t G_QBAR = SCR_IN_GROUP ? ((G_BAR_END + 16 + 127) / 128) * 128 : 0;
-    static constexpr size_t G_YT = SCR_IN_GROUP ? G_W : (YT_OVERLAY ? G_QBAR : G_KBAR + QB_BYTES);
-    static_assert(!YT_OVERLAY || YT_BYTES <= (SCR_IN_GROUP ? G_KBAR : G_KBAR - G_QBAR),
-                  "Y^T must fit over the regions it overlays");
-    static constexpr size_t G_SCR = SCR_IN_GROUP ? G_QBAR : ((G_BAR_END + 16 + 127) / 128) * 128;
-    static constexpr size_t GROUP_BYTES =
-        ((SCR_IN_GROUP ? G_QBAR + (SCR_BYTES > QB_BYTES ? SCR_BYTES : QB_BYTES) : G_SCR) + 127) / 128 * 128;
+    static constexpr size_t G_YT = YT_OVERLAY ? G_QBAR : G_KBAR + QB_BYTES;
+    static_assert(!YT_OVERLAY || YT_BYTES <= G_KBAR - G_QBAR, "Y^T must fit over the regions it overlays");
+    static constexpr size_t GROUP_BYTES = ((G_BAR_END + 16 + 127) / 128) * 128;
     static constexpr size_t PER_GROUP = GROUP_BYTES + WPU * WARP_BYTES;
 };
 
@@ -1121,383 +1097,6 @@ __device__ __forceinline__ void core_warp(const T* qbar, const T* kbar, const fl
     }
 }
 
-// ---- distributed core for m = 32: CW = m/16 warps, warp c owns rows 16c..16c+15 ----
-// The m x m operands no longer fit one warp's registers.  Each warp keeps the
-// A operands of its own rows (X and Z, fp16 pairs) and reads right-hand
-// factors from two shared-memory matrices (hi and lo planes, rows padded to
-// m + 8 halves so ldmatrix is conflict-free) that alternate roles: X in one,
-// -T2/4 in the other, T3/4 over X once every warp has used X, the next X over
-// -T2/4 once every warp has used it; three barriers per step.
-
-template <int M>
-__device__ __forceinline__ void dist_store(unsigned char* mat, int row, int col, const H2Pair& p) {
-    constexpr int SS = DistScratch<M>::SS;
-    *reinterpret_cast<uint32_t*>(mat + ((size_t)row * SS + col) * 2) = p.hi;
-    *reinterpret_cast<uint32_t*>(mat + DistScratch<M>::PLANE + ((size_t)row * SS + col) * 2) = p.lo;
-}
-
-// Own rows of s*acc into a scratch matrix.
-template <int M>
-__device__ __forceinline__ void dist_put(unsigned char* mat, const float (&acc)[M / 8][4], float s, int c, int g,
-                                         int t) {
-#pragma unroll
-    for (int n = 0; n < M / 8; ++n) {
-        dist_store<M>(mat, 16 * c + g, 8 * n + 2 * t, split_h2(s * acc[n][0], s * acc[n][1]));
-        dist_store<M>(mat, 16 * c + g + 8, 8 * n + 2 * t, split_h2(s * acc[n][2], s * acc[n][3]));
-    }
-}
-
-// The symmetric matrix defined by the lower triangle of s*acc: own blocks on
-// and below the diagonal (diagonal blocks mirrored) and their transposes.
-template <int M>
-__device__ __forceinline__ void dist_put_sym(unsigned char* mat, const float (&acc)[M / 8][4], float s, int c,
-                                             int g, int t, uint32_t sel) {
-#pragma unroll
-    for (int n = 0; n < M / 8; ++n)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int R = 2 * c + h;
-            if (R < n) continue;  // warp-uniform
-            H2Pair p = split_h2(s * acc[n][2 * h], s * acc[n][2 * h + 1]);
-            if (R == n) {
-                p.hi = prmt(p.hi, movmatrix_trans(p.hi), sel);
-                p.lo = prmt(p.lo, movmatrix_trans(p.lo), sel);
-                dist_store<M>(mat, 8 * R + g, 8 * n + 2 * t, p);
-            } else {
-                dist_store<M>(mat, 8 * R + g, 8 * n + 2 * t, p);
-                dist_store<M>(mat, 8 * n + g, 8 * R + 2 * t,
-                              H2Pair{movmatrix_trans(p.hi), movmatrix_trans(p.lo)});
-            }
-        }
-}
-
-// A operand of the own rows (tr: of the transpose's own rows) from a scratch matrix.
-template <int M, bool TR>
-__device__ __forceinline__ void dist_load_a(const unsigned char* mat, H2Pair (&a)[M / 16][4], int c, int lane) {
-    constexpr int SS = DistScratch<M>::SS;
-    const int blk = lane >> 3, rr = lane & 7;
-#pragma unroll
-    for (int kk = 0; kk < M / 16; ++kk) {
-        int row, col;
-        if (TR) {
-            row = 16 * kk + 8 * (blk >> 1) + rr;
-            col = 16 * c + 8 * (blk & 1);
-        } else {
-            row = 16 * c + 8 * (blk & 1) + rr;
-            col = 16 * kk + 8 * (blk >> 1);
-        }
-        uint32_t h[4], l[4];
-        const unsigned char* ph = mat + ((size_t)row * SS + col) * 2;
-        if (TR) {
-            ldsm_x4_t(h, ph);
-            ldsm_x4_t(l, ph + DistScratch<M>::PLANE);
-        } else {
-            ldsm_x4(h, ph);
-            ldsm_x4(l, ph + DistScratch<M>::PLANE);
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) a[kk][r] = H2Pair{h[r], l[r]};
-    }
-}
-
-// acc[a] = s I + A_a P^T over the own rows for NA left operands sharing the
-// right factor P (all m rows, from scratch); with CI also adds (-7I) P^T,
-// whose own-row block lies in k-step c (i7: its diagonal A register).
-template <int M, int NA, bool CI>
-__device__ __forceinline__ void dist_mm(const H2Pair (*const (&A)[NA])[4], const unsigned char* mat,
-                                        float (*const (&acc)[NA])[4], float s, uint32_t i7, int c, int g, int t,
-                                        int lane) {
-    using H = Mma16<__half>;
-    constexpr int SS = DistScratch<M>::SS, NT = M / 8;
-#pragma unroll
-    for (int a = 0; a < NA; ++a)
-#pragma unroll
-        for (int n = 0; n < NT; ++n)
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                acc[a][n][e] = ((16 * c + 8 * (e >> 1) + g) == (8 * n + (e & 1) + 2 * t)) ? s : 0.f;
-    const int blk = lane >> 3, rr = lane & 7;
-#pragma unroll
-    for (int kk = 0; kk < M / 16; ++kk)
-#pragma unroll
-        for (int jp = 0; jp < NT / 2; ++jp) {
-            uint32_t bh[4], bl[4];
-            const unsigned char* ph = mat + ((size_t)(16 * jp + 8 * (blk >> 1) + rr) * SS + 16 * kk + 8 * (blk & 1)) * 2;
-            ldsm_x4(bh, ph);
-            ldsm_x4(bl, ph + DistScratch<M>::PLANE);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int n = 2 * jp + h;
-#pragma unroll
-                for (int a = 0; a < NA; ++a) {
-                    const H2Pair* Ak = A[a][kk];
-                    const uint32_t ahi[4] = {Ak[0].hi, Ak[1].hi, Ak[2].hi, Ak[3].hi};
-                    const uint32_t alo[4] = {Ak[0].lo, Ak[1].lo, Ak[2].lo, Ak[3].lo};
-                    H::k16(acc[a][n], alo, bh[2 * h], bh[2 * h + 1]);
-                    H::k16(acc[a][n], ahi, bl[2 * h], bl[2 * h + 1]);
-                    H::k16(acc[a][n], ahi, bh[2 * h], bh[2 * h + 1]);
-                }
-                if (CI && kk == c) {
-                    const uint32_t ci[4] = {i7, 0u, 0u, i7};
-                    H::k16(acc[0][n], ci, bl[2 * h], bl[2 * h + 1]);
-                    H::k16(acc[0][n], ci, bh[2 * h], bh[2 * h + 1]);
-                }
-            }
-        }
-}
-
-// Core on CW = M/16 warps (warp c of them calls with its index; bar_id is a
-// named barrier reserved for these warps; mat0, mat1, aux: DistScratch
-// areas): G_A^n from the landmarks and m_U (gmu, log2 domain), the iteration
-// of step 4, Y = Z W (W: fp32, row stride NCOL + 4 at mW) stored as Y^T at
-// yT.  Same arithmetic as core_warp, except that X, -T2/4 and T3/4 are split
-// at the fixed scale 2^10 (their entries stay within a few units, since X's
-// eigenvalues lie in [0, 1]), which saves a barrier per scale; A is split at
-// 2^ea with its largest entry in [2^10, 2^11), Z renormalised every step.
-template <typename T, int M, int NCOL>
-__device__ __forceinline__ void dist_core(const T* qbar, const T* kbar, const float* gmu, const float* mW, T* yT,
-                                          unsigned char* mat0, unsigned char* mat1, float* aux, int iters, float sl2,
-                                          int c, int lane, int bar_id) {
-    using S = DistScratch<M>;
-    using O = Opnd<T>;
-    using D = typename O::DReg;
-    constexpr int CW = S::CW, KT = M / 16, NT = M / 8, LS = LmS<T>::LS, LO = LmS<T>::LO, WS = NCOL + 4,
-                  NTO = NCOL / 8, YS = YtS<T, M>::YS, YLO = YtS<T, M>::LO;
-    const int g = lane >> 2, t = lane & 3;
-    unsigned char* cur = mat0;
-    unsigned char* oth = mat1;
-    float* cols = aux;                // [CW][M] column-sum partials
-    float* slots = aux + CW * M;      // [4][CW] maxima
-    auto csync = [&]() { named_barrier(bar_id, CW * 32); };
-    const uint32_t sel = tril_selector(g, t);
-    constexpr float kS = 1024.f, kS2 = 1048576.f;  // fixed scale 2^10 of X, -T2/4, T3/4 (and its square)
-    uint32_t i7;  // A operand register of -7 kS I's diagonal blocks
-    {
-        const __half2 h = __floats2half2_rn(g == 2 * t ? -7.f * kS : 0.f, g == 2 * t + 1 ? -7.f * kS : 0.f);
-        i7 = *reinterpret_cast<const uint32_t*>(&h);
-    }
-    H2Pair Xa[KT][4], Za[KT][4];
-    float acc[NT][4], zc[NT][4];
-    // ---- G_A^n, own rows ----
-    {
-        D aq[2][4];
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-            const T* r0 = qbar + (16 * c + g) * LS + 16 * kk + 2 * t;
-            aq[kk][0] = DSt<T>::ld(r0, LO);
-            aq[kk][1] = DSt<T>::ld(r0 + 8 * LS, LO);
-            aq[kk][2] = DSt<T>::ld(r0 + 8, LO);
-            aq[kk][3] = DSt<T>::ld(r0 + 8 * LS + 8, LO);
-        }
-        const float mu0 = gmu[16 * c + g], mu1 = gmu[16 * c + g + 8];
-#pragma unroll
-        for (int n = 0; n < NT; ++n) {
-            float sa[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int kk = 0; kk < 2; ++kk) {
-                const T* kr = kbar + (8 * n + g) * LS + 16 * kk + 2 * t;
-                O::mma(sa, aq[kk], DSt<T>::ld(kr, LO), DSt<T>::ld(kr + 8, LO));
-            }
-            acc[n][0] = fmaf(sa[0], sl2, -mu0);  // log2 of G_A^n
-            acc[n][1] = fmaf(sa[1], sl2, -mu0);
-            acc[n][2] = fmaf(sa[2], sl2, -mu1);
-            acc[n][3] = fmaf(sa[3], sl2, -mu1);
-        }
-    }
-    // 2^ea G_A^n with its largest entry in [2^10, 2^11) (the shift enters the
-    // exponent, as in core_warp)
-    {
-        float lm = -INFINITY;
-#pragma unroll
-        for (int n = 0; n < NT; ++n)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) lm = fmaxf(lm, acc[n][e]);
-        lm = warp_max_f(lm);
-        if (lane == 0) slots[3 * CW + c] = lm;
-        csync();
-        float lmax = -INFINITY;
-#pragma unroll
-        for (int w = 0; w < CW; ++w) lmax = fmaxf(lmax, slots[3 * CW + w]);
-        const float fa = (lmax > -INFINITY && lmax < INFINITY) ? (float)(10 - (int)floorf(lmax)) : 0.f;
-#pragma unroll
-        for (int n = 0; n < NT; ++n)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[n][e] = ex2(acc[n][e] + fa);
-    }
-    // ---- ||A||_inf, ||A||_1 (A > 0) and A into scratch ----
-    {
-        float r0 = 0.f, r1 = 0.f;
-#pragma unroll
-        for (int n = 0; n < NT; ++n) {
-            r0 += acc[n][0] + acc[n][1];
-            r1 += acc[n][2] + acc[n][3];
-        }
-        r0 += __shfl_xor_sync(0xffffffffu, r0, 1);
-        r0 += __shfl_xor_sync(0xffffffffu, r0, 2);
-        r1 += __shfl_xor_sync(0xffffffffu, r1, 1);
-        r1 += __shfl_xor_sync(0xffffffffu, r1, 2);
-        const float rm = warp_max_nonneg(fmaxf(r0, r1));
-        if (lane == 0) slots[c] = rm;
-#pragma unroll
-        for (int n = 0; n < NT; ++n)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                float cs = acc[n][e] + acc[n][e + 2];
-                cs += __shfl_xor_sync(0xffffffffu, cs, 4);
-                cs += __shfl_xor_sync(0xffffffffu, cs, 8);
-                cs += __shfl_xor_sync(0xffffffffu, cs, 16);
-                if (g == 0) cols[c * M + 8 * n + 2 * t + e] = cs;
-            }
-    }
-    dist_put<M>(cur, acc, 1.f, c, g, t);  // 2^ea A
-    csync();
-    float alpha;  // a A A^T = alpha (2^ea A)(2^ea A)^T
-    {
-        float rmax = 0.f, cmax = 0.f;
-#pragma unroll
-        for (int w = 0; w < CW; ++w) rmax = fmaxf(rmax, slots[w]);
-        for (int col = lane; col < M; col += 32) {
-            float cs = 0.f;
-#pragma unroll
-            for (int w = 0; w < CW; ++w) cs += cols[w * M + col];
-            cmax = fmaxf(cmax, cs);
-        }
-        alpha = 1.f / (rmax * warp_max_nonneg(cmax));
-    }
-    {
-        H2Pair Aa[KT][4];
-#pragma unroll
-        for (int kk = 0; kk < KT; ++kk)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int n = 2 * kk + (r >> 1), e = 2 * (r & 1);
-                Aa[kk][r] = split_h2(acc[n][e], acc[n][e + 1]);
-            }
-        const H2Pair(*const As[1])[4] = {Aa};
-        float(*const Ds[1])[4] = {acc};
-        dist_mm<M, 1, false>(As, cur, Ds, 0.f, 0u, c, g, t, lane);  // (2^ea A)(2^ea A)^T
-    }
-    dist_load_a<M, true>(cur, Za, c, lane);  // Z_0 = (2^ea A)^T (a and 2^ea dropped)
-    dist_put_sym<M>(oth, acc, kS * alpha, c, g, t, sel);  // kS X_0
-    csync();
-    dist_load_a<M, false>(oth, Xa, c, lane);
-    {
-        unsigned char* tmp = cur;
-        cur = oth;
-        oth = tmp;
-    }
-    if (iters == 0) {
-#pragma unroll
-        for (int kk = 0; kk < KT; ++kk)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const uint32_t hb = Za[kk][r].hi, lb = Za[kk][r].lo;
-                const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&hb));
-                const float2 l = __half22float2(*reinterpret_cast<const __half2*>(&lb));
-                const int n = 2 * kk + (r >> 1), e = 2 * (r & 1);
-                zc[n][e] = h.x + l.x;
-                zc[n][e + 1] = h.y + l.y;
-            }
-    }
-    // ---- iteration (step 4): X in cur ----
-#pragma unroll 1
-    for (int it = 0; it < iters; ++it) {
-        {
-            const H2Pair(*const As[1])[4] = {Xa};
-            float(*const Ds[1])[4] = {acc};
-            dist_mm<M, 1, true>(As, cur, Ds, 15.f * kS2, i7, c, g, t, lane);  // kS^2 T2 = kS^2 (15I - 7X + X X)
-        }
-        dist_put<M>(oth, acc, -0.25f / kS, c, g, t);  // kS (-T2/4)
-        csync();
-        {
-            const H2Pair(*const As[1])[4] = {Xa};
-            float(*const Ds[1])[4] = {acc};
-            dist_mm<M, 1, false>(As, oth, Ds, 3.25f * kS2, 0u, c, g, t, lane);  // kS^2 T3/4
-        }
-        dist_put<M>(cur, acc, 1.f / kS, c, g, t);  // kS T3/4 (every warp is done with X)
-        csync();
-        if (it + 1 < iters) {
-            const H2Pair(*const As[2])[4] = {Za, Xa};
-            float(*const Ds[2])[4] = {zc, acc};
-            dist_mm<M, 2, false>(As, cur, Ds, 0.f, 0u, c, g, t, lane);  // Z kS T3/4, kS^2 X T3/4
-            dist_put_sym<M>(oth, acc, 1.f / kS, c, g, t, sel);       // every warp is done with -T2/4
-            float zm = 0.f;
-#pragma unroll
-            for (int n = 0; n < NT; ++n)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) zm = fmaxf(zm, fabsf(zc[n][e]));
-            zm = warp_max_nonneg(zm);
-            if (lane == 0) slots[CW + c] = zm;
-            csync();
-            dist_load_a<M, false>(oth, Xa, c, lane);
-            unsigned char* tmp = cur;
-            cur = oth;
-            oth = tmp;
-            float zmax = 0.f;
-#pragma unroll
-            for (int w = 0; w < CW; ++w) zmax = fmaxf(zmax, slots[CW + w]);
-            const float sc = (zmax > 0.f && zmax < INFINITY) ? pow2i(10 - ilogbf(zmax)) : 1.f;
-#pragma unroll
-            for (int kk = 0; kk < KT; ++kk)
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const int n = 2 * kk + (r >> 1), e = 2 * (r & 1);
-                    Za[kk][r] = split_h2(sc * zc[n][e], sc * zc[n][e + 1]);
-                }
-        } else {
-            const H2Pair(*const As[1])[4] = {Za};
-            float(*const Ds[1])[4] = {zc};
-            dist_mm<M, 1, false>(As, cur, Ds, 0.f, 0u, c, g, t, lane);  // Z T3/4
-        }
-    }
-    // ---- Y = Z W, own rows (split-tf32), stored as Y^T ----
-    {
-        float y[NTO][4];
-#pragma unroll
-        for (int j = 0; j < NTO; ++j) y[j][0] = y[j][1] = y[j][2] = y[j][3] = 0.f;
-#pragma unroll
-        for (int kk = 0; kk < NT; ++kk) {
-            const uint32_t ah[4] = {__float_as_uint(zc[kk][0]), __float_as_uint(zc[kk][2]), __float_as_uint(zc[kk][1]),
-                                    __float_as_uint(zc[kk][3])};
-            const uint32_t al[4] = {tf32_lo(zc[kk][0]), tf32_lo(zc[kk][2]), tf32_lo(zc[kk][1]), tf32_lo(zc[kk][3])};
-#pragma unroll
-            for (int j = 0; j < NTO; ++j) {
-                const float y0 = mW[(8 * kk + 2 * t) * WS + 8 * j + g];
-                const float y1 = mW[(8 * kk + 2 * t + 1) * WS + 8 * j + g];
-                const uint32_t bh0 = __float_as_uint(y0), bh1 = __float_as_uint(y1);
-                const uint32_t bl0 = tf32_lo(y0), bl1 = tf32_lo(y1);
-                mma_tf32(y[j], al[0], al[1], al[2], al[3], bh0, bh1);
-                mma_tf32(y[j], ah[0], ah[1], ah[2], ah[3], bl0, bl1);
-                mma_tf32(y[j], ah[0], ah[1], ah[2], ah[3], bh0, bh1);
-            }
-        }
-        float scale = 1.f;
-        if (O::kNarrowRange) {
-            float ym = 0.f;
-#pragma unroll
-            for (int j = 0; j < NTO; ++j)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) ym = fmaxf(ym, fabsf(y[j][e]));
-            ym = warp_max_nonneg(ym);
-            if (lane == 0) slots[2 * CW + c] = ym;
-            csync();
-            float ymax = 0.f;
-#pragma unroll
-            for (int w = 0; w < CW; ++w) ymax = fmaxf(ymax, slots[2 * CW + w]);
-            if (ymax > 0.f && ymax < INFINITY) scale = pow2i(14 - ilogbf(ymax));
-        }
-        csync();  // Y^T may overlay W, which every core warp reads in full
-#pragma unroll
-        for (int j = 0; j < NTO; ++j) {
-            const int rr = 16 * c + g, cc = 8 * j + 2 * t;
-            DSt<T>::put(yT + cc * YS + rr, YLO, y[j][0] * scale);
-            DSt<T>::put(yT + (cc + 1) * YS + rr, YLO, y[j][1] * scale);
-            DSt<T>::put(yT + cc * YS + rr + 8, YLO, y[j][2] * scale);
-            DSt<T>::put(yT + (cc + 1) * YS + rr + 8, YLO, y[j][3] * scale);
-        }
-    }
-}
-
 }  // namespace tc
 }  // namespace nystra
 
@@ -1592,7 +1191,7 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
     constexpr int LPW = TPW / L;  // landmarks owned by one warp
     static_assert(sizeof(T) == 2, "the grouped kernel takes 16-bit I/O (its layout assumes it)");
     static_assert(L <= TPW && TPW % L == 0, "segments must not straddle warps");
-    static_assert(CW == 1 || CW == M / 16, "the distributed core has one warp per 16 landmarks");
+    static_assert(CW == 1 || CW == M / 16, "a core on several warps has one per 16 landmarks");
 
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1629,25 +1228,18 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
             return named_barrier_or(1 + grp, GW * 32, f);
         }
     };
-    // distributed-core scratch
+    // scratch of the core on several warps
     unsigned char* mat0 = nullptr;
     unsigned char* mat1 = nullptr;
     unsigned char* wmat = nullptr;
     float* aux = nullptr;
     if constexpr (CW > 1) {
-        if constexpr (Lay::SCR_IN_STAGE) {
-            using SSc = ScScratch<64>;
-            unsigned char* w0 = smem_raw + (size_t)GROUPS * Lay::GROUP_BYTES + (size_t)(grp * WPU) * Lay::WARP_BYTES;
-            mat0 = w0 + Lay::WPART;
-            aux = reinterpret_cast<float*>(mat0 + SSc::MAT);
-            mat1 = w0 + Lay::WARP_BYTES + Lay::WPART;
-            wmat = mat1 + SSc::MAT;
-        } else {
-            using DSc = DistScratch<(M > 16 ? M : 32)>;
-            mat0 = gb + Lay::G_SCR;
-            mat1 = mat0 + DSc::MAT;
-            aux = reinterpret_cast<float*>(mat1 + DSc::MAT);
-        }
+        using Sc = ScScratch<64>;
+        unsigned char* w0 = smem_raw + (size_t)GROUPS * Lay::GROUP_BYTES + (size_t)(grp * WPU) * Lay::WARP_BYTES;
+        mat0 = w0 + Lay::WPART;
+        aux = reinterpret_cast<float*>(mat0 + Sc::MAT);
+        mat1 = w0 + Lay::WARP_BYTES + Lay::WPART;
+        wmat = mat1 + Sc::MAT;
     }
 
     // Only the first `active` groups of a CTA take units (see launch_cfg).
@@ -1770,7 +1362,7 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
                 pend_qk = true;
             }
         };
-        if constexpr (!Lay::SCR_IN_STAGE) prefetch_qk();
+        if constexpr (CW == 1) prefetch_qk();
 
         // ---------------- core: G_A^n, Z_0, iteration, Y ----------------
         if constexpr (CW == 1) {
@@ -1785,20 +1377,15 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
                 core_warp<T, M, NCOL>(qbar, kbar, mU, mW, yT, iters, sl2, g, t);
             }
         } else {
-            if constexpr (M == 64) {
-                if (r < CW) {
-                    float w[NCOL / 8][4];
-                    sc_load_w<NCOL>(mW, w, r, g, t);
-                    sc_core<T, M, NCOL>(qbar, kbar, gmu[16 * r + g], gmu[16 * r + g + 8], w, yT, mat0, mat1, wmat, aux,
-                                        iters, sl2, r, lane, 1 + GROUPS + grp);
-                }
-            } else if (r < CW) {
-                dist_core<T, (M > 16 ? M : 32), NCOL>(qbar, kbar, gmu, mW, yT, mat0, mat1, aux, iters, sl2, r, lane,
-                                                      1 + GROUPS + grp);
+            if (r < CW) {
+                float w[NCOL / 8][4];
+                sc_load_w<NCOL>(mW, w, r, g, t);
+                sc_core<T, M, NCOL>(qbar, kbar, gmu[16 * r + g], gmu[16 * r + g + 8], w, yT, mat0, mat1, wmat, aux,
+                                    iters, sl2, r, lane, 1 + GROUPS + grp);
             }
         }
         gsync();
-        if constexpr (Lay::SCR_IN_STAGE) prefetch_qk();
+        if constexpr (CW > 1) prefetch_qk();
 
         if (tok) {
             // ---------------- output: O = (G_L^n Y_:d) / (G_L^n Y_d) ----------------
@@ -1946,9 +1533,9 @@ cudaError_t launch_n(const void* q, const void* k, const void* v, void* out, lon
         if (m == 16)
             return wide ? launch_team<T, 16, 40>(q, k, v, out, n_units, d, iters, stream, fault, bias)
                         : launch_team<T, 16, 32>(q, k, v, out, n_units, d, iters, stream, fault, bias);
-        // m = 32 with d_h <= 30 fits two teams per SM; d_h = 32 only one, so it
-        // stays on the grouped kernel
-        if (m == 32 && !wide) return launch_team<T, 32, 32>(q, k, v, out, n_units, d, iters, stream, fault);
+        if (m == 32)
+            return wide ? launch_team<T, 32, 40>(q, k, v, out, n_units, d, iters, stream, fault)
+                        : launch_team<T, 32, 32>(q, k, v, out, n_units, d, iters, stream, fault);
     }
     if constexpr (TPW == 128 && WPU == 8) {
         if (m == 8)
@@ -1962,16 +1549,13 @@ cudaError_t launch_n(const void* q, const void* k, const void* v, void* out, lon
                         : launch_stream<T, 32, 32>(q, k, v, out, n_units, d, iters, stream, fault);
     }
     // The grouped kernel: m = 32 at 8x8 windows (core in one warp's registers;
-    // 20000 units of d_h = 30 take 400 us, on the wide kernel's two warps 519)
-    // and at 16x16 windows with d_h = 32 (core on two warps), m = 64 at 32x32
-    // windows.  The wide kernel: m = 64 at 8x8 and 16x16.
+    // 20000 units of d_h = 30 take 400 us, on the wide kernel's two warps 519) and
+    // m = 64 at 32x32 windows.  The wide kernel: m = 64 at 8x8 and 16x16.
     if (m == 32) {
         if constexpr (TPW == 64 && WPU == 1)
             return wide ? launch_cfg<T, 32, 40, 64, 1, 1>(q, k, v, out, n_units, d, iters, stream, fault)
                         : launch_cfg<T, 32, 32, 64, 1, 1>(q, k, v, out, n_units, d, iters, stream, fault);
-        if constexpr (TPW == 64 && WPU == 4)
-            return launch_cfg<T, 32, 40, 64, 4, 2>(q, k, v, out, n_units, d, iters, stream, fault);
-        return cudaErrorInvalidValue;  // not reached: the stream kernel takes 32x32 windows
+        return cudaErrorInvalidValue;  // not reached: the team and stream kernels take the larger windows
     }
     if (m == 64) {
         if constexpr (TPW * WPU == 1024)  // a token warp of 256 rows: W partials of 64 rows lie over its K/V rows

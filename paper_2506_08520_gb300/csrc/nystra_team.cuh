@@ -1,5 +1,5 @@
 // Team PnP-Nystra kernel for 16x16 windows (N = 256 tokens), m <= 32, even
-// d_h <= 32, 16-bit I/O (m = 32: the core runs on two warps, dist_core).  Included by the N = 256 translation unit after
+// d_h <= 32, 16-bit I/O (m = 32: the core runs on two warps, sc_core).  Included by the N = 256 translation unit after
 // nystra_tc.cuh, whose per-phase device functions it reuses.
 //
 // In the grouped kernel the m x m core runs on one warp of a unit's group
@@ -38,7 +38,7 @@ namespace tc {
 template <typename T, int M, int NCOL>
 struct TeamLayout {
     static constexpr int NT = 4, TPW = 64, N = NT * TPW;  // token warps, tokens per token warp
-    static constexpr int CWN = M > 16 ? M / 16 : 1;        // core warps (m = 32: distributed core)
+    static constexpr int CWN = M > 16 ? M / 16 : 1;        // core warps (m = 32: sc_core)
     static constexpr int DS = (NCOL == 32) ? 30 : 32;
     static constexpr int MP = M > 16 ? M : 16, LS = LmS<T>::LS, WS = NCOL + 4;
     static constexpr int KTL = (M >= 16) ? M / 16 : 1;
@@ -55,9 +55,9 @@ struct TeamLayout {
     // team memory: stages, two buffers, mbarriers
     static constexpr size_t T_BUF = NT * STAGE;
     static constexpr size_t T_BAR = T_BUF + 2 * BUF;  // barQK[4], barV[4], F[2], C[2]
-    static constexpr size_t T_SCR = ((T_BAR + 12 * 8 + 127) / 128) * 128;  // distributed core's scratch
+    static constexpr size_t T_SCR = ((T_BAR + 12 * 8 + 127) / 128) * 128;  // sc_core's scratch
     static constexpr size_t TEAM =
-        ((T_SCR + (CWN > 1 ? DistScratch<(M > 16 ? M : 32)>::BYTES : 0) + 127) / 128) * 128;
+        ((T_SCR + (CWN > 1 ? ScScratch<(M > 16 ? M : 32)>::BYTES : 0) + 127) / 128) * 128;
     static constexpr int TEAMS = (int)(kSmemLimit / TEAM) < 3 ? (int)(kSmemLimit / TEAM) : 3;
     static constexpr int WARPS = NT + CWN;  // per team
     static_assert(TEAMS >= 1, "team does not fit in shared memory");
@@ -143,13 +143,15 @@ nystra_team_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
                                                     reinterpret_cast<T*>(bb + Lay::B_YT), iters, sl2, g, t,
                                                     nullptr, bAu);
             } else {
-                using DSc = DistScratch<(M > 16 ? M : 32)>;
+                using Sc = ScScratch<(M > 16 ? M : 32)>;
                 unsigned char* scr = tb + Lay::T_SCR;
-                dist_core<T, (M > 16 ? M : 32), NCOLC>(
-                    reinterpret_cast<const T*>(bb + Lay::B_QB), reinterpret_cast<const T*>(bb + Lay::B_KB), gmu,
-                    reinterpret_cast<const float*>(bb + Lay::B_W), reinterpret_cast<T*>(bb + Lay::B_YT), scr,
-                    scr + DSc::MAT, reinterpret_cast<float*>(scr + 2 * DSc::MAT), iters, sl2, c, lane,
-                    1 + Lay::TEAMS + team);
+                float wr[NCOLC / 8][4];
+                sc_load_w<NCOLC>(reinterpret_cast<const float*>(bb + Lay::B_W), wr, c, g, t);
+                sc_core<T, (M > 16 ? M : 32), NCOLC>(
+                    reinterpret_cast<const T*>(bb + Lay::B_QB), reinterpret_cast<const T*>(bb + Lay::B_KB),
+                    gmu[16 * c + g], gmu[16 * c + g + 8], wr, reinterpret_cast<T*>(bb + Lay::B_YT), scr,
+                    scr + Sc::MAT, scr + 2 * Sc::MAT, reinterpret_cast<float*>(scr + 2 * Sc::MAT + Sc::WMAT), iters,
+                    sl2, c, lane, 1 + Lay::TEAMS + team);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(barC + b);
