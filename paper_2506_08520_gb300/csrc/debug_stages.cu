@@ -61,9 +61,14 @@ struct DumpOffsets {
     }
 };
 
-// RS: token order of the staged rows, as the product kernel takes it for
-// this d_h (row_step of its compile-time width), so that the dumped output
-// is the product kernel's bit for bit.
+// RS: order of the staged rows, as the product kernel takes it for this d_h
+// (row_order of its compile-time width), so that the dumped output is the
+// product kernel's bit for bit.  With kSlots the features of Qbar, Kbar, W and Y
+// lie in slot order.
+template <int RS>
+__device__ __forceinline__ int feature_at(int f) {
+    return RS == kSlots && f < 32 ? 4 * (f & 6) + 2 * (f >> 3) + (f & 1) : f;
+}
 template <typename T, int M, int NCOL, int PW, int RS>
 __global__ void __launch_bounds__(32, 1)
 nystra_stage_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, long long unit,
@@ -101,8 +106,8 @@ nystra_stage_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
     }
     __syncwarp();
     for (int i = lane; i < M * d; i += 32) {
-        dump[off.qbar + i] = lm_f32<T>(qbar + (i / d) * P::LS + i % d);
-        dump[off.kbar + i] = lm_f32<T>(kbar + (i / d) * P::LS + i % d);
+        dump[off.qbar + i] = lm_f32<T>(qbar + (i / d) * P::LS + feature_at<RS>(i % d));
+        dump[off.kbar + i] = lm_f32<T>(kbar + (i / d) * P::LS + feature_at<RS>(i % d));
     }
 
     // steps 2-3: S_L, m_L, G_L^n (the operand registers of O = G_L^n Y)
@@ -131,7 +136,8 @@ nystra_stage_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
         if (g < M) dump[off.mu + g] = mU[0][0] * 0.69314718055994531f;
         if (g + 8 < M) dump[off.mu + g + 8] = mU[0][1] * 0.69314718055994531f;
     }
-    for (int i = lane; i < M * (d + 1); i += 32) dump[off.w + i] = mW[(i / (d + 1)) * P::WS + i % (d + 1)];
+    for (int i = lane; i < M * (d + 1); i += 32)
+        dump[off.w + i] = mW[(i / (d + 1)) * P::WS + feature_at<RS>(i % (d + 1))];
 
     // steps 3-4, 6: G_A^n, the pseudo-inverse iteration, Y = Z W
     core_warp<T, M, NCOL, true>(qbar, kbar, mU, mW, yT, iters, sl2, g, t, dbg);
@@ -140,7 +146,8 @@ nystra_stage_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
         dump[off.ga + i] = dbg[i];
         dump[off.z + i] = dbg[M * M + i];
     }
-    for (int i = lane; i < M * (d + 1); i += 32) dump[off.y + i] = dbg[2 * M * M + (i / (d + 1)) * NCOL + i % (d + 1)];
+    for (int i = lane; i < M * (d + 1); i += 32)
+        dump[off.y + i] = dbg[2 * M * M + (i / (d + 1)) * NCOL + feature_at<RS>(i % (d + 1))];
 
     // step 7: O = (G_L^n Y_:d) / (G_L^n Y_d)
     output_rows<T, M, NCOL, 1, true, false, RS>(glf, Qs, kbar, yT, ob, d, g, t, lane, sl2);
@@ -152,8 +159,9 @@ template <typename T, int M, int NCOL, int PW>
 cudaError_t launch_stage(const void* q, const void* k, const void* v, long long unit, int d, int iters,
                          float* dump, cudaStream_t stream) {
     using P = StageLayout<T, M, NCOL>;
-    // the product kernel compiles d_h = 30 in (row_step(30)); other widths keep token order
-    auto kern = d == 30 ? nystra_stage_kernel<T, M, NCOL, PW, row_step(30)> : nystra_stage_kernel<T, M, NCOL, PW, 1>;
+    // the product kernel compiles d_h = 30 and 32 in; other widths keep token order
+    constexpr int kDc = NCOL == 32 ? 30 : 32;
+    auto kern = d == kDc ? nystra_stage_kernel<T, M, NCOL, PW, row_order<T>(kDc)> : nystra_stage_kernel<T, M, NCOL, PW, 1>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::BYTES);
     if (e != cudaSuccess) return e;
     const float sl2 = 1.4426950408889634f / sqrtf((float)d);

@@ -70,7 +70,7 @@ nystra_pool_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
     const int d = DC ? DC : d_in;  // d_h, a compile-time constant for the common head widths
     using P = PoolLayout<T, M, NCOL>;
     constexpr int L = 64 / M;  // tokens per landmark segment
-    constexpr int RS = row_step(DC);  // token order of the staged rows (bank-conflict-free fragment loads)
+    constexpr int RS = row_order<T>(DC);  // token order of the staged rows (bank-conflict-free fragment loads)
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;

@@ -118,7 +118,7 @@ nystra_stream_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
     using Lay = StreamLayout<T, M, NCOL>;
     using TL = typename Lay::TL;
     using R = typename Opnd<T>::DReg;
-    constexpr int RS = row_step(DC);  // token order of the chunk rows (bank-conflict-free fragment loads)
+    constexpr int RS = row_order<T>(DC);  // token order of the chunk rows (bank-conflict-free fragment loads)
     constexpr int NT = Lay::NT, TPW = Lay::TPW, N = Lay::N, MP = Lay::MP, WS = Lay::WS,
                   NSLOT = Lay::NSLOT, L = Lay::L, LPW = Lay::LPW, NTO = NCOL / 8, MT = Lay::MT;
 

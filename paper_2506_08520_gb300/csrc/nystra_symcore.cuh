@@ -38,8 +38,8 @@ namespace tc {
 // m = 64, 4096 units of 16x16 windows, d_h = 32, 0.93 -> 0.50 ms (in the wide
 // kernel, with three groups per SM instead of two), 1024 of 32x32 0.50 -> 0.37;
 // m = 32, 8192 units of 16x16, d_h = 30, 353 -> 290 us (d_h = 32 now in the team
-// kernel too: 557 -> 345); 1024 units of 32x32, d_h = 32, not bound by the core,
-// 144 us as before.  At m = 64, carrying V = Z W
+// kernel too: 557 -> 345, and 304 with 16-byte row loads); 1024 units of 32x32,
+// d_h = 32, not bound by the core, 144 us as before (134 with those loads).  At m = 64, carrying V = Z W
 // instead (V <- T3 V/4 with X = Z A: d_h + 1 columns instead of m, 20 tile
 // products a step, but V's column scales to agree on in every step) took 0.51 and
 // 0.46 ms, and was less accurate: under sharp attention (logit std 4) its

@@ -82,9 +82,26 @@ __device__ __forceinline__ float pow2i(int e) {
 // so the kernels pick the order freely.  Rows g and g + 8 of a 16-row tile tm
 // are tiles 2 tm and 2 tm + 1: tokens mtok<RS>(tm, g) and that + mrow<RS>().
 constexpr int row_step(int d) { return d <= 0 ? 1 : ((d / 2) % 2 == 1 ? 4 : ((d / 2) % 4 == 2 ? 2 : 1)); }
+// No order helps rows of w = 16 words (d_h = 32, 16-bit I/O): there a lane loads
+// 16 bytes at once instead (RS = kSlots, tokens in row order; the 32 lanes read
+// 512 consecutive bytes).  Lane t of a row then holds words 4t .. 4t + 3, and
+// fragment word j (0 .. 3) of lane t is word 4t + j instead of word t + 4j: the
+// features are taken in slot order, slot 8j + 2t + e for feature 8t + 2j + e.
+// Q, K and V are all read so, a contraction over features does not mind, and
+// what keeps features as rows or columns (Qbar, Kbar, W, Y^T) keeps them in slot
+// order, up to the output, where lane t holds features 8t .. 8t + 7: one 16-byte
+// store.  In place of 4-byte loads with four lanes to a bank, bf16, d_h = 32,
+// m = 16: 20250 units of 16x16 windows 398 -> 302 us, 5160 of 32x32 429 -> 342,
+// 81000 of 8x8 494 -> 438; m = 64, 4096 of 16x16 492 -> 452.
+constexpr int kSlots = 32;
+template <typename T>
+constexpr int row_order(int d) {
+    return sizeof(T) == 2 && d == 32 ? kSlots : row_step(d);
+}
 template <int RS>
 __device__ __forceinline__ int ctok(int j, int i) {
-    return 8 * RS * (j / RS) + (j % RS) + RS * i;
+    constexpr int S = RS == kSlots ? 1 : RS;
+    return 8 * S * (j / S) + (j % S) + S * i;
 }
 template <int RS>
 __device__ __forceinline__ int mtok(int tm, int g) {
@@ -92,7 +109,15 @@ __device__ __forceinline__ int mtok(int tm, int g) {
 }
 template <int RS>
 __host__ __device__ constexpr int mrow() {
-    return RS == 1 ? 8 : 1;
+    return RS == 1 || RS == kSlots ? 8 : 1;
+}
+// Words 4t .. 4t + 3 of a 64-byte row.
+template <typename T>
+__device__ __forceinline__ uint4 ld_row16(const T* row, int t) {
+    return *reinterpret_cast<const uint4*>(row + 8 * t);
+}
+__device__ __forceinline__ uint32_t word4(const uint4& x, int j) {
+    return j == 0 ? x.x : j == 1 ? x.y : j == 2 ? x.z : x.w;
 }
 static_assert(row_step(30) == 4 && row_step(28) == 2 && row_step(32) == 1 && row_step(0) == 1, "row steps");
 
@@ -394,6 +419,33 @@ __device__ __forceinline__ float warp_max_f(float x) {
 // down to 2^-13 of its largest one.
 __device__ __forceinline__ int h2_exponent(float x) { return (x > 0.f && x < INFINITY) ? 10 - ilogbf(x) : 0; }
 
+// A operand of a 16-token tile of Q: rows q0 (row g) and mrow<RS>() further on
+// (row g + 8).
+template <typename T, int RS>
+__device__ __forceinline__ void q_afrag(const T* q0, int d, int t, typename Opnd<T>::Reg (&a)[2][4]) {
+    using O = Opnd<T>;
+    const T* q1 = q0 + mrow<RS>() * d;
+    if constexpr (RS == kSlots) {
+        const uint4 x = ld_row16(q0, t), y = ld_row16(q1, t);
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk) {
+            a[kk][0] = word4(x, 2 * kk);
+            a[kk][1] = word4(y, 2 * kk);
+            a[kk][2] = word4(x, 2 * kk + 1);
+            a[kk][3] = word4(y, 2 * kk + 1);
+        }
+    } else {
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk) {
+            const int c0 = 16 * kk + 2 * t, c1 = c0 + 8;
+            a[kk][0] = c0 < d ? O::ld(q0 + c0) : O::zero();
+            a[kk][1] = c0 < d ? O::ld(q1 + c0) : O::zero();
+            a[kk][2] = c1 < d ? O::ld(q0 + c1) : O::zero();
+            a[kk][3] = c1 < d ? O::ld(q1 + c1) : O::zero();
+        }
+    }
+}
+
 // S_L for one 16-token tile of the stage and its G_L^n fragments (A operand
 // of O = G_L^n Y, k = landmarks).  q0: row g of the tile (token mtok<RS>(tm,
 // g) of its chunk); row g + 8 lies mrow<RS>() rows further on.
@@ -414,15 +466,7 @@ __device__ __forceinline__ void gl_tile(const T* q0, const T* kbar, int d, int g
         }
     }
     R a[2][4];
-    const T* q1 = q0 + mrow<RS>() * d;
-#pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-        const int c0 = 16 * kk + 2 * t, c1 = c0 + 8;
-        a[kk][0] = c0 < d ? O::ld(q0 + c0) : O::zero();
-        a[kk][1] = c0 < d ? O::ld(q1 + c0) : O::zero();
-        a[kk][2] = c1 < d ? O::ld(q0 + c1) : O::zero();
-        a[kk][3] = c1 < d ? O::ld(q1 + c1) : O::zero();
-    }
+    q_afrag<T, RS>(q0, d, t, a);
     float sl[NTL][4];
 #pragma unroll
     for (int j = 0; j < NTL; ++j) {
@@ -566,16 +610,29 @@ __device__ __forceinline__ void landmarks_acc(const T* X, int tok0, float (&c)[2
     for (int ks = 0; ks < 4; ++ks) {  // 16 tokens per k-step: 8-row tiles 2 ks and 2 ks + 1
         // A = X^T, features 16 mf + g (+8); k = 8 b + 2t (+1): token ctok(2 ks + b, 2t (+1))
         R a[2][4];
+        if constexpr (RS == kSlots) {
 #pragma unroll
-        for (int mf = 0; mf < 2; ++mf)
+            for (int h = 0; h < 2; ++h) {
+                const uint4 x = ld_row16(X + ctok<RS>(2 * ks + h, g) * d, t);
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int f0 = 16 * mf + 8 * (r & 1) + 2 * t;
-                const R x = f0 < d ? O::ld(X + ctok<RS>(2 * ks + (r >> 1), g) * d + f0) : O::zero();
-                a[mf][r] = O::tr(x);
+                for (int mf = 0; mf < 2; ++mf) {
+                    a[mf][2 * h] = O::tr(word4(x, 2 * mf));
+                    a[mf][2 * h + 1] = O::tr(word4(x, 2 * mf + 1));
+                }
             }
+        } else {
+#pragma unroll
+            for (int mf = 0; mf < 2; ++mf)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int f0 = 16 * mf + 8 * (r & 1) + 2 * t;
+                    const R x = f0 < d ? O::ld(X + ctok<RS>(2 * ks + (r >> 1), g) * d + f0) : O::zero();
+                    a[mf][r] = O::tr(x);
+                }
+        }
         // the k-step's tokens lie in [lo, hi] of the chunk
-        const int lo = 8 * RS * ((2 * ks) / RS), hi = 8 * RS * ((2 * ks + 1) / RS) + 8 * RS - 1;
+        constexpr int S = RS == kSlots ? 1 : RS;
+        const int lo = 8 * S * ((2 * ks) / S), hi = 8 * S * ((2 * ks + 1) / S) + 8 * S - 1;
         const int jlo = Pool::tile_lo(tok0 + lo), jhi = Pool::tile_hi(tok0 + hi - 15);
 #pragma unroll
         for (int j = 0; j < NTJ; ++j) {
@@ -672,7 +729,7 @@ __device__ __forceinline__ void su_w_chunk(const typename Opnd<T>::DReg (&aq)[2]
             } else {
 #pragma unroll
                 for (int nt = 0; nt < 8; ++nt) {
-                    if constexpr (RS == 1)
+                    if constexpr (RS == 1 || RS == kSlots)
                         b[nt] = real ? __ldg(reinterpret_cast<const float2*>(p + 8 * nt + 2 * t)) : make_float2(0.f, 0.f);
                     else
                         b[nt] = real ? make_float2(__ldg(p + ctok<RS>(nt, 2 * t)), __ldg(p + ctok<RS>(nt, 2 * t + 1)))
@@ -687,13 +744,19 @@ __device__ __forceinline__ void su_w_chunk(const typename Opnd<T>::DReg (&aq)[2]
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
         const T* kr = Kc + ctok<RS>(nt, g) * d;
+        if constexpr (RS == kSlots) {
+            const uint4 x = ld_row16(kr, t);
+            O::mmaz(s[nt], aq[0], x.x, x.y);
+            O::mma(s[nt], aq[1], x.z, x.w);
+        } else {
 #pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-            const int c0 = 16 * kk + 2 * t, c1 = c0 + 8;
-            const R b0 = c0 < d ? O::ld(kr + c0) : O::zero();
-            const R b1 = c1 < d ? O::ld(kr + c1) : O::zero();
-            if (kk == 0) O::mmaz(s[nt], aq[kk], b0, b1);
-            else O::mma(s[nt], aq[kk], b0, b1);
+            for (int kk = 0; kk < 2; ++kk) {
+                const int c0 = 16 * kk + 2 * t, c1 = c0 + 8;
+                const R b0 = c0 < d ? O::ld(kr + c0) : O::zero();
+                const R b1 = c1 < d ? O::ld(kr + c1) : O::zero();
+                if (kk == 0) O::mmaz(s[nt], aq[kk], b0, b1);
+                else O::mma(s[nt], aq[kk], b0, b1);
+            }
         }
     }
     if constexpr (BIAS) {  // scores in the log2 domain, bias included (rows beyond m stay unbiased)
@@ -735,12 +798,20 @@ __device__ __forceinline__ void su_w_chunk(const typename Opnd<T>::DReg (&aq)[2]
         a[1] = v1 ? e(s[2 * kt][2], s[2 * kt][3], mx1) : O::dzero();
         a[2] = v0 ? e(s[2 * kt + 1][0], s[2 * kt + 1][1], mx0) : O::dzero();
         a[3] = v1 ? e(s[2 * kt + 1][2], s[2 * kt + 1][3], mx1) : O::dzero();
+        if constexpr (RS == kSlots) {
+            const uint4 x = ld_row16(Vc + ctok<RS>(2 * kt, g) * d, t), y = ld_row16(Vc + ctok<RS>(2 * kt + 1, g) * d, t);
 #pragma unroll
-        for (int j = 0; j < NTO; ++j) {
-            const int c0 = 8 * j + 2 * t;
-            const R x0 = c0 < d ? O::ld(Vc + ctok<RS>(2 * kt, g) * d + c0) : (c0 == d ? O::one() : O::zero());
-            const R x1 = c0 < d ? O::ld(Vc + ctok<RS>(2 * kt + 1, g) * d + c0) : (c0 == d ? O::one() : O::zero());
-            O::mma(w[j], a, O::tr(x0), O::tr(x1));
+            for (int j = 0; j < 4; ++j) O::mma(w[j], a, O::tr(word4(x, j)), O::tr(word4(y, j)));
+            const R one = O::tr(t == 0 ? O::one() : O::zero());
+            O::mma(w[NTO - 1], a, one, one);
+        } else {
+#pragma unroll
+            for (int j = 0; j < NTO; ++j) {
+                const int c0 = 8 * j + 2 * t;
+                const R x0 = c0 < d ? O::ld(Vc + ctok<RS>(2 * kt, g) * d + c0) : (c0 == d ? O::one() : O::zero());
+                const R x1 = c0 < d ? O::ld(Vc + ctok<RS>(2 * kt + 1, g) * d + c0) : (c0 == d ? O::one() : O::zero());
+                O::mma(w[j], a, O::tr(x0), O::tr(x1));
+            }
         }
     }
 }
@@ -1105,6 +1176,31 @@ __device__ __forceinline__ void core_warp(const T* qbar, const T* kbar, const fl
 namespace nystra {
 namespace tc {
 
+// Rows o0 (row g) and mrow<RS>() further on (row g + 8) of an output tile, o
+// scaled by i0 and i1.
+template <typename T, int NTO, int RS>
+__device__ __forceinline__ void store_orows(T* o0, int d, int t, const float (&o)[NTO][4], float i0, float i1) {
+    using O = Opnd<T>;
+    T* o1 = o0 + mrow<RS>() * d;
+    if constexpr (RS == kSlots) {
+        *reinterpret_cast<uint4*>(o0 + 8 * t) =
+            make_uint4(O::pk(o[0][0] * i0, o[0][1] * i0), O::pk(o[1][0] * i0, o[1][1] * i0),
+                       O::pk(o[2][0] * i0, o[2][1] * i0), O::pk(o[3][0] * i0, o[3][1] * i0));
+        *reinterpret_cast<uint4*>(o1 + 8 * t) =
+            make_uint4(O::pk(o[0][2] * i1, o[0][3] * i1), O::pk(o[1][2] * i1, o[1][3] * i1),
+                       O::pk(o[2][2] * i1, o[2][3] * i1), O::pk(o[3][2] * i1, o[3][3] * i1));
+    } else {
+#pragma unroll
+        for (int j = 0; j < NTO; ++j) {
+            const int c = 8 * j + 2 * t;
+            if (c < d) {
+                O::st2(o0 + c, o[j][0] * i0, o[j][1] * i0);
+                O::st2(o1 + c, o[j][2] * i1, o[j][3] * i1);
+            }
+        }
+    }
+}
+
 // Output for one warp's NCH chunks: O = (G_L^n Y_:d) / (G_L^n Y_d) (steps
 // 5-7); G_L^n fragments come from glf (parked) or are recomputed from Qs and
 // Kbar; rows are written row-major to obase (N_w x d), each to its own token
@@ -1166,16 +1262,7 @@ __device__ __forceinline__ void output_rows(const uint32_t* glf, const T* Qs, co
                 }
             const float i0 = __fdividef(1.f, __shfl_sync(0xffffffffu, d0, src));
             const float i1 = __fdividef(1.f, __shfl_sync(0xffffffffu, d1, src));
-            T* o0 = obase + (ch * 64 + mtok<RS>(tm, g)) * d;
-            T* o1 = o0 + mrow<RS>() * d;
-#pragma unroll
-            for (int j = 0; j < NTO; ++j) {
-                const int c = 8 * j + 2 * t;
-                if (c < d) {
-                    O::st2(o0 + c, o[j][0] * i0, o[j][1] * i0);
-                    O::st2(o1 + c, o[j][2] * i1, o[j][3] * i1);
-                }
-            }
+            store_orows<T, NTO, RS>(obase + (ch * 64 + mtok<RS>(tm, g)) * d, d, t, o, i0, i1);
         }
 }
 

@@ -74,7 +74,7 @@ nystra_team_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
     using Lay = TeamLayout<T, M, NCOL>;
     constexpr int NT = Lay::NT, TPW = Lay::TPW, N = Lay::N, MP = Lay::MP, WS = Lay::WS, NCOLC = NCOL;
     constexpr int L = N / M, LPW = TPW / L;
-    constexpr int RS = row_step(DC);  // token order of the staged rows (bank-conflict-free fragment loads)
+    constexpr int RS = row_order<T>(DC);  // token order of the staged rows (bank-conflict-free fragment loads)
     static_assert(L <= TPW && TPW % L == 0, "segments must not straddle warps");
 
     extern __shared__ __align__(128) unsigned char smem_raw[];

@@ -16,7 +16,8 @@
 // a group per SM, and the SM's other groups fill the wait.  Three groups of
 // four warps run per SM (73 KB each at N = 256), against two groups with 108 KB
 // and two token warps each on the grouped kernel.
-// Measured (bf16): 4096 units of 16x16 windows, d_h = 32: 0.93 -> 0.50 ms;
+// Measured (bf16): 4096 units of 16x16 windows, d_h = 32: 0.93 -> 0.50 ms (0.45
+// with the rows read 16 bytes at a time);
 // 8640 units of 8x8 windows, d_h = 30: 1.45 -> 0.78 ms.
 //
 // Every wait on an mbarrier is bounded; the warps of a group share its
@@ -51,8 +52,9 @@ struct WideLayout {
 };
 
 // Landmark means of X (N rows of d) into xbar, thread id of n: fp32 sums of L
-// 16-bit values times 1/L (a power of two), stored as DSt does.
-template <typename T, int M, int N>
+// 16-bit values times 1/L (a power of two), stored as DSt does (in slot order
+// for RS = kSlots).
+template <typename T, int M, int N, int RS>
 __device__ __forceinline__ void wide_landmarks(const T* X, T* xbar, int d, int id, int n) {
     constexpr int L = N / M, LS = LmS<T>::LS, LO = LmS<T>::LO;
     for (int i = id; i < M * 16; i += n) {
@@ -67,8 +69,9 @@ __device__ __forceinline__ void wide_landmarks(const T* X, T* xbar, int d, int i
                 b += f.y;
             }
         }
-        DSt<T>::put(xbar + j * LS + c, LO, a * (1.f / L));
-        DSt<T>::put(xbar + j * LS + c + 1, LO, b * (1.f / L));
+        const int p = RS == kSlots ? 4 * (c & 6) + 2 * (c >> 3) : c;
+        DSt<T>::put(xbar + j * LS + p, LO, a * (1.f / L));
+        DSt<T>::put(xbar + j * LS + p + 1, LO, b * (1.f / L));
     }
 }
 
@@ -100,16 +103,8 @@ __device__ __forceinline__ void wide_output_tile(T* q0, const T* kbar, const T* 
     using D = typename O::DReg;
     constexpr int NTL = M / 8, KT = M / 16, NTO = NCOL / 8, LS = LmS<T>::LS, LO = LmS<T>::LO, YS = YtS<T, M>::YS,
                   YLO = YtS<T, M>::LO;
-    T* q1 = q0 + mrow<RS>() * d;
     R a[2][4];
-#pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-        const int c0 = 16 * kk + 2 * t, c1 = c0 + 8;
-        a[kk][0] = c0 < d ? O::ld(q0 + c0) : O::zero();
-        a[kk][1] = c0 < d ? O::ld(q1 + c0) : O::zero();
-        a[kk][2] = c1 < d ? O::ld(q0 + c1) : O::zero();
-        a[kk][3] = c1 < d ? O::ld(q1 + c1) : O::zero();
-    }
+    q_afrag<T, RS>(q0, d, t, a);
     float sl[NTL][4];
     float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
@@ -160,14 +155,7 @@ __device__ __forceinline__ void wide_output_tile(T* q0, const T* kbar, const T* 
         }
     const float i0 = __fdividef(1.f, __shfl_sync(0xffffffffu, d0, src));
     const float i1 = __fdividef(1.f, __shfl_sync(0xffffffffu, d1, src));
-#pragma unroll
-    for (int j = 0; j < NTO; ++j) {
-        const int c = 8 * j + 2 * t;
-        if (c < d) {
-            O::st2(q0 + c, o[j][0] * i0, o[j][1] * i0);
-            O::st2(q1 + c, o[j][2] * i1, o[j][3] * i1);
-        }
-    }
+    store_orows<T, NTO, RS>(q0, d, t, o, i0, i1);
 }
 
 template <typename T, int M, int NCOL, int N, int DC>
@@ -178,7 +166,7 @@ nystra_wide_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
     using Sc = typename Lay::Sc;
     constexpr int CW = Lay::CW, NTO = NCOL / 8;
     const int d = DC ? DC : d_in;
-    constexpr int RS = row_step(DC);
+    constexpr int RS = row_order<T>(DC);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int grp = warp / CW, c = warp - grp * CW;
@@ -233,8 +221,8 @@ nystra_wide_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
     for (; u < n_units; u += stride) {
         // ---------------- landmarks (Algorithm 1 step 1) ----------------
         wait(barQK);
-        wide_landmarks<T, M, N>(Qs, qbar, d, c * 32 + lane, CW * 32);
-        wide_landmarks<T, M, N>(Ks, kbar, d, c * 32 + lane, CW * 32);
+        wide_landmarks<T, M, N, RS>(Qs, qbar, d, c * 32 + lane, CW * 32);
+        wide_landmarks<T, M, N, RS>(Ks, kbar, d, c * 32 + lane, CW * 32);
         wait(barV);
         if (named_barrier_or(bar, CW * 32, failed)) break;
         pend = false;
