@@ -31,7 +31,7 @@
 // warps per SM, DRAM 5%), so chunks are as long as one score tile per thread
 // allows: chunks of 72 and 88 tokens with more CTAs per SM were 4-12% slower.
 // Measured: 6144 units of 16x16 windows, d_h = 30, m = 16, fp32 1.52 -> 0.62 ms
-// (1.2 TB/s of Q, K, V, O); 11094 units of 12x12, fp16 1.62 -> 0.74 ms; 1668
+// (1.2 TB/s of Q, K, V, O); 11094 units of 12x12, fp16 1.62 -> 0.76 ms; 1668
 // units of 16x16, d_h = 32, m = 32 with a score bias 3.94 -> 0.40 ms, against a
 // kernel with one shared load per operand and 32-token chunks.
 #pragma once
@@ -54,8 +54,8 @@ struct Bound {
     static_assert((MS / 4) % 2 == 1, "odd granules");
     // W's tiles (17 column groups at d_h = 64) may outnumber the score tiles
     static constexpr int kTiles = JG * 17 > CH / 4 * JG ? JG * 17 : CH / 4 * JG;
-    static constexpr int kThreads = (kTiles + 31) / 32 * 32;
-    static constexpr int kCtas = MP == 8 ? 5 : (MP == 16 ? 4 : (MP == 32 ? 2 : 1));
+    static constexpr int kThreads = kTiles > 128 ? (kTiles + 31) / 32 * 32 : 128;
+    static constexpr int kCtas = MP <= 16 ? 4 : (MP == 32 ? 2 : 1);
 };
 
 // Region sizes in floats for one call; DS: row stride of d_h columns.
@@ -66,7 +66,7 @@ struct Shape {
     int ns;                   // row stride of anything with token columns: odd granules
     int kv, p;
     static constexpr int kLm = MP * DS, kMat = MP * B::MS;
-    __host__ __device__ Shape(int N, int d) {
+    __host__ __device__ Shape(int N, int d, int min_threads) {
         const int chunks = (N + B::CH - 1) / B::CH;
         ch = 4 * ((N + 4 * chunks - 1) / (4 * chunks));
         ns = 4 * ((ch / 4) | 1);
@@ -74,6 +74,7 @@ struct Shape {
         const int tiles = B::JG * c4;
         threads = ch / 4 * B::JG;
         threads = ((threads > tiles ? threads : tiles) + 31) / 32 * 32;
+        threads = threads > min_threads ? threads : min_threads;
         ks = threads / tiles;
         if (ks > ch / 4) ks = ch / 4;
         kv = ch * DS;                                               // Q or K rows
@@ -169,8 +170,8 @@ __device__ __forceinline__ void run(const T* __restrict__ q, const T* __restrict
                                     float scale, const NystraBias& bias, float* sm) {
     using B = Bound<MP>;
     constexpr int JG = B::JG, MS = B::MS;
-    const Shape<MP, DS> G(N, d);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nth = blockDim.x, NW = nth >> 5;
+    const Shape<MP, DS> G(N, d, nth);
     const int ch = G.ch, ns = G.ns, c4 = G.c4, ks = G.ks, L = N / m, m4 = (m + 3) & ~3;
     const int kg = (d + 3) >> 2, pl = 4 * kg <= 16 ? 3 : (4 * kg <= 32 ? 4 : 5);
     float* KV = sm;                 // Q or K rows (DS), V^T (ns), W^T's splits, the core's matrices, O rows
@@ -469,7 +470,11 @@ cudaError_t launch_ds(const void* q, const void* k, const void* v, void* out, lo
     int pw = 0;  // window width for square patches
     if (pool != 0)
         while ((pw + 1) * (pw + 1) <= N) ++pw;
-    const Shape<MP, DS> G(N, d);
+    // Few units, a CTA or so per SM: at least four warps, for a unit's latency (108
+    // units of 7x7 windows, m = 7: 33 us with one warp, 22 with four); else the
+    // tiles' threads only, for more CTAs per SM.
+    constexpr long long kFewUnits = 4 * 152;
+    const Shape<MP, DS> G(N, d, n_units <= kFewUnits ? 128 : 32);
     const long long grid = n_units < (1LL << 30) ? n_units : (1LL << 30);
     kern<<<(unsigned)grid, G.threads, G.bytes(), stream>>>(q, k, v, out, n_units, N, d, m, iters, pw, dtype,
                                                            1.0f / sqrtf((float)d), bias);

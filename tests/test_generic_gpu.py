@@ -55,3 +55,18 @@ def test_generic_score_bias(N, d, m, per_window):
     ref = oracle.nystra_attention(q, k, v, m, 5, "segments", B.double().numpy() if per_window else B.double().numpy()[None])
     err = per_unit_rel(out.cpu().double().numpy(), ref)
     assert err.max() <= TOL["f32"], err
+
+
+@pytest.mark.parametrize("units", [608, 609])
+@pytest.mark.parametrize("N,d,m", [(5, 3, 5), (49, 30, 7), (36, 20, 4), (81, 16, 9)])
+def test_generic_few_and_many_units(N, d, m, units):
+    # up to 608 units a CTA has four warps at least, above only its tiles' threads
+    q, k, v = workloads.random_qkv(units, N, d, "f32", seed=N + d)
+    out = binding.nystra(q.cuda(), k.cuda(), v.cuda(), m, 5)
+    torch.cuda.synchronize()
+    at = [0, units // 2, units - 1]
+    q, k, v = q[at], k[at], v[at]
+    ref = oracle.nystra_attention(q, k, v, m, 5)
+    err = per_unit_rel(units_view(out[at].cpu()).double().numpy(), ref)
+    bar = np.maximum(4.0 * per_unit_rel(nystra_float32(q, k, v, m, 5), ref), 1e-6)  # as above
+    assert (err <= np.minimum(bar, TOL["f32"])).all(), f"{err} > {bar}"
