@@ -45,7 +45,7 @@ namespace tc {
 
 template <typename T, int M, int NCOL, bool PAIR>
 struct QkvLayout {
-    using PL = PoolLayout<T, M, NCOL>;
+    using PL = PoolLayout<T, M, NCOL, 4, false>;
     static constexpr size_t HDR = 128;               // the shared stages' mbarriers
     static constexpr size_t FRAG = 3 * 4 * 32 * 8;   // weight fragments per k-step: 3 blocks x 4 n-tiles x 32 lanes x 8 B
     // warps per CTA: 12 on 6 shared stages (C <= 64), else as many with a

@@ -836,13 +836,13 @@ __device__ __forceinline__ void qbar_afrag(const T* qbar, int mt, int g, int t, 
 // the row maxima (log2 domain) are returned in mU.
 // BIAS: bu is the unit's M x N block B_U of the score bias, offset to the
 // first key of Ks (row stride bn).
+// su_w_regs leaves W_r in registers (wall), store_w stores it.
 template <typename T, int M, int NCOL, int NCH, bool BIAS = false, int RS = 1>
-__device__ __forceinline__ void front_su_w(const T* qbar, const T* Ks, const T* Vs, int d, int g, int t, float sl2,
-                                           float* dst, int ws, float (&mU)[(M + 15) / 16][2],
-                                           const float* bu = nullptr, int bn = 0) {
+__device__ __forceinline__ void su_w_regs(const T* qbar, const T* Ks, const T* Vs, int d, int g, int t, float sl2,
+                                          float (&wall)[(M + 15) / 16][NCOL / 8][4], float (&mU)[(M + 15) / 16][2],
+                                          const float* bu = nullptr, int bn = 0) {
     using R = typename Opnd<T>::DReg;
     constexpr int MT = (M + 15) / 16, NTO = NCOL / 8;
-    float wall[MT][NTO][4];
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt) {
         R aq[2][4];
@@ -859,7 +859,9 @@ __device__ __forceinline__ void front_su_w(const T* qbar, const T* Ks, const T* 
         mU[mt][0] = run0;
         mU[mt][1] = run1;
     }
-    __syncwarp();
+}
+template <int MT, int NTO>
+__device__ __forceinline__ void store_w(const float (&wall)[MT][NTO][4], float* dst, int ws, int g, int t) {
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
@@ -868,6 +870,15 @@ __device__ __forceinline__ void front_su_w(const T* qbar, const T* Ks, const T* 
             *reinterpret_cast<float2*>(dst + rr * ws + c) = make_float2(wall[mt][j][0], wall[mt][j][1]);
             *reinterpret_cast<float2*>(dst + (rr + 8) * ws + c) = make_float2(wall[mt][j][2], wall[mt][j][3]);
         }
+}
+template <typename T, int M, int NCOL, int NCH, bool BIAS = false, int RS = 1>
+__device__ __forceinline__ void front_su_w(const T* qbar, const T* Ks, const T* Vs, int d, int g, int t, float sl2,
+                                           float* dst, int ws, float (&mU)[(M + 15) / 16][2],
+                                           const float* bu = nullptr, int bn = 0) {
+    float wall[(M + 15) / 16][NCOL / 8][4];
+    su_w_regs<T, M, NCOL, NCH, BIAS, RS>(qbar, Ks, Vs, d, g, t, sl2, wall, mU, bu, bn);
+    __syncwarp();
+    store_w(wall, dst, ws, g, t);
 }
 
 // Combine (several warps per unit): the warps' partial (W_r, m_r), stored in
@@ -912,10 +923,15 @@ __device__ __forceinline__ void combine_partials(const float* part0, size_t wstr
 // DUMP (test-only stage dump): dbg receives G_A^n (M x M), Z (M x M) and
 // Y = Z W (M x NCOL), row-major fp32, with the dropped factors restored.
 // BIAS: ba is the unit's M x M block B_A of the score bias.
-template <typename T, int M, int NCOL, bool DUMP = false, bool BIAS = false>
+// landmarks_read is called once this lane has read Qbar and Kbar for the last
+// time: a caller may put W over them there (mW is read after the iteration).
+struct NoStep {
+    __device__ __forceinline__ void operator()() const {}
+};
+template <typename T, int M, int NCOL, bool DUMP = false, bool BIAS = false, typename F = NoStep>
 __device__ __forceinline__ void core_warp(const T* qbar, const T* kbar, const float (&mU)[(M + 15) / 16][2],
                                           const float* mW, T* yT, int iters, float sl2, int g, int t,
-                                          float* dbg = nullptr, const float* ba = nullptr) {
+                                          float* dbg = nullptr, const float* ba = nullptr, F landmarks_read = F()) {
     using O = Opnd<T>;
     using D = typename O::DReg;
     constexpr int MT = (M + 15) / 16, LS = LmS<T>::LS, LO = LmS<T>::LO, WS = NCOL + 4, NTO = NCOL / 8;
@@ -966,6 +982,7 @@ __device__ __forceinline__ void core_warp(const T* qbar, const T* kbar, const fl
                 }
             }
         }
+        landmarks_read();
         // 2^ea G_A^n with its largest entry in [2^10, 2^11): the shift enters
         // the exponent, so no entry underflows for being small in absolute
         // terms (sharp attention can put a whole row of G_A^n far below 1).
@@ -1207,7 +1224,12 @@ __device__ __forceinline__ void store_orows(T* o0, int d, int t, const float (&o
 // (tiles in the RS token order of the chunks).
 // BIAS (recomputed G_L^n only): bl is B_L of the score bias at the warp's
 // first token (row stride M).
-template <typename T, int M, int NCOL, int NCH, bool GLS, bool BIAS = false, int RS = 1>
+// OVER (parked G_L^n, one chunk): obase is glf itself and what follows it, Y^T
+// too.  Y^T is read first; two tiles' rows lie within 64 d values of 16 bits,
+// so with parked fragments of 1 KB a tile they only reach fragments of their own
+// two tiles, which are then read before either is stored; smaller ones are all
+// read first.
+template <typename T, int M, int NCOL, int NCH, bool GLS, bool BIAS = false, int RS = 1, bool OVER = false>
 __device__ __forceinline__ void output_rows(const uint32_t* glf, const T* Qs, const T* kbar, const T* yT,
                                             T* obase, int d, int g, int t, int lane, float sl2,
                                             const float* bl = nullptr) {
@@ -1225,12 +1247,23 @@ __device__ __forceinline__ void output_rows(const uint32_t* glf, const T* Qs, co
         }
     const int jd = d >> 3, tdn = (d & 7) >> 1;
     const int src = (lane & ~3) | tdn;
+    static_assert(!OVER || (GLS && NCH == 1 && KTL == 1), "parked fragments of one chunk");
+    constexpr int NF = !OVER ? 1 : (sizeof(T) == 2 && GlPark<T, M>::BYTES == 32 ? 2 : 4);  // tiles read ahead
+    R fo[NF][4];
 #pragma unroll 1
     for (int ch = 0; ch < NCH; ++ch)
 #pragma unroll
         for (int tm = 0; tm < 4; ++tm) {
             R f[KTL][4];
-            if constexpr (GLS) {
+            if constexpr (OVER) {
+                if (tm % NF == 0) {
+#pragma unroll
+                    for (int i = 0; i < NF; ++i) GlPark<T, M>::get(glf, (tm + i) * 32 + lane, fo[i]);
+                    __syncwarp();
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) f[0][i] = fo[tm % NF][i];
+            } else if constexpr (GLS) {
 #pragma unroll
                 for (int kk = 0; kk < KTL; ++kk) GlPark<T, M>::get(glf, ((ch * 4 + tm) * KTL + kk) * 32 + lane, f[kk]);
             } else {
