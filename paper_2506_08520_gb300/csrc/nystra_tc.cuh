@@ -712,9 +712,11 @@ __device__ __forceinline__ void su_w_chunk(const typename Opnd<T>::DReg (&aq)[2]
     // those of four n-tiles are eight consecutive keys: two 16-byte loads.  With 32
     // 4-byte loads after the products instead, the bias cost 103 us on 21600
     // units of 16x16 windows (421 against 318 us); so it costs 43 (360).
+    // In token order (RS = 1, d_h read at run time) they are loaded after the products,
+    // for want of registers: 6144 units of 8x8 windows, d_h = 24, 44.3 us before, 42.9
+    // after them; 1800 of 32x32 139 and 136, 6144 of 16x16 119 and 122.
     float2 b0[BIAS ? 8 : 1], b1[BIAS ? 8 : 1];
-    if constexpr (BIAS) {
-        auto load = [&](const float* p, bool real, float2(&b)[8]) {
+    auto load = [&](const float* p, bool real, float2(&b)[BIAS ? 8 : 1]) {
             if constexpr (RS == 4) {
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
@@ -737,6 +739,7 @@ __device__ __forceinline__ void su_w_chunk(const typename Opnd<T>::DReg (&aq)[2]
                 }
             }
         };
+    if constexpr (BIAS && RS != 1) {
         load(bu, v0, b0);
         load(bu + 8 * bn, v1, b1);
     }
@@ -758,6 +761,10 @@ __device__ __forceinline__ void su_w_chunk(const typename Opnd<T>::DReg (&aq)[2]
                 else O::mma(s[nt], aq[kk], b0, b1);
             }
         }
+    }
+    if constexpr (BIAS && RS == 1) {
+        load(bu, v0, b0);
+        load(bu + 8 * bn, v1, b1);
     }
     if constexpr (BIAS) {  // scores in the log2 domain, bias included (rows beyond m stay unbiased)
 #pragma unroll
