@@ -74,9 +74,9 @@ struct Shape {
         const int tiles = B::JG * c4;
         threads = ch / 4 * B::JG;
         threads = ((threads > tiles ? threads : tiles) + 31) / 32 * 32;
-        threads = threads > min_threads ? threads : min_threads;
-        ks = threads / tiles;
+        ks = threads / tiles;  // (before min_threads: a unit's sums do not depend on how many units there are)
         if (ks > ch / 4) ks = ch / 4;
+        threads = threads > min_threads ? threads : min_threads;
         kv = ch * DS;                                               // Q or K rows
         if (4 * c4 * ns > kv) kv = 4 * c4 * ns;                     // V^T
         if (ks * 4 * c4 * B::MS > kv) kv = ks * 4 * c4 * B::MS;     // W^T's splits

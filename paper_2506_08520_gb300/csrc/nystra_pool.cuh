@@ -49,10 +49,12 @@ struct PoolLayout {
     static constexpr size_t QB = GLF + 4 * KTL * 32 * GlPark<T, M>::BYTES;
     static constexpr size_t KB = QB + LmS<T>::bytes(MP);
     static constexpr size_t END_L = KB + LmS<T>::bytes(MP);
-    static constexpr size_t W = OVER ? QB : END_L;  // fp32 MP x NCOL, row stride WS: OVER, stored after the last landmark read
-    static constexpr size_t YT = QB;                // Y^T: written after the last read of landmarks and W
+    // W (fp32 MP x NCOL, row stride WS; OVER: stored after the last landmark read)
+    static constexpr size_t W = OVER ? QB : END_L;
+    static constexpr size_t YT = QB;  // Y^T: written after the last read of landmarks and W
     static constexpr size_t END_Y = YT + YtS<T, M>::bytes(NCOL);
-    static constexpr size_t OUT = OVER ? GLF : END_Y;  // output tile: OVER, written after the reads of Y^T and fragments
+    // output tile (OVER: written after the reads of Y^T and fragments)
+    static constexpr size_t OUT = OVER ? GLF : END_Y;
     static constexpr size_t END_W = W + MP * WS * 4, END_O = OUT + 64 * DS * ES;
     static constexpr size_t max2(size_t a, size_t b) { return a > b ? a : b; }
     static constexpr size_t BAR = (max2(max2(END_L, END_W), max2(END_Y, END_O)) + 15) / 16 * 16;
@@ -239,7 +241,8 @@ cudaError_t launch_pool(const void* q, const void* k, const void* v, void* out, 
         if constexpr (sizeof(T) == 2) {  // (fp32 I/O: d_h read at run time)
             constexpr int kDc = NCOL == 32 ? 30 : 32;
             if (d == kDc)
-                return launch_pool_dc<T, M, NCOL, kDc, PW, true>(q, k, v, out, n_units, d, iters, stream, fault, *bias);
+                return launch_pool_dc<T, M, NCOL, kDc, PW, true>(q, k, v, out, n_units, d, iters, stream, fault,
+                                                                 *bias);
         }
         return launch_pool_dc<T, M, NCOL, 0, PW, true>(q, k, v, out, n_units, d, iters, stream, fault, *bias);
     }

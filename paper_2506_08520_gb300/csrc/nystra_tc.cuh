@@ -717,28 +717,28 @@ __device__ __forceinline__ void su_w_chunk(const typename Opnd<T>::DReg (&aq)[2]
     // after them; 1800 of 32x32 139 and 136, 6144 of 16x16 119 and 122.
     float2 b0[BIAS ? 8 : 1], b1[BIAS ? 8 : 1];
     auto load = [&](const float* p, bool real, float2(&b)[BIAS ? 8 : 1]) {
-            if constexpr (RS == 4) {
+        if constexpr (RS == 4) {
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-                    const float4 x = real ? __ldg(reinterpret_cast<const float4*>(p + 32 * q + 8 * t)) : z;
-                    const float4 y = real ? __ldg(reinterpret_cast<const float4*>(p + 32 * q + 8 * t + 4)) : z;
-                    b[4 * q] = make_float2(x.x, y.x);
-                    b[4 * q + 1] = make_float2(x.y, y.y);
-                    b[4 * q + 2] = make_float2(x.z, y.z);
-                    b[4 * q + 3] = make_float2(x.w, y.w);
-                }
-            } else {
-#pragma unroll
-                for (int nt = 0; nt < 8; ++nt) {
-                    if constexpr (RS == 1 || RS == kSlots)
-                        b[nt] = real ? __ldg(reinterpret_cast<const float2*>(p + 8 * nt + 2 * t)) : make_float2(0.f, 0.f);
-                    else
-                        b[nt] = real ? make_float2(__ldg(p + ctok<RS>(nt, 2 * t)), __ldg(p + ctok<RS>(nt, 2 * t + 1)))
-                                     : make_float2(0.f, 0.f);
-                }
+            for (int q = 0; q < 2; ++q) {
+                const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                const float4 x = real ? __ldg(reinterpret_cast<const float4*>(p + 32 * q + 8 * t)) : z;
+                const float4 y = real ? __ldg(reinterpret_cast<const float4*>(p + 32 * q + 8 * t + 4)) : z;
+                b[4 * q] = make_float2(x.x, y.x);
+                b[4 * q + 1] = make_float2(x.y, y.y);
+                b[4 * q + 2] = make_float2(x.z, y.z);
+                b[4 * q + 3] = make_float2(x.w, y.w);
             }
-        };
+        } else {
+#pragma unroll
+            for (int nt = 0; nt < 8; ++nt) {
+                if constexpr (RS == 1 || RS == kSlots)
+                    b[nt] = real ? __ldg(reinterpret_cast<const float2*>(p + 8 * nt + 2 * t)) : make_float2(0.f, 0.f);
+                else
+                    b[nt] = real ? make_float2(__ldg(p + ctok<RS>(nt, 2 * t)), __ldg(p + ctok<RS>(nt, 2 * t + 1)))
+                                 : make_float2(0.f, 0.f);
+            }
+        }
+    };
     if constexpr (BIAS && RS != 1) {
         load(bu, v0, b0);
         load(bu + 8 * bn, v1, b1);
