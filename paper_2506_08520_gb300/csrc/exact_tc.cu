@@ -9,12 +9,14 @@
 // they lie in HBM, take a 4-byte load and, for V, an 8x8 transpose per
 // register, with two-way conflicts).  Warp r computes output rows 64r .. 64r +
 // 63, 32 at a time so that a fragment serves two 16-row tiles, streaming the
-// keys in chunks of 32 with the online (running-max) softmax: S = Q K_c^T
+// keys in chunks of 64 with the online (running-max) softmax: S = Q K_c^T
 // (mma.sync, fp32 accumulate), P = exp(S - m) in registers fed directly as the
 // A operand of P [V_c | 1], whose last column accumulates the row sums of the
-// same rounded P.  Scores are scaled by log2(e)/sqrt(d_h) so each exponential
-// is half a packed FMA and one ex2.  This is the computation PnP-Nystra
-// replaces; it is the in-library comparator.
+// same rounded P.  P is rounded to 16 bits relative to the maximum so far, so
+// the chunk length is part of the result (32 keys at a time move it by 1.4e-3
+// in bf16, at the same distance of 2.1e-3 from float64).  Scores are scaled by
+// log2(e)/sqrt(d_h) so each exponential is half a packed FMA and one ex2.  This
+// is the computation PnP-Nystra replaces; it is the in-library comparator.
 //
 // What bounds it: at 32x32 windows the tensor pipe, 69% busy (32 MMAs and 32
 // ex2 per warp for 32 rows and 32 keys); at 16x16 windows also laying out K and
@@ -36,9 +38,11 @@ template <typename T>
 struct ExactOp {  // 16-bit I/O: one plane
     using E = T;
     static constexpr int NP = 1;
-    // per SM, with two key chunks unrolled: at N = 64 twelve warps of up to 168
-    // registers beat sixteen (86400 units: 253 against 267 us), elsewhere not
-    static constexpr int warps(int wpu) { return wpu == 1 ? 12 : 16; }
+    // per SM: the scores of 32 rows and 64 keys take twelve warps' registers
+    // (160 of up to 168; 128 of sixteen warps spill up to 156 bytes: 6144 units of
+    // 16x16 windows 201 us, d_h = 32 240, against 179 and 192); the sixteen warps
+    // of a 32x32 window have 128
+    static constexpr int warps(int wpu) { return wpu <= 4 ? 12 : 16; }
 };
 template <>
 struct ExactOp<float> {
@@ -183,10 +187,10 @@ exact_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
                 for (int j = 0; j < NTO; ++j) o[mt][j][0] = o[mt][j][1] = o[mt][j][2] = o[mt][j][3] = 0.f;
             }
 #pragma unroll 2
-            for (int c = 0; c < N; c += 32) {
-                float s[2][4][4];
+            for (int c = 0; c < N; c += 64) {
+                float s[2][8][4];
 #pragma unroll
-                for (int nt = 0; nt < 4; ++nt) {
+                for (int nt = 0; nt < 8; ++nt) {
                     R b[4];
                     ld_frag<false>(b, kf + (c + 8 * nt) * kRow * 2, PL);
 #pragma unroll
@@ -202,7 +206,7 @@ exact_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
                     for (int e = 0; e < 2; ++e) {
                         float m = fmaxf(s[mt][0][2 * e], s[mt][0][2 * e + 1]);
 #pragma unroll
-                        for (int nt = 1; nt < 4; ++nt) m = fmaxf(m, fmaxf(s[mt][nt][2 * e], s[mt][nt][2 * e + 1]));
+                        for (int nt = 1; nt < 8; ++nt) m = fmaxf(m, fmaxf(s[mt][nt][2 * e], s[mt][nt][2 * e + 1]));
                         m = fmaxf(run[mt][e], quad_max(m) * sl2);
                         const float f = ex2(run[mt][e] - m);
                         run[mt][e] = m;
@@ -210,7 +214,7 @@ exact_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
                         for (int j = 0; j < NTO; ++j) mul_x2(o[mt][j][2 * e], o[mt][j][2 * e + 1], f);
                     }
 #pragma unroll
-                for (int kt = 0; kt < 2; ++kt) {
+                for (int kt = 0; kt < 4; ++kt) {
                     R a[2][4];
 #pragma unroll
                     for (int mt = 0; mt < 2; ++mt)

@@ -58,3 +58,32 @@ def test_generic_tile_edges(units, N, d, dtype):
     q, k, v = workloads.random_qkv(units, N, d, dtype, seed=units + N + d)
     # fp32 throughout: a few ulp of the longest sums (2^-24 x sqrt(1024) = 2e-6)
     _check(q, k, v, 2e-6 if dtype == "f32" else TOL[dtype])
+
+
+def _rounded_p(q, k, v, chunk):
+    """Eq. 1 with the online softmax over chunks of keys: float64 but for P,
+    rounded to the I/O type relative to the running maximum, and the result."""
+    T = q.dtype
+    q, k, v = q.double(), k.double(), v.double()
+    N, d = q.shape[1:]
+    s = torch.einsum("utd,ukd->utk", q, k) * (1.4426950408889634 / d ** 0.5)
+    run = torch.full(s.shape[:2] + (1,), -float("inf"), dtype=torch.float64)
+    num, den = torch.zeros_like(q), torch.zeros_like(run)
+    for c in range(0, N, chunk):
+        m = torch.maximum(run, s[..., c:c + chunk].amax(-1, keepdim=True))
+        f, p = torch.exp2(run - m), torch.exp2(s[..., c:c + chunk] - m).to(T).double()
+        num, den, run = num * f + p @ v[:, c:c + chunk], den * f + p.sum(-1, keepdim=True), m
+    return (num / den).to(T).double()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("units,N,d", [(6, 256, 30), (6, 256, 32), (6, 256, 18), (2, 1024, 30), (2, 1024, 32), (2, 1024, 8)])
+def test_probabilities_are_rounded_at_the_maxima_of_64_keys(units, N, d, dtype):
+    # another chunk length rounds other values: the results lie some 2^-9 apart in
+    # bf16, 2^-12 in fp16, and fp32 sums and ex2 move at most a quarter of that
+    # (fp16, 1024 keys: a relative 2^-22 of P moves one value in 500 to its
+    # neighbour).  Within half of it, the output belongs to the one and not the other
+    q, k, v = workloads.random_qkv(units, N, d, dtype, seed=N + d)
+    out = units_view(binding.exact(q.cuda(), k.cuda(), v.cuda()).cpu()).double()
+    ref, other = _rounded_p(q, k, v, 64), _rounded_p(q, k, v, 32)
+    assert (out - ref).norm() <= 0.5 * (other - ref).norm()
