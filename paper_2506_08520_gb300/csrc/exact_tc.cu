@@ -22,11 +22,13 @@
 // ex2 per warp for 32 rows and 32 keys); at 16x16 windows also laying out K and
 // V, at 8x8 windows HBM.  The next unit's rows are brought to L2 meanwhile.
 // Measured (d_h = 30, bf16) against fragments loaded from 60-byte rows by one
-// 16-row tile: 5520 units of 32x32 windows 3.33 -> 1.98 ms, 6144 of 16x16
-// 0.27 -> 0.19 ms, 86400 of 8x8 266 -> 253 us; fp32, 2000 units of 16x16: 0.50 ->
-// 0.16 ms.
+// 16-row tile: 5520 units of 32x32 windows 3.34 -> 2.02 ms, 6144 of 16x16
+// 271 -> 176 us, 86400 of 8x8 269 -> 224 us; fp32, 2000 units of 16x16: 502 ->
+// 163 us.
 #include "common.cuh"
 #include "ptx.cuh"
+
+#include <type_traits>
 
 namespace nystra {
 namespace {
@@ -41,23 +43,26 @@ struct ExactOp {  // 16-bit I/O: one plane
     // per SM: the scores of 32 rows and 64 keys take twelve warps' registers
     // (160 of up to 168; 128 of sixteen warps spill up to 156 bytes: 6144 units of
     // 16x16 windows 201 us, d_h = 32 240, against 179 and 192); the sixteen warps
-    // of a 32x32 window have 128
-    static constexpr int warps(int wpu) { return wpu <= 4 ? 12 : 16; }
+    // of a 32x32 window have 128, and at 8x8 windows with d_h read at run time
+    // sixteen (124 registers) are faster, laying out K and V being most of the work
+    // (40000 units, d_h = 24, 103 against 117 us; d_h = 30, compiled in, 267 against 220
+    // with twelve for 86400 units)
+    static constexpr int warps(int wpu, int dc) { return wpu == 16 || (wpu == 1 && dc == 0) ? 16 : 12; }
 };
 template <>
 struct ExactOp<float> {
     using E = __nv_bfloat16;
     static constexpr int NP = 2;
-    static constexpr int warps(int) { return 8; }
+    static constexpr int warps(int, int) { return 8; }
 };
 
-template <typename T, int WPU>
+template <typename T, int WPU, int DC>
 struct ExactLayout {
     static constexpr int N = 64 * WPU;
     static constexpr size_t PLANE = (size_t)N * kRow * 2;
     static constexpr size_t GROUP = 2 * ExactOp<T>::NP * PLANE;  // K, then V
     static constexpr int by_smem = (int)(kSmemLimit / GROUP);
-    static constexpr int by_warps = ExactOp<T>::warps(WPU) / WPU;
+    static constexpr int by_warps = ExactOp<T>::warps(WPU, DC) / WPU;
     static constexpr int GROUPS = by_smem < by_warps ? by_smem : by_warps;
     static_assert(GROUPS >= 1, "does not fit");
 };
@@ -97,13 +102,14 @@ __device__ __forceinline__ void ld_frag(RegPair (&r)[4], const unsigned char* p,
 }
 
 template <typename T, int NCOL, int WPU, int DC>
-__global__ void __launch_bounds__(ExactLayout<T, WPU>::GROUPS * WPU * 32, 1)
+__global__ void __launch_bounds__(ExactLayout<T, WPU, DC>::GROUPS * WPU * 32, 1)
 exact_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ out,
                 long long n_units, int d_in, float sl2) {
-    using Lay = ExactLayout<T, WPU>;
+    using Lay = ExactLayout<T, WPU, DC>;
     using O = Opnd<T>;
     using R = typename O::Reg;
-    constexpr int N = Lay::N, NTO = NCOL / 8, GROUPS = Lay::GROUPS;
+    constexpr int N = Lay::N, NTO = NCOL / 8;
+    const int groups = blockDim.x / (WPU * 32);
     constexpr size_t PL = Lay::PLANE;
     const int d = DC ? DC : d_in, h = d >> 1;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -116,22 +122,26 @@ exact_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
         if constexpr (WPU == 1) __syncwarp();
         else named_barrier(1 + grp, WPU * 32);
     };
-    // columns d .. 31: zeros, in V a ones column first (d = 32 has it as a constant fragment)
-    for (int i = id; i < N * (kRow / 2 - h); i += WPU * 32) {
-        const int row = i / (kRow / 2 - h), c = h + i - row * (kRow / 2 - h);
-        st_plane(Ks + (row * kRow + 2 * c) * 2, PL, O::zero());
-        st_plane(Vs + (row * kRow + 2 * c) * 2, PL, c == h ? O::one() : O::zero());
-    }
+    // columns d .. 31: zeros, in V a ones column first (d = 32 has it as a constant
+    // fragment); the columns from 32 on are never read
+    for (int row = id; row < N; row += WPU * 32)
+        for (int c = h; c < 16; ++c) {
+            st_plane(Ks + (row * kRow + 2 * c) * 2, PL, O::zero());
+            st_plane(Vs + (row * kRow + 2 * c) * 2, PL, c == h ? O::one() : O::zero());
+        }
     // fragment addresses: rows 8 (lane / 8) .. of an ldmatrix x4
     const unsigned char* kf = Ks + ((lane & 7) * kRow + 8 * (lane >> 3)) * 2;                              // 8 keys x 32
     const unsigned char* vf = Vs + (((lane & 7) + 8 * ((lane >> 3) & 1)) * kRow + 8 * (lane >> 4)) * 2;  // 16 keys x 16
     R one0;  // B fragment of the ones column at d = 32: column 0 (lanes g = 0) is 1
     if constexpr (NCOL > 32) one0 = g == 0 ? O::pk(1.f, 1.f) : O::zero();
+    // i / h for i < 2^14 and 2 <= h <= 16 (2^32 / h rounded up errs by less than i h / 2^32 < 1 / h)
+    const uint32_t magic = DC ? 0u : 0xffffffffu / (uint32_t)h + 1u;
+    auto row_of = [&](int i) { return DC ? i / h : h == 1 ? i : (int)__umulhi((uint32_t)i, magic); };
     const int jd = d >> 3, src = (lane & ~3) | ((d & 7) >> 1);
 
-    for (long long u = (long long)blockIdx.x * GROUPS + grp; u < n_units; u += (long long)gridDim.x * GROUPS) {
+    for (long long u = (long long)blockIdx.x * groups + grp; u < n_units; u += (long long)gridDim.x * groups) {
         const size_t base = (size_t)u * N * d;
-        const long long un = u + (long long)gridDim.x * GROUPS;
+        const long long un = u + (long long)gridDim.x * groups;
         if (id == 0 && un < n_units) {  // the next unit's rows on their way to L2
             const size_t nb = (size_t)un * N * d;
             const uint32_t bytes = (uint32_t)(N * d * sizeof(T));
@@ -140,11 +150,12 @@ exact_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
             bulk_prefetch_l2(q + nb, bytes);
         }
         gsync();  // every warp is done with the previous unit's K and V
-        {
-            // four elements (two words) a load; word i of the unit belongs to row i / h, 20 words long here
+        // four elements (two words) a load, U loads in flight; word i of the unit
+        // belongs to row i / h, 20 words long here
+        auto stage = [&](auto batch) {
+            constexpr int U = decltype(batch)::value;
             const T* ku = k + base;
             const T* vu = v + base;
-            constexpr int U = 4;
             const int n = N * h / 2;
             for (int i0 = id; i0 < n; i0 += U * WPU * 32) {
                 decltype(ld_global4(ku)) x[U], y[U];
@@ -157,14 +168,24 @@ exact_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
 #pragma unroll
                 for (int e = 0; e < U; ++e) {
                     const int i = 2 * min(i0 + e * WPU * 32, n - 1);  // the last words may be written twice
-                    const int a0 = 4 * i + (i / h) * (2 * kRow - 4 * h), a1 = 4 * (i + 1) + ((i + 1) / h) * (2 * kRow - 4 * h);
+                    const int a0 = 4 * i + row_of(i) * (2 * kRow - 4 * h), a1 = 4 * (i + 1) + row_of(i + 1) * (2 * kRow - 4 * h);
                     st_plane(Ks + a0, PL, word(x[e], 0));
                     st_plane(Ks + a1, PL, word(x[e], 1));
                     st_plane(Vs + a0, PL, word(y[e], 0));
                     st_plane(Vs + a1, PL, word(y[e], 1));
                 }
             }
-        }
+        };
+        // One warp makes h such loads per tensor and lane: all in one go where d_h is
+        // compiled in (86400 units, d_h = 30, 245 -> 222 us), else in batches with little
+        // over, as lanes beyond the end repeat its last words (40000 units, four at a
+        // time, eight, twelve: d_h = 24, 121, 108 and 103 us; 28, 134, 118 and 126).
+        // Four warps: eight at a time (6144 units, 178 -> 173 us), fp32 four (2000 units,
+        // 163 us, eight 180).
+        if constexpr (WPU > 1) stage(std::integral_constant<int, WPU == 4 && sizeof(T) == 2 ? 8 : 4>());
+        else if constexpr (DC != 0) stage(std::integral_constant<int, 16>());
+        else if (h > 8 && h <= 12) stage(std::integral_constant<int, 12>());
+        else stage(std::integral_constant<int, 8>());
         gsync();
 #pragma unroll 1
         for (int blk = 0; blk < 2; ++blk) {
@@ -186,7 +207,10 @@ exact_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
 #pragma unroll
                 for (int j = 0; j < NTO; ++j) o[mt][j][0] = o[mt][j][1] = o[mt][j][2] = o[mt][j][3] = 0.f;
             }
-#pragma unroll 2
+            // two chunks in a loop body where registers allow (5520 units of 32x32 windows
+            // 2.09 -> 2.02 ms; fp32 would spill: 163 -> 184 us)
+            constexpr int CU = ExactOp<T>::NP == 1 ? 2 : 1;
+#pragma unroll CU
             for (int c = 0; c < N; c += 64) {
                 float s[2][8][4];
 #pragma unroll
@@ -271,17 +295,23 @@ exact_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
 template <typename T, int NCOL, int WPU, int DC>
 cudaError_t launch_dc(const void* q, const void* k, const void* v, void* out, long long n_units, int d,
                       cudaStream_t stream) {
-    using Lay = ExactLayout<T, WPU>;
+    using Lay = ExactLayout<T, WPU, DC>;
     constexpr int kThreads = Lay::GROUPS * WPU * 32;
     auto kern = exact_tc_kernel<T, NCOL, WPU, DC>;
     const size_t smem = (size_t)Lay::GROUPS * Lay::GROUP;
     static std::atomic<int> s_blocks[kMaxDevices];  // persistent grid size per device
     int blocks = 0;
     if (cudaError_t e = persistent_grid(kern, kThreads, smem, s_blocks, &blocks); e != cudaSuccess) return e;
-    const long long want = (n_units + Lay::GROUPS - 1) / Lay::GROUPS;
+    // the fewest groups per CTA that still reach the minimal number of rounds: few
+    // units spread over the SMs (384 units of 8x8 windows, d_h = 30, 7.2 -> 3.9 us; 6 of
+    // 16x16 13.6 -> 6.6) and more of them share an SM no longer than needed
+    const long long rounds = (n_units + blocks * Lay::GROUPS - 1) / (blocks * Lay::GROUPS);
+    const long long groups = (n_units + blocks * rounds - 1) / (blocks * rounds);
+    const long long want = (n_units + groups - 1) / groups;
     const long long grid = want < blocks ? want : blocks;
     const float sl2 = 1.4426950408889634f / sqrtf((float)d);
-    kern<<<(unsigned)grid, kThreads, smem, stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)out, n_units, d, sl2);
+    kern<<<(unsigned)grid, (unsigned)(groups * WPU * 32), (size_t)groups * Lay::GROUP, stream>>>(
+        (const T*)q, (const T*)k, (const T*)v, (T*)out, n_units, d, sl2);
     return cudaGetLastError();
 }
 

@@ -37,6 +37,16 @@ def test_units_and_widths(units, N, d, dtype):
     _check(q, k, v, TOL[dtype])
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("d", range(2, 33, 2))
+def test_every_head_width(d, dtype):
+    # rows of d / 2 words laid out in batches, d read at run time but for 30 and 32;
+    # one group per CTA, and (457 units) up to four, the last one idle in some
+    for units, N in ((5, 64), (457, 64), (2, 256)):
+        q, k, v = workloads.random_qkv(units, N, d, dtype, seed=units + N + d)
+        _check(q, k, v, TOL[dtype])
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
 @pytest.mark.parametrize("N", [64, 256])
 def test_late_maximum(N, dtype):
