@@ -370,7 +370,7 @@ def _two_pass(nw, N, heads, d, m, iters, landmarks, x, w_qkv, b_qkv, pooled, bw,
             or (N == 64 and C >= 80 and T >= 65536)):
         return False
     inputs = (x, w_qkv, b_qkv) + (tuple(pooled) if pooled is not None else ())
-    return (x.dtype in (torch.bfloat16, torch.float16)
+    return (nw > 0 and x.dtype in (torch.bfloat16, torch.float16)
             and (stream is None or isinstance(stream, torch.cuda.Stream))
             and d % 2 == 0 and 2 <= d <= 32 and heads * d <= QKV_MAX_C and 0 <= iters <= 12
             and (m in (8, 16) or (m == 32 and N == 1024 and pooled is None)) and (landmarks == "segments" or m == 16)

@@ -297,3 +297,14 @@ def test_valid_calls_without_an_sm103_device_return_edevice(lib):
     assert nb.nystra_debug_stages(P, 2 * P, 3 * P, 4, 2, 64, 30, 16, 6, 0, 1, 0, 4 * P, None) == nb.NYSTRA_EDEVICE
     assert nb.lib().nystra_debug_wait_timeout(10_000, None) == nb.NYSTRA_EDEVICE
     assert nb.strerror(nb.NYSTRA_EDEVICE) == "unsupported device (sm_103 required)"
+
+
+@pytest.mark.parametrize("N", [64, 256, 1024])
+@pytest.mark.parametrize("heads,d", [(1, 32), (6, 30)])
+def test_an_empty_batch_has_no_second_form(N, heads, d):
+    # nystra_qkv without windows goes to the C entry, which does nothing
+    import torch
+    x = torch.zeros(0, N, heads * d, dtype=torch.bfloat16)
+    w = torch.zeros(3 * heads * d, heads * d, dtype=torch.bfloat16)
+    out = torch.zeros(0, heads, N, d, dtype=torch.bfloat16)
+    assert not nb._two_pass(0, N, heads, d, 16, 6, "segments", x, w, None, None, 0, out, None)

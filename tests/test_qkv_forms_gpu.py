@@ -84,6 +84,19 @@ def test_what_was_refused_stays_refused():
     assert binding.status() == binding.NYSTRA_OK
 
 
+@pytest.mark.parametrize("N,heads,d", [(64, 6, 30), (256, 1, 32), (256, 6, 30), (1024, 1, 16), (1024, 6, 30)])
+@pytest.mark.parametrize("kind", [None, "heads", "windows"])
+def test_no_windows_is_a_no_op(N, heads, d, kind):
+    x, w, b = (t.cuda() for t in workloads.random_x_wqkv(1, N, heads, d, "bf16", seed=N))
+    pooled = None
+    if kind is not None:
+        lead = (heads,) if kind == "heads" else (0, heads)
+        pooled = tuple(torch.zeros(lead + s, device="cuda") for s in ((N, 16), (16, N), (16, 16)))
+    out = binding.nystra_qkv(x[:0], w, heads, 16, 6, b_qkv=b, pooled=pooled)
+    torch.cuda.synchronize()
+    assert out.shape == (0, heads, N, d) and binding.status() == binding.NYSTRA_OK
+
+
 def test_without_memory_and_under_capture(monkeypatch):
     x, w, b = (t.cuda() for t in workloads.random_x_wqkv(6, 1024, 2, 32, "bf16", seed=2))
     ref = binding.nystra_qkv(x, w, 2, 16, 6, b_qkv=b)
