@@ -300,7 +300,9 @@ def nystra_qkv(x: torch.Tensor, w_qkv: torch.Tensor, heads: int, m: int = 16, it
     ``nystra_biased``).  Returns ``[n_windows, heads, N, C / heads]``.  Runs as
     one fused kernel (nystra_attention_qkv) or, where that is faster, as the
     projection and the attention by turns over a workspace of up to
-    ``QKV_WORKSPACE`` bytes (`_two_pass`)."""
+    ``QKV_WORKSPACE`` bytes from torch's allocator (`_two_pass`); without memory
+    for it, and in a stream capture with ``out`` or ``stream`` given, as the fused
+    kernel, which needs none."""
     if x.dim() != 3 or w_qkv.dim() != 2:
         raise ValueError("expected x [n_windows, N, C] and w_qkv [3C, C]")
     nw, N, C = x.shape
@@ -309,7 +311,8 @@ def nystra_qkv(x: torch.Tensor, w_qkv: torch.Tensor, heads: int, m: int = 16, it
     d = C // heads
     if tuple(w_qkv.shape) != (3 * C, C):
         raise ValueError(f"w_qkv must be [{3 * C}, {C}]")
-    out = torch.empty((nw, heads, N, d), dtype=x.dtype, device=x.device) if out is None else out
+    own = out is None
+    out = torch.empty((nw, heads, N, d), dtype=x.dtype, device=x.device) if own else out
     for t in (x, w_qkv, out):
         if not t.is_cuda or not t.is_contiguous() or t.dtype != x.dtype:
             raise ValueError("x, w_qkv and out must be contiguous CUDA tensors of one dtype (no CPU path)")
@@ -330,7 +333,8 @@ def nystra_qkv(x: torch.Tensor, w_qkv: torch.Tensor, heads: int, m: int = 16, it
     lm, dt = _lm(landmarks, factors), _DTYPE_CODE[x.dtype]
     with torch.cuda.device(x.device):
         two = _two_pass(nw, N, heads, d, m, iters, landmarks, x, w_qkv, b_qkv, pooled, bw, out, stream)
-        rc = _qkv_two_pass(x, w_qkv, bp, out, nw, heads, N, d, m, iters, lm, bL, bU, bA, bw, dt, stream) if two else None
+        rc = (_qkv_two_pass(x, w_qkv, bp, out, own, nw, heads, N, d, m, iters, lm, bL, bU, bA, bw, dt, stream)
+              if two else None)
         if rc is None:
             rc = nystra_attention_qkv(x.data_ptr(), w_qkv.data_ptr(), bp, out.data_ptr(), nw, heads, N, d, m, iters,
                                       lm, bL, bU, bA, bw, dt, _stream_ptr(stream))
@@ -379,18 +383,32 @@ def _two_pass(nw, N, heads, d, m, iters, landmarks, x, w_qkv, b_qkv, pooled, bw,
             and out.data_ptr() % 16 == 0)
 
 
-def _qkv_two_pass(x, w_qkv, bp, out, nw, heads, N, d, m, iters, lm, bL, bU, bA, bw, dt, stream):
-    """The status code, or None if there is no memory for the workspace."""
+def _qkv_two_pass(x, w_qkv, bp, out, own, nw, heads, N, d, m, iters, lm, bL, bU, bA, bw, dt, stream):
+    """The status code, or None if there is no memory to use as the workspace.
+
+    A captured graph goes on using the workspace after this call has returned.  Only
+    the allocator's own captures give such memory a pool of its own, and who began
+    a capture cannot be told, so the workspace then lies behind ``out`` in the same
+    storage and lives as long as the graph's result does.  Where ``out`` is the
+    caller's (``own`` false), or lies in another stream's memory, there is no such
+    place, and nothing is allocated."""
     win = heads * N * d * 2  # bytes of one window's Q (as of its tokens and its output)
     per = max(1, min(nw, QKV_WORKSPACE // (3 * win)))
     per = -(-nw // (-(-nw // per)))  # chunks of equal length
     try:
         # from the pool of the stream it is used on: safe to reuse in stream order once freed
         with contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
-            ws = torch.empty(3 * per * win, dtype=torch.uint8, device=x.device)
-    except torch.OutOfMemoryError:
+            if not torch.cuda.is_current_stream_capturing():
+                ws, start = torch.empty(3 * per * win, dtype=torch.uint8, device=x.device), 0
+            elif own and stream is None:
+                start = -(-nw * win // 512) * 512
+                ws = torch.empty(start + 3 * per * win, dtype=torch.uint8, device=x.device)
+                out.set_(ws.untyped_storage(), 0, out.shape, out.stride())
+            else:
+                return None
+    except RuntimeError:  # out of memory, or the allocator may not grow now
         return None
-    q, k, v = (ws.data_ptr() + i * per * win for i in range(3))
+    q, k, v = (ws.data_ptr() + start + i * per * win for i in range(3))
     xp, op, wp, st = x.data_ptr(), out.data_ptr(), w_qkv.data_ptr(), _stream_ptr(stream)
     for i in range(0, nw, per):
         n = min(per, nw - i)

@@ -308,3 +308,21 @@ def test_an_empty_batch_has_no_second_form(N, heads, d):
     w = torch.zeros(3 * heads * d, heads * d, dtype=torch.bfloat16)
     out = torch.zeros(0, heads, N, d, dtype=torch.bfloat16)
     assert not nb._two_pass(0, N, heads, d, 16, 6, "segments", x, w, None, None, 0, out, None)
+
+
+@pytest.mark.parametrize("own,stream", [(False, None), (True, "given")])
+def test_a_capture_allocates_nothing_beside_the_result(own, stream, monkeypatch):
+    # whatever is captured uses its workspace again at every replay: where it cannot
+    # share the result's storage, nystra_qkv takes the kernel that needs none
+    import contextlib
+
+    import torch
+    x = torch.zeros(2, 1024, 64, dtype=torch.bfloat16)
+    w, out = torch.zeros(192, 64, dtype=torch.bfloat16), torch.zeros(2, 2, 1024, 32, dtype=torch.bfloat16)
+
+    def no_memory(*a, **k):
+        raise AssertionError("allocated in a capture")
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: True)
+    monkeypatch.setattr(torch.cuda, "stream", lambda s: contextlib.nullcontext())
+    monkeypatch.setattr(torch, "empty", no_memory)
+    assert nb._qkv_two_pass(x, w, 0, out, own, 2, 2, 1024, 32, 16, 6, 0, 0, 0, 0, 0, 1, stream) is None

@@ -2,6 +2,8 @@
 projection and attention by turns over a workspace, in one chunk and in several
 (a ragged last one, per-window score biases, streams), and the calls at the
 edges of the rule that picks between them."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -109,3 +111,49 @@ def test_without_memory_and_under_capture(monkeypatch):
     monkeypatch.setattr(binding, "_qkv_two_pass", lambda *a: None)  # no memory: the fused kernel
     out = binding.nystra_qkv(x, w, 2, 16, 6, b_qkv=b)
     assert torch.equal(out, _fused(x, w, 2, 16, 6, b, None, "segments"))
+
+
+@pytest.mark.parametrize("given", [False, True])
+def test_a_capture_begun_outside_torch(given):
+    # the runtime captures, and torch's allocator knows nothing of it: what the
+    # graph writes at a replay is the result's own storage, not what came after it
+    x, w, b = (t.cuda() for t in workloads.random_x_wqkv(6, 1024, 2, 32, "bf16", seed=3))
+    rt = ctypes.CDLL("libcudart.so.13")
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    graph, run = ctypes.c_void_p(), ctypes.c_void_p()
+    with torch.cuda.stream(s):
+        ref = binding.nystra_qkv(x, w, 2, 16, 6, b_qkv=b)
+        fused = _fused(x, w, 2, 16, 6, b, None, "segments")
+        mine = torch.zeros_like(ref) if given else None
+        s.synchronize()
+        assert rt.cudaStreamBeginCapture(ctypes.c_void_p(s.cuda_stream), 2) == 0  # relaxed
+        out = binding.nystra_qkv(x, w, 2, 16, 6, b_qkv=b, out=mine)
+        assert rt.cudaStreamEndCapture(ctypes.c_void_p(s.cuda_stream), ctypes.byref(graph)) == 0
+        assert rt.cudaGraphInstantiate(ctypes.byref(run), graph, ctypes.c_ulonglong(0)) == 0
+        later = [torch.full((n,), 7, dtype=torch.uint8, device="cuda") for n in [6 * 2 * 1024 * 32 * 2 * 3] * 4]
+        out.zero_()
+        for _ in range(2):
+            assert rt.cudaGraphLaunch(run, ctypes.c_void_p(s.cuda_stream)) == 0
+        s.synchronize()
+    assert torch.equal(out, fused if given else ref)
+    assert all(bool((t == 7).all()) for t in later)
+    assert rt.cudaGraphExecDestroy(run) == 0 and rt.cudaGraphDestroy(graph) == 0
+    assert binding.status() == binding.NYSTRA_OK
+
+
+@pytest.mark.parametrize("explicit", [False, True])
+def test_a_failing_workspace_allocation(explicit, monkeypatch):
+    x, w, b = (t.cuda() for t in workloads.random_x_wqkv(6, 1024, 2, 32, "bf16", seed=4))
+    fused, real = _fused(x, w, 2, 16, 6, b, None, "segments"), torch.empty
+    torch.cuda.synchronize()
+
+    def empty(*a, **k):
+        if k.get("dtype") is torch.uint8:
+            raise torch.OutOfMemoryError("no memory for the workspace")
+        return real(*a, **k)
+    monkeypatch.setattr(torch, "empty", empty)
+    s = torch.cuda.Stream() if explicit else None
+    out = binding.nystra_qkv(x, w, 2, 16, 6, b_qkv=b, stream=s)
+    torch.cuda.synchronize()
+    assert torch.equal(out, fused)
