@@ -244,13 +244,12 @@ nystra_qkv_stream_kernel(const T* __restrict__ x, const T* __restrict__ wqkv, co
             } else {
                 using Sc = ScScratch<(M > 16 ? M : 32)>;
                 unsigned char* scr = tb + Lay::T_SCR;
-                float wr[NCOL / 8][4];
-                sc_load_w<NCOL>(reinterpret_cast<const float*>(bb + Lay::B_W), wr, c, g, t);
-                sc_core<T, (M > 16 ? M : 32), NCOL>(
+                float w[NCOL / 8][4];
+                sc_core<T, (M > 16 ? M : 32), NCOL, false>(
                     reinterpret_cast<const T*>(bb + Lay::B_QB), reinterpret_cast<const T*>(bb + Lay::B_KB),
-                    gmu[16 * c + g], gmu[16 * c + g + 8], wr, reinterpret_cast<T*>(bb + Lay::B_YT), scr,
-                    scr + Sc::MAT, scr + 2 * Sc::MAT, reinterpret_cast<float*>(scr + 2 * Sc::MAT + Sc::WMAT), iters,
-                    sl2, c, lane, 1 + TEAMS + team);
+                    gmu[16 * c + g], gmu[16 * c + g + 8], w, reinterpret_cast<T*>(bb + Lay::B_YT), scr, scr + Sc::MAT,
+                    reinterpret_cast<float*>(bb + Lay::B_W), reinterpret_cast<float*>(scr + 2 * Sc::MAT), iters, sl2, c,
+                    lane, 1 + TEAMS + team);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(barC + b);

@@ -28,18 +28,20 @@ namespace tc {
 // rows padded to m + 8 halves so ldmatrix is conflict-free) that alternate
 // roles: X in one, -T2/4 in the other, T3/4 over X once every warp has used X,
 // the next X over -T2/4 once every warp has used it; three barriers per step.
-// W waits for Y = Z W in its own matrix (m rows of 40 columns), split at a power
-// of two per column (the features and the ones column are independent outputs
-// of any scale) that puts its largest entry in [2^10, 2^11).
+// Z is carried in fp32 between the steps (and split at a power of two per warp
+// for its product), and Y = Z W is a split-tf32 product of fp32 Z and W: neither
+// factor's entries have a bounded range, and both parts of a tf32 split have
+// fp32's exponent, while fp16 pairs lose bits of entries 2^13 below the largest.
 //
 // What bounds it: the tensor pipe's mma.sync rate and, between two barriers,
 // a chain of 6 or 12 dependent MMAs with the split and store of their results.
 // Measured (bf16) against full products and scales agreed on over the warps:
-// m = 64, 4096 units of 16x16 windows, d_h = 32, 0.93 -> 0.50 ms (in the wide
-// kernel, with three groups per SM instead of two), 1024 of 32x32 0.50 -> 0.37;
-// m = 32, 8192 units of 16x16, d_h = 30, 353 -> 290 us (d_h = 32 now in the team
-// kernel too: 557 -> 345, and 304 with 16-byte row loads); 1024 units of 32x32,
-// d_h = 32, not bound by the core, 144 us as before (134 with those loads).  At m = 64, carrying V = Z W
+// m = 64, 4096 units of 16x16 windows, d_h = 32, 925 -> 452 us (in the wide
+// kernel, with three groups per SM instead of two), 1024 of 32x32 499 -> 377;
+// m = 32, 8192 units of 16x16, d_h = 30, 354 -> 283 us (d_h = 32 now in the team
+// kernel too: 560 -> 294); 1024 units of 32x32, d_h = 32, 145 -> 133, the step mostly
+// in the token loads.  Y = Z W from fp16 pairs, W's scaled by a power of two per
+// column, was no faster (453, 372, 292, 306 and 135 us).  At m = 64, carrying V = Z W
 // instead (V <- T3 V/4 with X = Z A: d_h + 1 columns instead of m, 20 tile
 // products a step, but V's column scales to agree on in every step) took 0.51 and
 // 0.46 ms, and was less accurate: under sharp attention (logit std 4) its
@@ -188,7 +190,8 @@ __device__ __forceinline__ void sc_sym_mm(const H2Pair (&Ao)[M / 16][4], const H
 }
 
 // All tiles of the own rows of A P^T (P in mat), column block (c + i / 2) mod CW
-// in tiles i, i + 1: acc = A P^T; A in the cyclic k order from block c.
+// in tiles i, i + 1: acc = A P^T; A in the cyclic k order from block c, as the
+// C-layout tiles of such a product hold it.
 template <int M>
 __device__ __forceinline__ void sc_row_mm(const H2Pair (&A)[M / 16][4], const unsigned char* mat,
                                           float (&acc)[M / 8][4], int c, int lane) {
@@ -226,130 +229,80 @@ __device__ __forceinline__ void sc_row_mm(const H2Pair (&A)[M / 16][4], const un
     }
 }
 
-// Own rows of A W (W in wmat): acc = A W, A in the k order of sc_load_a from block b0.
+// x as two tf32 values, both rounded to nearest: hi + lo equals x to within
+// 2^-22 |x| (a NaN stays one in lo).
+__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
+    hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+    lo = __float_as_uint(x - __uint_as_float(hi)) + 0x1000u;  // (the tensor core ignores the low bits)
+}
+
+// Own rows of Z W: acc = z W, z as sc_row_mm leaves it, W fp32 with row stride
+// NCOL + 4 (so that a B fragment's loads fall into 32 banks).  A step of eight
+// landmarks takes columns 2t and 2t + 1 of z's tile as its k = t and t + 4, and
+// the rows of W likewise.
 template <int M, int NCOL>
-__device__ __forceinline__ void sc_w_mm(const H2Pair (&A)[M / 16][4], const unsigned char* wmat,
-                                          float (&acc)[NCOL / 8][4], int b0, int lane) {
-    constexpr int WS = ScScratch<M>::WS, CW = M / 16, NTO = NCOL / 8;
-    constexpr size_t PL = ScScratch<M>::WPLANE;
-    const int blk = lane >> 3, rr = lane & 7;
+__device__ __forceinline__ void sc_w_mm(const float (&z)[M / 8][4], const float* W, float (&acc)[NCOL / 8][4], int c,
+                                        int g, int t) {
+    constexpr int WS = NCOL + 4, CW = M / 16, NTO = NCOL / 8;
 #pragma unroll
     for (int n = 0; n < NTO; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
 #pragma unroll
-    for (int j = 0; j < CW; ++j) {
-        const int kk = (b0 + j) % CW;
-        uint32_t bh[NTO][2], bl[NTO][2];
+    for (int i = 0; i < M / 8; ++i) {
+        uint32_t ah[4], al[4], bh[NTO][2], bl[NTO][2];
 #pragma unroll
-        for (int n = 0; n < NTO; n += 2) {
-            const unsigned char* ph = wmat + ((size_t)(16 * kk + 8 * (blk & 1) + rr) * WS + 8 * (n + (blk >> 1))) * 2;
-            if (n + 1 < NTO) {
-                uint32_t x[4], y[4];
-                ldsm_x4_t(x, ph);
-                ldsm_x4_t(y, ph + PL);
-                bh[n][0] = x[0]; bh[n][1] = x[1]; bh[n + 1][0] = x[2]; bh[n + 1][1] = x[3];
-                bl[n][0] = y[0]; bl[n][1] = y[1]; bl[n + 1][0] = y[2]; bl[n + 1][1] = y[3];
-            } else {
-                ph = wmat + ((size_t)(16 * kk + 8 * (blk & 1) + rr) * WS + 8 * n) * 2;
-                ldsm_x2_t(bh[n], ph);
-                ldsm_x2_t(bl[n], ph + PL);
-            }
-        }
-        float(*D[NTO])[4];
-        const H2Pair(*Ap[NTO])[4];
-        const uint32_t *ph[NTO], *pl[NTO];
+        for (int e = 0; e < 4; ++e) split_tf32(z[i][2 * (e & 1) + (e >> 1)], ah[e], al[e]);
+        const float* w = W + (16 * ((c + i / 2) % CW) + 8 * (i & 1) + 2 * t) * WS + g;
 #pragma unroll
         for (int n = 0; n < NTO; ++n) {
-            D[n] = &acc[n];
-            Ap[n] = &A[j];
-            ph[n] = bh[n];
-            pl[n] = bl[n];
-        }
-        sc_mma<NTO>(D, Ap, ph, pl);
-    }
-}
-
-// Column maxima of |w| over this warp's rows into slot[0 .. NCOL).
-template <int NCOL>
-__device__ __forceinline__ void sc_colmax(const float (&v)[NCOL / 8][4], float* slot, int g, int t) {
-#pragma unroll
-    for (int n = 0; n < NCOL / 8; ++n)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            float x = fmaxf(fabsf(v[n][e]), fabsf(v[n][e + 2]));
-            x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 4));
-            x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 8));
-            x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 16));
-            if (g == 0) slot[8 * n + 2 * t + e] = x;
-        }
-}
-
-// Own rows of W into wmat, column by column scaled by 2^ev with ev from the
-// column's largest entry (over the warps' slots; per lane columns 8n + 2t,
-// 8n + 2t + 1), within +-120, so that both powers of two are normal numbers.
-template <int M, int NCOL>
-__device__ __forceinline__ void sc_put_w(unsigned char* wmat, const float (&v)[NCOL / 8][4], const float* slots,
-                                         int (&ev)[NCOL / 8][2], int c, int g, int t) {
-    constexpr int WS = ScScratch<M>::WS, CW = M / 16;
-#pragma unroll
-    for (int n = 0; n < NCOL / 8; ++n) {
-        float s[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            float x = 0.f;
-#pragma unroll
-            for (int w = 0; w < CW; ++w) x = fmaxf(x, slots[w * NCOL + 8 * n + 2 * t + e]);
-            ev[n][e] = max(-120, min(120, h2_exponent(x)));
-            s[e] = pow2i(ev[n][e]);
+            split_tf32(w[8 * n], bh[n][0], bl[n][0]);
+            split_tf32(w[8 * n + WS], bh[n][1], bl[n][1]);
         }
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const H2Pair p = split_h2(s[0] * v[n][2 * h], s[1] * v[n][2 * h + 1]);
-            unsigned char* q = wmat + ((size_t)(16 * c + g + 8 * h) * WS + 8 * n + 2 * t) * 2;
-            *reinterpret_cast<uint32_t*>(q) = p.hi;
-            *reinterpret_cast<uint32_t*>(q + ScScratch<M>::WPLANE) = p.lo;
-        }
+        for (int n = 0; n < NTO; ++n) mma_tf32(acc[n], al[0], al[1], al[2], al[3], bh[n][0], bh[n][1]);
+#pragma unroll
+        for (int n = 0; n < NTO; ++n) mma_tf32(acc[n], ah[0], ah[1], ah[2], ah[3], bl[n][0], bl[n][1]);
+#pragma unroll
+        for (int n = 0; n < NTO; ++n) mma_tf32(acc[n], ah[0], ah[1], ah[2], ah[3], bh[n][0], bh[n][1]);
     }
 }
 
 // Core on CW = M/16 warps (warp c of them calls with its index; bar_id is a
-// named barrier reserved for these warps; mat0, mat1, wmat, aux: ScScratch
-// areas): G_A^n from the landmarks and the m_U of the own rows (mu0, mu1: rows
-// 16c + g and + 8, log2 domain), the iteration of step 4, Y = Z W (on entry w:
-// the own rows of W, C layout) stored as Y^T at yT, or where yT is null over
-// the scratch matrix that is free by then; returns its place.  wmat may overlay
-// Qbar (first written after every warp has read its rows).  As in core_warp, A
-// is split at 2^ea with its largest entry in [2^10, 2^11); X, -T2/4 and T3/4
-// are split at the fixed scale 2^10 (their entries stay within a few units,
-// since X's eigenvalues lie in [0, 1]).  Scalar factors of Z cancel in step 7
-// and are dropped; the warps' and columns' powers of two are taken back.
-template <typename T, int M, int NCOL>
+// named barrier reserved for these warps; mat0, mat1, aux: ScScratch areas):
+// G_A^n from the landmarks and the m_U of the own rows (mu0, mu1: rows 16c + g
+// and + 8, log2 domain), the iteration of step 4, Y = Z W (W: fp32, row stride
+// NCOL + 4) stored as Y^T at yT, or where yT is null over the scratch matrix that
+// is free by then; returns its place.  WREG: w holds the own rows of W on entry
+// (C layout), and W, which may overlay Qbar, is first written after every warp
+// has read its rows.  yT may overlay W.  As in core_warp, A is split at 2^ea
+// with its largest entry in [2^10, 2^11); X, -T2/4 and T3/4 are split at the
+// fixed scale 2^10 (their entries stay within a few units, since X's
+// eigenvalues lie in [0, 1]).  Scalar factors of Z cancel in step 7 and are
+// dropped; the warps' powers of two are taken back.
+template <typename T, int M, int NCOL, bool WREG>
 __device__ __forceinline__ T* sc_core(const T* qbar, const T* kbar, float mu0, float mu1, float (&w)[NCOL / 8][4],
-                                      T* yT, unsigned char* mat0, unsigned char* mat1, unsigned char* wmat, float* aux,
-                                      int iters, float sl2, int c, int lane, int bar_id) {
+                                      T* yT, unsigned char* mat0, unsigned char* mat1, float* W, float* aux, int iters,
+                                      float sl2, int c, int lane, int bar_id) {
     using S = ScScratch<M>;
     using O = Opnd<T>;
     using D = typename O::DReg;
     constexpr int CW = S::CW, KT = M / 16, NT = M / 8, LS = LmS<T>::LS, LO = LmS<T>::LO, NTO = NCOL / 8,
                   YS = YtS<T, M>::YS, YLO = YtS<T, M>::LO, NTL = ScTiles<M>::N;
-    static_assert(NCOL <= S::WS, "W's rows");
     const int g = lane >> 2, t = lane & 3;
     unsigned char* cur = mat0;
     unsigned char* oth = mat1;
     float* cols = aux;                // [CW][M] column-sum partials
     float* slots = aux + CW * M;      // [4][CW] maxima
-    float* wslots = slots + 4 * CW;   // [CW][NCOL] column maxima of W
     auto csync = [&]() { named_barrier(bar_id, CW * 32); };
     const uint32_t sel = tril_selector(g, t);
     const ScTiles<M> tl(c);
     constexpr float kS = 1024.f, kS2 = 1048576.f;  // fixed scale 2^10 of X, -T2/4, T3/4 (and its square)
-    H2Pair Xa[KT][4], X5[KT][4], Za[KT][4];
-    float acc[NTL][4];
-    int ev[NTO][2], ez = 0;  // powers of two of W's columns and of Z's rows
-    float alpha;             // a A A^T = alpha (2^ea A)(2^ea A)^T
+    H2Pair Xa[KT][4], X5[KT][4];
+    float acc[NTL][4], z[NT][4];  // z: the own rows of 2^ez Z, tiles as in sc_row_mm
+    int ez = 0;
+    float alpha;  // a A A^T = alpha (2^ea A)(2^ea A)^T
     {
         float a[NT][4];
         // ---- G_A^n's own rows ----
-        sc_colmax<NCOL>(w, wslots + c * NCOL, g, t);
         {
             D aq[2][4];
 #pragma unroll
@@ -420,7 +373,14 @@ __device__ __forceinline__ T* sc_core(const T* qbar, const T* kbar, float mu0, f
                 }
         }
         sc_put<M>(cur, a, c, g, t);  // 2^ea A
-        sc_put_w<M, NCOL>(wmat, w, wslots, ev, c, g, t);
+        if constexpr (WREG) {
+#pragma unroll
+            for (int n = 0; n < NTO; ++n)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    *reinterpret_cast<float2*>(W + (16 * c + g + 8 * h) * (NCOL + 4) + 8 * n + 2 * t) =
+                        make_float2(w[n][2 * h], w[n][2 * h + 1]);
+        }
         csync();
         float rmax = 0.f, cmax = 0.f;
 #pragma unroll
@@ -456,7 +416,18 @@ __device__ __forceinline__ T* sc_core(const T* qbar, const T* kbar, float mu0, f
     sc_load_a<M, false>(cur, X5, tl.r5, tl.b5, lane);
     zero();
     sc_sym_mm<M>(Xa, X5, cur, acc, tl, lane);
-    sc_load_a<M, true>(cur, Za, c, c, lane);
+    {
+        H2Pair Za[KT][4];
+        sc_load_a<M, true>(cur, Za, c, c, lane);
+#pragma unroll
+        for (int j = 0; j < KT; ++j)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float2 v = entries(Za, j, r >> 1, r & 1);
+                z[2 * j + (r >> 1)][2 * (r & 1)] = v.x;
+                z[2 * j + (r >> 1)][2 * (r & 1) + 1] = v.y;
+            }
+    }
     sc_put_sym<M>(oth, acc, kS * alpha, tl, g, t, sel);  // kS X_0
     csync();
     {
@@ -499,8 +470,6 @@ __device__ __forceinline__ T* sc_core(const T* qbar, const T* kbar, float mu0, f
             sc_put_sym<M>(oth, acc, 1.f / kS, tl, g, t, sel);  // every warp is done with -T2/4
         }
         {
-            float z[NT][4];
-            sc_row_mm<M>(Za, cur, z, c, lane);  // kS Z T3/4
             float zm = 0.f;
 #pragma unroll
             for (int n = 0; n < NT; ++n)
@@ -509,13 +478,15 @@ __device__ __forceinline__ T* sc_core(const T* qbar, const T* kbar, float mu0, f
             const int e = h2_exponent(warp_max_nonneg(zm));
             const float s = pow2i(e);
             ez += e + 10;  // and kS
+            H2Pair Za[KT][4];
 #pragma unroll
             for (int j = 0; j < KT; ++j)
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    const int n = 2 * j + (r >> 1), x = 2 * (r & 1);
-                    Za[j][r] = split_h2(s * z[n][x], s * z[n][x + 1]);
+                    const int n = 2 * j + (r >> 1), v = 2 * (r & 1);
+                    Za[j][r] = split_h2(s * z[n][v], s * z[n][v + 1]);
                 }
+            sc_row_mm<M>(Za, cur, z, c, lane);  // kS Z T3/4
         }
         if (more) {
             csync();
@@ -524,17 +495,13 @@ __device__ __forceinline__ T* sc_core(const T* qbar, const T* kbar, float mu0, f
             oth = tmp;
         }
     }
-    // ---- Y = Z W, own rows, without the powers of two, stored as Y^T ----
-    sc_w_mm<M, NCOL>(Za, wmat, w, c, lane);
+    // ---- Y = Z W, own rows, without the warp's power of two, stored as Y^T ----
+    sc_w_mm<M, NCOL>(z, W, w, c, g, t);
     const float sz = pow2i(-ez);
 #pragma unroll
-    for (int n = 0; n < NTO; ++n) {
-        const float s0 = pow2i(-ev[n][0]), s1 = pow2i(-ev[n][1]);
-        w[n][0] = sz * w[n][0] * s0;
-        w[n][2] = sz * w[n][2] * s0;
-        w[n][1] = sz * w[n][1] * s1;
-        w[n][3] = sz * w[n][3] * s1;
-    }
+    for (int n = 0; n < NTO; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) w[n][e] *= sz;
     float scale = 1.f;
     if (O::kNarrowRange) {
         float ym = 0.f;
@@ -549,7 +516,7 @@ __device__ __forceinline__ T* sc_core(const T* qbar, const T* kbar, float mu0, f
 #pragma unroll
         for (int x = 0; x < CW; ++x) ymax = fmaxf(ymax, slots[2 * CW + x]);
         if (ymax > 0.f && ymax < INFINITY) scale = pow2i(14 - ilogbf(ymax));
-    }
+    } else if (yT) csync();  // Y^T may overlay W, which every warp reads in full
     // free: after the last step -T2/4's matrix (its readers have passed a
     // barrier since), without steps A's
     if constexpr (YtS<T, M>::bytes(NCOL) <= S::MAT)  // (m = 32: the caller has a place)
@@ -563,18 +530,6 @@ __device__ __forceinline__ T* sc_core(const T* qbar, const T* kbar, float mu0, f
         DSt<T>::put(yT + (cc + 1) * YS + rr + 8, YLO, w[j][3] * scale);
     }
     return yT;
-}
-
-// The own rows of W (fp32, row stride NCOL + 4 at mW) as sc_core takes them.
-template <int NCOL>
-__device__ __forceinline__ void sc_load_w(const float* mW, float (&v)[NCOL / 8][4], int c, int g, int t) {
-    constexpr int WS = NCOL + 4;
-#pragma unroll
-    for (int n = 0; n < NCOL / 8; ++n) {
-        const float2 x = *reinterpret_cast<const float2*>(mW + (16 * c + g) * WS + 8 * n + 2 * t);
-        const float2 y = *reinterpret_cast<const float2*>(mW + (16 * c + g + 8) * WS + 8 * n + 2 * t);
-        v[n][0] = x.x; v[n][1] = x.y; v[n][2] = y.x; v[n][3] = y.y;
-    }
 }
 
 }  // namespace tc

@@ -123,18 +123,14 @@ static_assert(row_step(30) == 4 && row_step(28) == 2 && row_step(32) == 1 && row
 
 // Shared scratch of the core with symmetric products (nystra_symcore.cuh): two
 // matrices of fp16 pairs (hi plane, then lo plane; rows padded to m + 8 halves
-// so ldmatrix is conflict-free), W (m rows of 40 columns, likewise) and an
-// auxiliary float area.
+// so ldmatrix is conflict-free) and an auxiliary float area.
 template <int M>
 struct ScScratch {
-    static constexpr int CW = M / 16, SS = M + 8, WS = 40;
+    static constexpr int CW = M / 16, SS = M + 8;
     static constexpr size_t PLANE = (size_t)M * SS * 2;
     static constexpr size_t MAT = 2 * PLANE;
-    static constexpr size_t WPLANE = (size_t)M * WS * 2;
-    static constexpr size_t WMAT = 2 * WPLANE;
-    // column sums of A, maxima, column maxima of W
-    static constexpr size_t AUX = ((size_t)CW * M * 4 + 4 * CW * 4 + CW * WS * 4 + 15) / 16 * 16;
-    static constexpr size_t BYTES = ((2 * MAT + WMAT + AUX + 127) / 128) * 128;  // mat0 | mat1 | W | aux
+    static constexpr size_t AUX = ((size_t)CW * M * 4 + 4 * CW * 4 + 15) / 16 * 16;  // column sums of A, maxima
+    static constexpr size_t BYTES = ((2 * MAT + AUX + 127) / 128) * 128;             // mat0 | mat1 | aux
 };
 
 template <typename T, int M>
@@ -166,7 +162,7 @@ struct Layout {
     // token warps' K/V rows (consumed by the combine before the core starts; the
     // next unit's K and V are copied after the core).
     static_assert(CW == 1 || (M == 64 && CW == 4 && WPU >= 2 &&
-                              ScScratch<64>::MAT + ScScratch<64>::WMAT <= 2 * (size_t)TPW * DS * 2),
+                              ScScratch<64>::MAT + ScScratch<64>::AUX <= 2 * (size_t)TPW * DS * 2),
                   "scratch must fit in two warps' K/V rows");
     static constexpr size_t QB_BYTES = LmS<T>::bytes(MP);
     static constexpr size_t YT_BYTES = YtS<T, M>::bytes(NCOL);
@@ -1358,7 +1354,6 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
     // scratch of the core on several warps
     unsigned char* mat0 = nullptr;
     unsigned char* mat1 = nullptr;
-    unsigned char* wmat = nullptr;
     float* aux = nullptr;
     if constexpr (CW > 1) {
         using Sc = ScScratch<64>;
@@ -1366,7 +1361,6 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
         mat0 = w0 + Lay::WPART;
         aux = reinterpret_cast<float*>(mat0 + Sc::MAT);
         mat1 = w0 + Lay::WARP_BYTES + Lay::WPART;
-        wmat = mat1 + Sc::MAT;
     }
 
     // Only the first `active` groups of a CTA take units (see launch_cfg).
@@ -1506,9 +1500,8 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
         } else {
             if (r < CW) {
                 float w[NCOL / 8][4];
-                sc_load_w<NCOL>(mW, w, r, g, t);
-                sc_core<T, M, NCOL>(qbar, kbar, gmu[16 * r + g], gmu[16 * r + g + 8], w, yT, mat0, mat1, wmat, aux,
-                                    iters, sl2, r, lane, 1 + GROUPS + grp);
+                sc_core<T, M, NCOL, false>(qbar, kbar, gmu[16 * r + g], gmu[16 * r + g + 8], w, yT, mat0, mat1, mW, aux,
+                                           iters, sl2, r, lane, 1 + GROUPS + grp);
             }
         }
         gsync();

@@ -16,9 +16,8 @@
 // a group per SM, and the SM's other groups fill the wait.  Three groups of
 // four warps run per SM (73 KB each at N = 256), against two groups with 108 KB
 // and two token warps each on the grouped kernel.
-// Measured (bf16): 4096 units of 16x16 windows, d_h = 32: 0.93 -> 0.50 ms (0.45
-// with the rows read 16 bytes at a time);
-// 8640 units of 8x8 windows, d_h = 30: 1.45 -> 0.78 ms.
+// Measured (bf16): 4096 units of 16x16 windows, d_h = 32: 0.92 -> 0.45 ms; 8640
+// units of 8x8 windows, d_h = 30: 1.44 -> 0.72 ms.
 //
 // Every wait on an mbarrier is bounded; the warps of a group share its
 // barriers, and a wait that gives up is agreed on at the next one.
@@ -39,7 +38,8 @@ struct WideLayout {
     static constexpr size_t G_KV = ROWS;  // K, V; the core's two matrices
     static constexpr size_t KV = ((2 * ROWS > 2 * Sc::MAT ? 2 * ROWS : 2 * Sc::MAT) + 15) / 16 * 16;
     static constexpr size_t G_QV = G_KV + KV;  // Qbar; the core's W
-    static constexpr size_t QV = LmS<T>::bytes(M) > Sc::WMAT ? LmS<T>::bytes(M) : Sc::WMAT;
+    static constexpr size_t WMAT = (size_t)M * (NCOL + 4) * 4;
+    static constexpr size_t QV = LmS<T>::bytes(M) > WMAT ? LmS<T>::bytes(M) : WMAT;
     static constexpr size_t G_KBAR = G_QV + QV;
     static constexpr size_t G_AUX = G_KBAR + LmS<T>::bytes(M);
     static constexpr size_t G_BAR = G_AUX + Sc::AUX;  // Q and K rows; V rows
@@ -241,9 +241,9 @@ nystra_wide_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
         }
         // ---------------- core ----------------
         // (its first write to the K and V rows comes after a barrier of its own)
-        const T* yT = sc_core<T, M, NCOL>(qbar, kbar, run0, run1, w, nullptr, gb + Lay::G_KV,
-                                          gb + Lay::G_KV + Sc::MAT, gb + Lay::G_QV,
-                                          reinterpret_cast<float*>(gb + Lay::G_AUX), iters, sl2, c, lane, bar);
+        const T* yT = sc_core<T, M, NCOL, true>(qbar, kbar, run0, run1, w, nullptr, gb + Lay::G_KV,
+                                                gb + Lay::G_KV + Sc::MAT, reinterpret_cast<float*>(gb + Lay::G_QV),
+                                                reinterpret_cast<float*>(gb + Lay::G_AUX), iters, sl2, c, lane, bar);
         gsync();
         // ---------------- output, in place over Q ----------------
 #pragma unroll 1

@@ -55,3 +55,23 @@ def test_columns_of_any_scale(N, dtype, lo, hi):
     bar = TOL[dtype] if dtype == "bf16" else TOL[dtype] + 2.0 ** -25 / (0.02 * 2.0 ** lo)
     assert col.max() <= bar, col.max()
     assert per_unit_rel(a, ref).max() <= TOL[dtype]
+
+
+@pytest.mark.parametrize("N,m", [(64, 32), (64, 64), (256, 32), (256, 64), (1024, 32), (1024, 64)])
+def test_landmarks_of_any_scale(N, m):
+    # two groups of tokens that attend to their own group alone: feature 0 is +20 or
+    # -20, so a score across is 146 below one within and its exponential 0 in fp32.
+    # The rows of V (and of W) of one group are scaled by 2^-40, exact in bf16: so
+    # is its output, to all its digits, whatever the other group's rows of W hold
+    q, k, v = (x.bfloat16() for x in workloads.random_qkv(3, N, 30, "f32", seed=N + m))
+    near = torch.arange(N) < N // 2
+    for x in (q, k):
+        x[..., 0] = torch.where(near, 20.0, -20.0)
+    s = torch.where(near, 2.0 ** -40, 1.0)[:, None]
+    out = binding.nystra(q.cuda(), k.cuda(), (v.float() * s).bfloat16().cuda(), m, 6)
+    torch.cuda.synchronize()
+    assert binding.status() == binding.NYSTRA_OK
+    out = units_view(out.cpu()).double().numpy() / s.double().numpy()
+    ref = oracle.nystra_attention(q, k, v, m, 6)
+    for rows in (slice(0, N // 2), slice(N // 2, N)):
+        assert per_unit_rel(out[:, rows], ref[:, rows]).max() <= TOL["bf16"]
