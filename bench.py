@@ -488,11 +488,13 @@ def run_cuda_qkv(args, wl):
     bp = (0, 0, 0) if pooled is None else tuple(t.data_ptr() for t in pooled)
     dcode = {"bf16": 1, "f16": 2}[wl.dtype]
 
+    def fused(xd, od, sptr):
+        return binding.nystra_attention_qkv(xd.data_ptr(), wd.data_ptr(), 0, od.data_ptr(), wl.n_windows, wl.heads,
+                                            wl.N, wl.d, wl.m, wl.iters, binding._lm(wl.landmarks, wl.factors), *bp,
+                                            1 if pooled is not None else 0, dcode, sptr)
+
     def step(i):
-        xd, od = sets[i % nsets]
-        rc = binding.nystra_attention_qkv(xd.data_ptr(), wd.data_ptr(), 0, od.data_ptr(), wl.n_windows, wl.heads,
-                                          wl.N, wl.d, wl.m, wl.iters, binding._lm(wl.landmarks, wl.factors), *bp,
-                                          1 if pooled is not None else 0, dcode, sptr)
+        rc = fused(*sets[i % nsets], sptr)
         if rc != 0:
             raise binding.NystraError(rc, "bench step")
 
@@ -576,8 +578,9 @@ def run_cuda_qkv(args, wl):
         xd, od = sets[i % 2]
         with torch.cuda.stream(streams[i % 2]):
             xd.copy_(hx, non_blocking=True)
-            binding.nystra_qkv(xd, wd, wl.heads, wl.m, wl.iters, pooled=pooled, out=od, landmarks=wl.landmarks,
-                               factors=wl.factors)
+            rc = fused(xd, od, streams[i % 2].cuda_stream)
+            if rc != 0:
+                raise binding.NystraError(rc, "bench e2e step")
             hos[i % 2].copy_(od, non_blocking=True)
 
     e2e_steps = max(4, min(args.steps, 50))

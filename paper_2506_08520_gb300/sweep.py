@@ -13,7 +13,7 @@ the speedup over exact attention (which runs without the bias).  A mix
 one stream and is timed as one.  A workload with a relative-position bias
 pools it once (a model constant) and times the biased call.  A fused-projection
 workload ("-qkv": tokens X and W_QKV in, algorithmic bytes X + W + O) is timed
-against the unfused path it replaces: one cuBLAS projection X W_QKV^T (torch),
+on the fused kernel, nystra_attention_qkv, against the unfused path it replaces: one cuBLAS projection X W_QKV^T (torch),
 the copy that splits heads, and nystra_attention; and against the library's
 own two-pass path: nystra_project_qkv (the projection with the head split on
 the tcgen05 tensor cores, timed alone too) followed by nystra_attention.
@@ -85,12 +85,17 @@ def run_qkv(wl: workloads.Workload, l2_bytes: int, peak: float, reps: int = 50) 
     w = w.to(dev)
     bias = workloads.make_bias(wl)
     pooled = None if bias is None else binding.pool_bias(bias.to(dev), wl.m, wl.landmarks)
+    blocks = (0, 0, 0) if pooled is None else tuple(t.data_ptr() for t in pooled)
+    dcode = binding._DTYPE_CODE[x.dtype]
     sets = [(x.to(dev), torch.empty(wl.shape, dtype=x.dtype, device=dev)) for _ in range(n_sets)]
 
     def fused(i):
         xs, o = sets[i]
-        binding.nystra_qkv(xs, w, wl.heads, wl.m, wl.iters, pooled=pooled, out=o, landmarks=wl.landmarks,
-                           factors=wl.factors)
+        rc = binding.nystra_attention_qkv(xs.data_ptr(), w.data_ptr(), 0, o.data_ptr(), wl.n_windows, wl.heads, wl.N,
+                                          wl.d, wl.m, wl.iters, binding._lm(wl.landmarks, wl.factors), *blocks,
+                                          0 if pooled is None else 1, dcode, torch.cuda.current_stream().cuda_stream)
+        if rc != binding.NYSTRA_OK:
+            raise binding.NystraError(rc, "nystra_attention_qkv")
 
     def unfused(i):
         xs, o = sets[i]

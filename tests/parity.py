@@ -25,6 +25,20 @@ def gpu_nystra(q, k, v, m, iters, landmarks="segments"):
     return out
 
 
+def fused_qkv(x, w, heads, m, iters, b=None, pooled=None, landmarks="segments", factors="pairs"):
+    """The fused projection's C entry point on device tensors (binding.nystra_qkv
+    takes another route for some sizes)."""
+    nw, N, C = x.shape
+    out = torch.empty((nw, heads, N, C // heads), dtype=x.dtype, device=x.device)
+    bl = (0, 0, 0) if pooled is None else tuple(t.data_ptr() for t in pooled)
+    bw = 0 if pooled is None else pooled[0].numel() // (heads * N * m)
+    rc = binding.nystra_attention_qkv(x.data_ptr(), w.data_ptr(), 0 if b is None else b.data_ptr(), out.data_ptr(), nw,
+                                      heads, N, C // heads, m, iters, binding._lm(landmarks, factors), *bl, bw,
+                                      binding._DTYPE_CODE[x.dtype], torch.cuda.current_stream().cuda_stream)
+    assert rc == binding.NYSTRA_OK, rc
+    return out
+
+
 def gpu_exact(q, k, v):
     qd, kd, vd = (x.cuda() for x in (q, k, v))
     out = binding.exact(qd, kd, vd)

@@ -13,7 +13,7 @@ import torch
 
 import oracle
 from paper_2506_08520_gb300 import binding, workloads
-from tests.parity import TOL, per_unit_rel
+from tests.parity import TOL, fused_qkv, per_unit_rel
 
 pytestmark = pytest.mark.gpu
 
@@ -152,7 +152,7 @@ def test_projection_then_attention(N, m):
     xd, wd, bd = x.cuda(), w.cuda(), b.cuda()
     q, k, v = binding.project_qkv(xd, wd, 6, bd)
     out = binding.nystra(q, k, v, m, 6)
-    fused = binding.nystra_qkv(xd, wd, 6, m, 6, b_qkv=bd)
+    fused = fused_qkv(xd, wd, 6, m, 6, b=bd)
     torch.cuda.synchronize()
     assert binding.status() == binding.NYSTRA_OK
     ref = oracle.nystra_attention_qkv(x, w, b, 6, m, 6)

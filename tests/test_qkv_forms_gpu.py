@@ -10,7 +10,7 @@ import torch
 
 import oracle
 from paper_2506_08520_gb300 import binding, workloads
-from tests.parity import TOL, per_unit_rel
+from tests.parity import TOL, fused_qkv, per_unit_rel
 
 pytestmark = pytest.mark.gpu
 
@@ -19,18 +19,6 @@ pytestmark = pytest.mark.gpu
 def _built():
     from paper_2506_08520_gb300 import build
     build.build()
-
-
-def _fused(x, w, heads, m, iters, b, pooled, lm):
-    nw, N, C = x.shape
-    out = torch.empty((nw, heads, N, C // heads), dtype=x.dtype, device=x.device)
-    bl = [t.data_ptr() for t in pooled] if pooled is not None else [0, 0, 0]
-    bw = pooled[0].numel() // (heads * N * m) if pooled is not None else 0
-    rc = binding.nystra_attention_qkv(x.data_ptr(), w.data_ptr(), b.data_ptr(), out.data_ptr(), nw, heads, N,
-                                      C // heads, m, iters, binding.LANDMARKS[lm], *bl, bw,
-                                      binding._DTYPE_CODE[x.dtype], torch.cuda.current_stream().cuda_stream)
-    assert rc == binding.NYSTRA_OK
-    return out
 
 
 CASES = [  # windows, heads, N, d, m, pooling, bias (None, "heads", "windows"), dtype
@@ -52,7 +40,7 @@ def test_both_forms_match_the_oracle(nw, heads, N, d, m, lm, kind, dtype, monkey
     assert binding._two_pass(nw, N, heads, d, m, 5, lm, xd, wd, bd, pooled, nw if kind == "windows" else 1,
                              torch.empty_like(xd), None)
     one = binding.nystra_qkv(xd, wd, heads, m, 5, b_qkv=bd, pooled=pooled, landmarks=lm)
-    fused = _fused(xd, wd, heads, m, 5, bd, pooled, lm)
+    fused = fused_qkv(xd, wd, heads, m, 5, bd, pooled, lm)
     monkeypatch.setattr(binding, "QKV_WORKSPACE", 3 * (nw // 2) * heads * N * d * 2)  # two or three chunks
     s = torch.cuda.Stream()
     s.wait_stream(torch.cuda.current_stream())
@@ -110,7 +98,7 @@ def test_without_memory_and_under_capture(monkeypatch):
     assert torch.equal(out, ref)
     monkeypatch.setattr(binding, "_qkv_two_pass", lambda *a: None)  # no memory: the fused kernel
     out = binding.nystra_qkv(x, w, 2, 16, 6, b_qkv=b)
-    assert torch.equal(out, _fused(x, w, 2, 16, 6, b, None, "segments"))
+    assert torch.equal(out, fused_qkv(x, w, 2, 16, 6, b))
 
 
 @pytest.mark.parametrize("given", [False, True])
@@ -124,7 +112,7 @@ def test_a_capture_begun_outside_torch(given):
     graph, run = ctypes.c_void_p(), ctypes.c_void_p()
     with torch.cuda.stream(s):
         ref = binding.nystra_qkv(x, w, 2, 16, 6, b_qkv=b)
-        fused = _fused(x, w, 2, 16, 6, b, None, "segments")
+        fused = fused_qkv(x, w, 2, 16, 6, b)
         mine = torch.zeros_like(ref) if given else None
         s.synchronize()
         assert rt.cudaStreamBeginCapture(ctypes.c_void_p(s.cuda_stream), 2) == 0  # relaxed
@@ -145,7 +133,7 @@ def test_a_capture_begun_outside_torch(given):
 @pytest.mark.parametrize("explicit", [False, True])
 def test_a_failing_workspace_allocation(explicit, monkeypatch):
     x, w, b = (t.cuda() for t in workloads.random_x_wqkv(6, 1024, 2, 32, "bf16", seed=4))
-    fused, real = _fused(x, w, 2, 16, 6, b, None, "segments"), torch.empty
+    fused, real = fused_qkv(x, w, 2, 16, 6, b), torch.empty
     torch.cuda.synchronize()
 
     def empty(*a, **k):

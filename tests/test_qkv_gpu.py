@@ -1,5 +1,5 @@
 """The fused Q/K/V projection front end on the GPU against the float64
-oracle (the projections of Eq. 1, then PnP-Nystra).  The oracle projects
+oracle (the projections of Eq. 1, then PnP-Nystra).  Every test calls the fused kernel's C entry point.  The oracle projects
 without rounding; the kernel rounds Q, K, V to the I/O type as an unfused
 projection would store them, and over the paper's 0-6 iterations the same bar
 holds with that rounding."""
@@ -9,7 +9,7 @@ import torch
 
 import oracle
 from paper_2506_08520_gb300 import binding, workloads
-from tests.parity import TOL, per_unit_rel, sample_units
+from tests.parity import TOL, fused_qkv, per_unit_rel, sample_units
 
 pytestmark = pytest.mark.gpu
 
@@ -21,8 +21,8 @@ def _built():
 
 
 def _run(x, w, b, heads, m, iters=6, pool="segments", pooled=None):
-    out = binding.nystra_qkv(x.cuda(), w.cuda(), heads, m, iters, b_qkv=None if b is None else b.cuda(),
-                             pooled=pooled, landmarks=pool)
+    out = fused_qkv(x.cuda(), w.cuda(), heads, m, iters, b=None if b is None else b.cuda(), pooled=pooled,
+                    landmarks=pool)
     torch.cuda.synchronize()
     assert binding.status() == binding.NYSTRA_OK
     return out.cpu()
@@ -130,7 +130,7 @@ def test_fused_workloads(name):
     pooled, B = None, workloads.make_bias(wl)
     if B is not None:
         pooled = binding.pool_bias(B.cuda(), wl.m, wl.landmarks)
-    out = binding.nystra_qkv(x.cuda(), w.cuda(), wl.heads, wl.m, wl.iters, pooled=pooled, landmarks=wl.landmarks)
+    out = fused_qkv(x.cuda(), w.cuda(), wl.heads, wl.m, wl.iters, pooled=pooled, landmarks=wl.landmarks)
     torch.cuda.synchronize()
     assert binding.status() == binding.NYSTRA_OK
     idx = sample_units(wl.units, 96)
@@ -213,7 +213,7 @@ def test_fused_projection_with_16bit_factors():
     ref = oracle.nystra_attention_qkv(x, w, b, 6, 16, 6)
     outs = []
     for factors in ("pairs", "16"):
-        o = binding.nystra_qkv(x.cuda(), w.cuda(), 6, 16, 6, b_qkv=b.cuda(), factors=factors)
+        o = fused_qkv(x.cuda(), w.cuda(), 6, 16, 6, b=b.cuda(), factors=factors)
         torch.cuda.synchronize()
         assert binding.status() == binding.NYSTRA_OK
         outs.append(o.cpu())
@@ -299,8 +299,31 @@ def test_fused_large_windows_many_windows_and_16bit_factors():
     pos = np.searchsorted(uw, win)
     ref = oracle.nystra_attention(q[pos, head], k[pos, head], v[pos, head], m, 6)
     for factors in ("pairs", "16"):
-        out = binding.nystra_qkv(x.cuda(), w.cuda(), heads, m, 6, b_qkv=b.cuda(), factors=factors)
+        out = fused_qkv(x.cuda(), w.cuda(), heads, m, 6, b=b.cuda(), factors=factors)
         torch.cuda.synchronize()
         assert binding.status() == binding.NYSTRA_OK
         got = out.reshape(nw * heads, N, d)[torch.from_numpy(idx)].cpu().double().numpy()
         assert per_unit_rel(got, ref).max() <= TOL["bf16"], factors
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("factors", ["pairs", "16"])
+def test_fused_two_warp_core_over_several_units(dtype, factors):
+    """m = 32 at 32x32 windows: the core's two warps share scratch that the next
+    unit's core uses again, and both buffers of a team's state.  Four units per
+    team (two teams on each of at most 160 SMs).  Sampled units; the bar is that of
+    m = 16 on the same soft inputs, per factor mode."""
+    nw, N, heads, d, m = 640, 1024, 2, 32, 32
+    x, w, b = workloads.random_x_wqkv(nw, N, heads, d, dtype, seed=78)
+    idx = sample_units(nw * heads, 48)
+    win, head = idx // heads, idx % heads
+    uw = np.unique(win)
+    q, k, v = oracle.project_qkv(x[torch.from_numpy(uw)], w, b, heads)
+    pos = np.searchsorted(uw, win)
+    ref = oracle.nystra_attention(q[pos, head], k[pos, head], v[pos, head], m, 6)
+    out = fused_qkv(x.cuda(), w.cuda(), heads, m, 6, b=b.cuda(), factors=factors)
+    torch.cuda.synchronize()
+    assert binding.status() == binding.NYSTRA_OK
+    err = per_unit_rel(out.reshape(nw * heads, N, d)[torch.from_numpy(idx)].cpu().double().numpy(), ref)
+    print(f"m = 32, {dtype}, {factors}: max rel err {err.max():.3e}")
+    assert err.max() <= TOL[dtype], f"max rel err {err.max():.3e} at unit {int(idx[err.argmax()])}"
