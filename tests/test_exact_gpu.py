@@ -61,10 +61,11 @@ def test_late_maximum(N, dtype):
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
 @pytest.mark.parametrize("units,N,d", [(2, 1, 1), (3, 63, 16), (3, 64, 17), (2, 65, 20), (2, 127, 21), (2, 129, 33),
-                                       (3, 200, 36), (2, 256, 37), (2, 100, 64), (1, 1024, 30), (1, 1000, 63)])
+                                       (3, 200, 36), (2, 256, 37), (2, 100, 64), (1, 1024, 30), (1, 1000, 63),
+                                       (5, 4, 16), (2, 15, 33), (3, 16, 20), (2, 16, 64), (2, 17, 30)])
 def test_generic_tile_edges(units, N, d, dtype):
     # blocks of 64 rows and chunks of 64 keys, one more or less than whole
-    # ones; the head widths at which row strides and key splits change
+    # ones, and the single ones of 16 that small windows take; the head widths at which row strides and key splits change
     q, k, v = workloads.random_qkv(units, N, d, dtype, seed=units + N + d)
     # fp32 throughout: a few ulp of the longest sums (2^-24 x sqrt(1024) = 2e-6)
     _check(q, k, v, 2e-6 if dtype == "f32" else TOL[dtype])
