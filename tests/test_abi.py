@@ -326,3 +326,15 @@ def test_a_capture_allocates_nothing_beside_the_result(own, stream, monkeypatch)
     monkeypatch.setattr(torch.cuda, "stream", lambda s: contextlib.nullcontext())
     monkeypatch.setattr(torch, "empty", no_memory)
     assert nb._qkv_two_pass(x, w, 0, out, own, 2, 2, 1024, 32, 16, 6, 0, 0, 0, 0, 0, 1, stream) is None
+
+
+@pytest.mark.parametrize("heads,d,T,two", [(6, 30, 65536, True), (6, 30, 49152, True), (6, 30, 32768, False),
+                                           (4, 20, 65536, True), (4, 20, 65472, False), (8, 28, 65472, False),
+                                           (3, 32, 262144, False), (4, 32, 98304, True), (9, 32, 65536, False),
+                                           (10, 32, 262144, False), (20, 16, 262144, False), (11, 30, 65536, True)])
+def test_second_form_at_8x8_windows(heads, d, T, two):
+    # where it was measured to be the faster one: not for heads of 32 in short calls
+    # or few features, nor for 320 features
+    import torch
+    x, w, out = (torch.zeros(16, dtype=torch.bfloat16) for _ in range(3))
+    assert nb._two_pass(T // 64, 64, heads, d, 16, 6, "segments", x, w, None, None, 0, out, None) == two
