@@ -8,6 +8,12 @@ from paper_2506_08520_gb300 import binding
 
 # Max over units of ||O_gpu - O_ref||_F / ||O_ref||_F.
 TOL = {"f32": 1e-4, "bf16": 2e-2, "f16": 2e-2}
+# One rounding to the I/O type moves no element by more than this share of it
+# (half the spacing just above a power of two), and so no unit.  On soft inputs
+# that is what the output's own rounding makes of a kernel whose other errors are
+# those of fp32 or of 16-bit pairs (2^-16 at most); other 16-bit roundings on the
+# way (stored projections, probabilities, single 16-bit factors) count beside it.
+ROUND = {"f32": 1e-4, "bf16": 2.0 ** -8, "f16": 2.0 ** -11}
 DT = {torch.float32: "f32", torch.bfloat16: "bf16", torch.float16: "f16"}
 
 

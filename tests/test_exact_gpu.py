@@ -8,9 +8,12 @@ import torch
 
 import oracle
 from paper_2506_08520_gb300 import binding, workloads
-from tests.parity import TOL, per_unit_rel, units_view
+from tests.parity import ROUND, TOL, per_unit_rel, units_view
 
 pytestmark = pytest.mark.gpu
+
+# P and the output are rounded to 16 bits; fp32 I/O takes 16-bit pairs
+BAR = {"f32": TOL["f32"], "bf16": 2 * ROUND["bf16"], "f16": 2 * ROUND["f16"]}
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -34,7 +37,7 @@ def test_units_and_widths(units, N, d, dtype):
     if N == 1024 and dtype == "f32":
         pytest.skip("32x32 windows in fp32 take the generic kernel")
     q, k, v = workloads.random_qkv(units, N, d, dtype, seed=units + N + d)
-    _check(q, k, v, TOL[dtype])
+    _check(q, k, v, BAR[dtype])
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
@@ -44,7 +47,7 @@ def test_every_head_width(d, dtype):
     # one group per CTA, and (457 units) up to four, the last one idle in some
     for units, N in ((5, 64), (457, 64), (2, 256)):
         q, k, v = workloads.random_qkv(units, N, d, dtype, seed=units + N + d)
-        _check(q, k, v, TOL[dtype])
+        _check(q, k, v, BAR[dtype])
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
@@ -56,7 +59,7 @@ def test_late_maximum(N, dtype):
     T = workloads.DTYPES[dtype]
     k[:, -1] = 0.0
     q[..., 0], k[..., 0] = 4.0, torch.linspace(-30, 30, N)
-    _check(q.to(T), k.to(T), v.to(T), TOL[dtype])
+    _check(q.to(T), k.to(T), v.to(T), BAR[dtype])
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
@@ -68,7 +71,7 @@ def test_generic_tile_edges(units, N, d, dtype):
     # ones, and the single ones of 16 that small windows take; the head widths at which row strides and key splits change
     q, k, v = workloads.random_qkv(units, N, d, dtype, seed=units + N + d)
     # fp32 throughout: a few ulp of the longest sums (2^-24 x sqrt(1024) = 2e-6)
-    _check(q, k, v, 2e-6 if dtype == "f32" else TOL[dtype])
+    _check(q, k, v, 2e-6 if dtype == "f32" else ROUND[dtype])
 
 
 def _rounded_p(q, k, v, chunk):

@@ -10,7 +10,7 @@ import torch
 
 import oracle
 from paper_2506_08520_gb300 import binding, workloads
-from tests.parity import TOL, fused_qkv, per_unit_rel
+from tests.parity import ROUND, fused_qkv, per_unit_rel
 
 pytestmark = pytest.mark.gpu
 
@@ -55,7 +55,7 @@ def test_both_forms_match_the_oracle(nw, heads, N, d, m, lm, kind, dtype, monkey
     ref = oracle.nystra_attention(q, k, v, m, 5, lm, bb).reshape(-1, N, d)
     for out in (one, fused):
         err = per_unit_rel(out.cpu()[idx].double().numpy(), ref)
-        assert err.max() <= TOL[dtype], err.max()
+        assert err.max() <= 3 * ROUND[dtype], err.max()  # Q and K, V and the output are rounded
 
 
 def test_what_was_refused_stays_refused():

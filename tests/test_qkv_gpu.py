@@ -9,7 +9,7 @@ import torch
 
 import oracle
 from paper_2506_08520_gb300 import binding, workloads
-from tests.parity import TOL, fused_qkv, per_unit_rel, sample_units
+from tests.parity import ROUND, TOL, fused_qkv, per_unit_rel, sample_units
 
 pytestmark = pytest.mark.gpu
 
@@ -311,8 +311,8 @@ def test_fused_large_windows_many_windows_and_16bit_factors():
 def test_fused_two_warp_core_over_several_units(dtype, factors):
     """m = 32 at 32x32 windows: the core's two warps share scratch that the next
     unit's core uses again, and both buffers of a team's state.  Four units per
-    team (two teams on each of at most 160 SMs).  Sampled units; the bar is that of
-    m = 16 on the same soft inputs, per factor mode."""
+    team (two teams on each of at most 160 SMs).  Sampled units; Q and K, V and the
+    output are rounded, and with single 16-bit factors G_L, G_U, the landmarks and Y."""
     nw, N, heads, d, m = 640, 1024, 2, 32, 32
     x, w, b = workloads.random_x_wqkv(nw, N, heads, d, dtype, seed=78)
     idx = sample_units(nw * heads, 48)
@@ -326,4 +326,4 @@ def test_fused_two_warp_core_over_several_units(dtype, factors):
     assert binding.status() == binding.NYSTRA_OK
     err = per_unit_rel(out.reshape(nw * heads, N, d)[torch.from_numpy(idx)].cpu().double().numpy(), ref)
     print(f"m = 32, {dtype}, {factors}: max rel err {err.max():.3e}")
-    assert err.max() <= TOL[dtype], f"max rel err {err.max():.3e} at unit {int(idx[err.argmax()])}"
+    assert err.max() <= (3 if factors == "pairs" else 7) * ROUND[dtype], f"max rel err {err.max():.3e} at unit {int(idx[err.argmax()])}"

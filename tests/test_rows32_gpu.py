@@ -6,7 +6,7 @@ import torch
 
 import oracle
 from paper_2506_08520_gb300 import binding, workloads
-from tests.parity import TOL, per_unit_rel, units_view
+from tests.parity import ROUND, per_unit_rel, units_view
 
 pytestmark = pytest.mark.gpu
 
@@ -36,7 +36,9 @@ def test_every_feature_keeps_its_place(units, N, m, dtype, factors):
     out = units_view(out.cpu()).double().numpy() / s.double().numpy()
     ref = oracle.nystra_attention(q, k, v, m, 6) / s.double().numpy()
     err = per_unit_rel(out, ref)
-    assert err.max() <= TOL[dtype], f"{err.max():.3e} at unit {int(np.argmax(err))}"
+    # single 16-bit factors: G_L, G_U, the landmarks and Y are rounded too
+    bar = (1 if factors == "pairs" else 5) * ROUND[dtype]
+    assert err.max() <= bar, f"{err.max():.3e} at unit {int(np.argmax(err))}"
     col = np.linalg.norm(out - ref, axis=(0, 1)) / np.linalg.norm(ref, axis=(0, 1))
     # a column's own error: rounding of the output and of W's column, as for the whole
-    assert col.max() <= 2 * TOL[dtype], col.max()
+    assert col.max() <= 2 * bar, col.max()

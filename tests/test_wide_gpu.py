@@ -7,7 +7,7 @@ import torch
 
 import oracle
 from paper_2506_08520_gb300 import binding, workloads
-from tests.parity import TOL, per_unit_rel, units_view
+from tests.parity import ROUND, TOL, per_unit_rel, units_view
 
 pytestmark = pytest.mark.gpu
 
@@ -33,7 +33,8 @@ def _run(q, k, v, iters, factors="pairs"):
 def test_units_steps_and_widths(units, N, d, iters, dtype, factors):
     q, k, v = workloads.random_qkv(units, N, d, dtype, seed=N + d + iters)
     err = per_unit_rel(_run(q, k, v, iters, factors), oracle.nystra_attention(q, k, v, 64, iters))
-    assert err.max() <= TOL[dtype], f"{err.max():.3e} at unit {int(np.argmax(err))}"
+    # single 16-bit factors: G_L, G_U, the landmarks and Y are rounded too
+    assert err.max() <= (1 if factors == "pairs" else 5) * ROUND[dtype], f"{err.max():.3e} at unit {int(np.argmax(err))}"
 
 
 @pytest.mark.parametrize("dtype,lo,hi", [("bf16", -30, 30), ("f16", -10, 5)])
@@ -51,10 +52,12 @@ def test_columns_of_any_scale(N, dtype, lo, hi):
     b = _run(q, k, (v.float() * s).to(T), 6) / s.double().numpy()
     ref = oracle.nystra_attention(q, k, v, 64, 6)
     col = np.linalg.norm(b - ref, axis=1) / np.linalg.norm(ref, axis=1)
-    # fp16 outputs below 2^-14 are subnormal: 2^-25 absolute on outputs of about 0.1 2^lo
-    bar = TOL[dtype] if dtype == "bf16" else TOL[dtype] + 2.0 ** -25 / (0.02 * 2.0 ** lo)
+    # fp16 outputs below 2^-14 are subnormal: 2^-25 absolute on outputs of about 0.1 2^lo;
+    # and Y^T's fp16 pairs, at one scale, end 2^-39 below its largest entry, 2^-24 below
+    # those of the smallest column, which Z may exceed the output 10^4 times
+    bar = ROUND[dtype] if dtype == "bf16" else TOL[dtype] + 2.0 ** -25 / (0.02 * 2.0 ** lo)
     assert col.max() <= bar, col.max()
-    assert per_unit_rel(a, ref).max() <= TOL[dtype]
+    assert per_unit_rel(a, ref).max() <= ROUND[dtype]
 
 
 @pytest.mark.parametrize("N,m", [(64, 32), (64, 64), (256, 32), (256, 64), (1024, 32), (1024, 64)])
@@ -74,4 +77,4 @@ def test_landmarks_of_any_scale(N, m):
     out = units_view(out.cpu()).double().numpy() / s.double().numpy()
     ref = oracle.nystra_attention(q, k, v, m, 6)
     for rows in (slice(0, N // 2), slice(N // 2, N)):
-        assert per_unit_rel(out[:, rows], ref[:, rows]).max() <= TOL["bf16"]
+        assert per_unit_rel(out[:, rows], ref[:, rows]).max() <= ROUND["bf16"]
