@@ -459,17 +459,17 @@ nystra_generic_kernel(const T* q, const T* k, const T* v, T* out, long long n_un
 template <int MP, int DS, typename T>
 cudaError_t launch_ds(const void* q, const void* k, const void* v, void* out, long long n_units, int N, int d, int m,
                       int iters, int pool, cudaStream_t stream, const NystraBias& bias) {
-    static std::atomic<int> s_ready[kMaxDevices];
+    static std::atomic<int> s_sms[kMaxDevices];
     auto kern = nystra_generic_kernel<MP, DS, T>;
-    if (cudaError_t e = opt_in_smem(kern, s_ready); e != cudaSuccess) return e;
+    int sms = 0;
+    if (cudaError_t e = opt_in_smem(kern, s_sms, &sms); e != cudaSuccess) return e;
     int pw = 0;  // window width for square patches
     if (pool != 0)
         while ((pw + 1) * (pw + 1) <= N) ++pw;
-    // Few units, a CTA or so per SM: at least four warps, for a unit's latency (108
-    // units of 7x7 windows, m = 7: 33 us with one warp, 22 with four); else the
+    // Few units, up to four CTAs per SM: at least four warps, for a unit's latency
+    // (108 units of 7x7 windows, m = 7: 33 us with one warp, 22 with four); else the
     // tiles' threads only, for more CTAs per SM.
-    constexpr long long kFewUnits = 4 * 152;
-    const Shape<MP, DS> G(N, d, n_units <= kFewUnits ? 128 : 32);
+    const Shape<MP, DS> G(N, d, n_units <= 4LL * sms ? 128 : 32);
     const long long grid = n_units < (1LL << 30) ? n_units : (1LL << 30);
     kern<<<(unsigned)grid, G.threads, G.bytes(), stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)out, n_units, N, d,
                                                            m, iters, pw, 1.0f / sqrtf((float)d), bias);

@@ -9,19 +9,22 @@ namespace simt {
 
 constexpr size_t kSmemLimit = 232448;  // opt-in dynamic shared memory per CTA
 
-// Opts `kern` in to kSmemLimit once per device; `ready` is a zero-initialised
-// static of the launcher.
+// Opts `kern` in to kSmemLimit once per device; `cache` is a zero-initialised
+// static of the launcher that keeps the device's number of SMs, returned in *sms.
 template <typename K>
-cudaError_t opt_in_smem(K kern, std::atomic<int> (&ready)[kMaxDevices]) {
+cudaError_t opt_in_smem(K kern, std::atomic<int> (&cache)[kMaxDevices], int* sms = nullptr) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    if (ready[dev].load(std::memory_order_relaxed) == 0) {
+    int n = cache[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
         if (e != cudaSuccess) return e;
-        ready[dev].store(1, std::memory_order_relaxed);
+        if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        cache[dev].store(n, std::memory_order_relaxed);
     }
+    if (sms) *sms = n;
     return cudaSuccess;
 }
 
