@@ -31,9 +31,9 @@
 //            written as partial sectors); [P2] S_L and G_L^n recomputed from
 //            a still-resident Q.
 //
-// Grouped kernel (nystra_tc_kernel; m = 32 at 8x8 windows, m = 64 at 32x32).  A group of token warps owns one unit at a time, plus
-// helper warps when the core needs more warps than there are
-// token warps; a CTA holds GROUPS groups and the grid is persistent.  The
+// Grouped kernel (nystra_tc_kernel; m = 32 at 8x8 windows, m = 64 at 32x32).  A
+// group of token warps, one or four, owns one unit at a time and runs its core
+// too; a CTA holds GROUPS groups and the grid is persistent.  The
 // next unit's Q and K are copied after the combine ([P2]: K only, Q after the
 // output), V once the output store has read its staging.  P1 ("G_L parked")
 // is used when it fits as many groups as P2.
@@ -138,33 +138,32 @@ struct GlPark;  // parked G_L^n fragments (defined with the front phase)
 
 template <typename T, int M, int NCOL, int TPW, int WPU, bool GLS, int CW = 1>
 struct Layout {
+    static_assert((M == 32 && WPU == 1 && CW == 1) || (M == 64 && WPU == 4 && CW == 4),
+                  "one warp a unit, its core included, or four token warps that run the core too");
     static constexpr int N = TPW * WPU;
-    static constexpr int GW = WPU > CW ? WPU : CW;       // warps per group (token warps first)
     static constexpr int NCH = TPW / 64;                 // 64-token chunks per warp
     static constexpr int DS = (NCOL == 32) ? 30 : 32;    // staged row width bound (d_h <= DS)
-    static constexpr int MT = (M + 15) / 16;             // landmark m-tiles
-    static constexpr int MP = MT * 16;                   // padded landmark count
+    static constexpr int MT = M / 16;                    // landmark m-tiles
     static constexpr int LS = LmS<T>::LS;                // Qbar/Kbar row stride
     static constexpr int WS = NCOL + 4;                  // fp32 W row stride
     static constexpr int YS = YtS<T, M>::YS;             // Y^T row stride
-    static constexpr int KTL = (M >= 16) ? M / 16 : 1;   // k-steps of O = G_L^n Y
+    static constexpr int KTL = M / 16;                   // k-steps of O = G_L^n Y
     static constexpr int GLB = GlPark<T, M>::BYTES;      // bytes per lane per G_L fragment
     // per-warp private memory: stage (Q, K, V rows of the warp), G_L fragments
     static constexpr size_t STAGE = 3 * (size_t)TPW * DS * 2;
     static constexpr size_t GLF = STAGE;
     static constexpr size_t WARP_BYTES = ((GLF + (GLS ? (size_t)NCH * 4 * KTL * 32 * GLB : 0) + 127) / 128) * 128;
-    // A warp's partial W (fp32 MP x NCOL, row stride WS, then MP row maxima)
+    // A warp's partial W (fp32 M x NCOL, row stride WS, then M row maxima)
     // lives in its stage right after the Q rows, once K and V are consumed.
     static constexpr size_t WPART = (size_t)TPW * DS * 2;
-    static_assert(WPU == 1 || (size_t)MP * WS * 4 + MP * 4 <= 2 * (size_t)TPW * DS * 2,
+    static_assert(WPU == 1 || (size_t)M * WS * 4 + M * 4 <= 2 * (size_t)TPW * DS * 2,
                   "W partial must fit in K+V");
     // The core on several warps (CW > 1, m = 64) has its scratch in the first two
     // token warps' K/V rows (consumed by the combine before the core starts; the
     // next unit's K and V are copied after the core).
-    static_assert(CW == 1 || (M == 64 && CW == 4 && WPU >= 2 &&
-                              ScScratch<64>::MAT + ScScratch<64>::AUX <= 2 * (size_t)TPW * DS * 2),
+    static_assert(CW == 1 || ScScratch<64>::MAT + ScScratch<64>::AUX <= 2 * (size_t)TPW * DS * 2,
                   "scratch must fit in two warps' K/V rows");
-    static constexpr size_t QB_BYTES = LmS<T>::bytes(MP);
+    static constexpr size_t QB_BYTES = LmS<T>::bytes(M);
     static constexpr size_t YT_BYTES = YtS<T, M>::bytes(NCOL);
     // Per-group shared memory: Qbar | W | m_U | Kbar (| Y^T) | bars.  Y^T is
     // written by the core once every core warp has read Qbar, W and m_U for the
@@ -174,9 +173,9 @@ struct Layout {
     // the next unit's Q lands).
     static constexpr bool YT_OVERLAY = (WPU == 1) || !GLS;
     static constexpr size_t G_QBAR = 0;
-    static constexpr size_t G_W = QB_BYTES;            // fp32 MP x WS
-    static constexpr size_t G_MU = G_W + MP * WS * 4;  // m_U, log2 domain
-    static constexpr size_t G_KBAR = ((G_MU + MP * 4 + 15) / 16) * 16;
+    static constexpr size_t G_W = QB_BYTES;            // fp32 M x WS
+    static constexpr size_t G_MU = G_W + M * WS * 4;  // m_U, log2 domain
+    static constexpr size_t G_KBAR = ((G_MU + M * 4 + 15) / 16) * 16;
     static constexpr size_t G_BAR =
         (((YT_OVERLAY ? G_KBAR + QB_BYTES : G_KBAR + QB_BYTES + YT_BYTES) + 15) / 16) * 16;
     static constexpr size_t G_BAR_END = G_BAR + 16 * WPU;  // two mbarriers per token warp
@@ -727,11 +726,8 @@ __device__ __forceinline__ void su_w_chunk(const typename Opnd<T>::DReg (&aq)[2]
         } else {
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
-                if constexpr (RS == 1 || RS == kSlots)
-                    b[nt] = real ? __ldg(reinterpret_cast<const float2*>(p + 8 * nt + 2 * t)) : make_float2(0.f, 0.f);
-                else
-                    b[nt] = real ? make_float2(__ldg(p + ctok<RS>(nt, 2 * t)), __ldg(p + ctok<RS>(nt, 2 * t + 1)))
-                                 : make_float2(0.f, 0.f);
+                static_assert(RS == 1 || RS == 4 || RS == kSlots, "keys 2t and 2t + 1 of an n-tile are neighbours");
+                b[nt] = real ? __ldg(reinterpret_cast<const float2*>(p + 8 * nt + 2 * t)) : make_float2(0.f, 0.f);
             }
         }
     };
@@ -1303,27 +1299,23 @@ __device__ __forceinline__ void output_rows(const uint32_t* glf, const T* Qs, co
 }
 
 template <typename T, int M, int NCOL, int TPW, int WPU, int GROUPS, bool GLS, int CW>
-__global__ void __launch_bounds__(GROUPS * Layout<T, M, NCOL, TPW, WPU, GLS, CW>::GW * 32, 1)
+__global__ void __launch_bounds__(GROUPS * WPU * 32, 1)
 nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                  T* __restrict__ out, long long n_units, int d, int iters, float sl2,
                  unsigned int* fault, int active) {
     using Lay = Layout<T, M, NCOL, TPW, WPU, GLS, CW>;
-    constexpr int N = Lay::N, NCH = Lay::NCH, MT = Lay::MT, MP = Lay::MP, WS = Lay::WS, KTL = Lay::KTL,
-                  GW = Lay::GW;
+    constexpr int N = Lay::N, NCH = Lay::NCH, MT = Lay::MT, WS = Lay::WS, KTL = Lay::KTL;
     constexpr int L = N / M;      // tokens per landmark segment (<= TPW)
     constexpr int LPW = TPW / L;  // landmarks owned by one warp
     static_assert(sizeof(T) == 2, "the grouped kernel takes 16-bit I/O (its layout assumes it)");
     static_assert(L <= TPW && TPW % L == 0, "segments must not straddle warps");
-    static_assert(CW == 1 || CW == M / 16, "a core on several warps has one per 16 landmarks");
 
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int grp = warp / GW, r = warp - grp * GW;
-    const bool tok = (GW == WPU) || r < WPU;  // token warp (owns TPW tokens); others only help the core
+    const int grp = warp / WPU, r = warp - grp * WPU;
     const int g = lane >> 2, t = lane & 3;
     unsigned char* gb = smem_raw + (size_t)grp * Lay::GROUP_BYTES;
-    unsigned char* wb = smem_raw + (size_t)GROUPS * Lay::GROUP_BYTES +
-                        (size_t)(grp * WPU + (r < WPU ? r : WPU - 1)) * Lay::WARP_BYTES;
+    unsigned char* wb = smem_raw + (size_t)GROUPS * Lay::GROUP_BYTES + (size_t)(grp * WPU + r) * Lay::WARP_BYTES;
     const int td = TPW * d;  // elements per staged tensor
     T* Qs = reinterpret_cast<T*>(wb);
     T* Ks = Qs + td;
@@ -1339,16 +1331,16 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
     uint64_t* barV = barQK + 1;                                                // V rows
 
     auto gsync = [&]() {
-        if constexpr (GW == 1) __syncwarp();
-        else named_barrier(1 + grp, GW * 32);
+        if constexpr (WPU == 1) __syncwarp();
+        else named_barrier(1 + grp, WPU * 32);
     };
     // group barrier that also tells every warp whether any warp's wait gave up
     auto gsync_or = [&](bool f) -> bool {
-        if constexpr (GW == 1) {
+        if constexpr (WPU == 1) {
             __syncwarp();
             return f;
         } else {
-            return named_barrier_or(1 + grp, GW * 32, f);
+            return named_barrier_or(1 + grp, WPU * 32, f);
         }
     };
     // scratch of the core on several warps
@@ -1377,25 +1369,25 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
         bulk_g2s(Vs, v + unit_off(unit), tile_bytes, barV);
     };
 
-    if (tok && lane == 0) {
+    if (lane == 0) {
         mbar_init(barQK, 1);
         mbar_init(barV, 1);
         fence_mbar_init();
     }
     gsync();
-    if (tok && u < n_units && lane == 0) {
+    if (u < n_units && lane == 0) {
         arm_qk();
         issue_q(u);
         issue_k(u);
         issue_v(u);
     }
     uint32_t phase_qk = 0, phase_v = 0;
-    bool pend_qk = tok && u < n_units, pend_v = pend_qk;  // copies issued and not yet seen complete
+    bool pend_qk = u < n_units, pend_v = pend_qk;  // copies issued and not yet seen complete
     bool failed = false;  // a bounded wait of this warp gave up (warp-uniform)
 
     for (; u < n_units; u += stride) {
         // ---------------- stage: bounded wait for Q and K ----------------
-        if (tok && !failed) {
+        if (!failed) {
             if (__all_sync(0xffffffffu, mbar_wait_bounded(barQK, phase_qk, kWaitNs))) {
                 phase_qk ^= 1u;
                 pend_qk = false;
@@ -1406,18 +1398,12 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
         }
 
         // ---------------- front: landmarks (Algorithm 1 step 1) ----------------
-        if (tok) {
-            landmarks_mma<T, TPW, L>(Qs, qbar, r * LPW, d, g, t);
-            landmarks_mma<T, TPW, L>(Ks, kbar, r * LPW, d, g, t);
-            if (M < MP && r == 0) {  // zero the padding landmark rows
-                landmarks_zero<T>(qbar, M, MP, lane, 32);
-                landmarks_zero<T>(kbar, M, MP, lane, 32);
-            }
-        }
+        landmarks_mma<T, TPW, L>(Qs, qbar, r * LPW, d, g, t);
+        landmarks_mma<T, TPW, L>(Ks, kbar, r * LPW, d, g, t);
         if (gsync_or(failed)) break;
 
         // ---------------- front [P1]: S_L, G_L^n fragments ----------------
-        if (GLS && tok) {
+        if constexpr (GLS) {
 #pragma unroll 1
             for (int ch = 0; ch < NCH; ++ch)
 #pragma unroll
@@ -1431,7 +1417,7 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
         }
 
         // ---------------- stage: bounded wait for V ----------------
-        if (tok && !failed) {
+        if (!failed) {
             if (__all_sync(0xffffffffu, mbar_wait_bounded(barV, phase_v, kWaitNs))) {
                 phase_v ^= 1u;
                 pend_v = false;
@@ -1440,30 +1426,27 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
                 if (lane == 0) atomicOr(fault, 1u);
             }
         }
-        if (GW == 1 && failed) break;
+        if (WPU == 1 && failed) break;
 
         // ------- front: S_U, running m_U, G_U^n, W_r = G_U^n [V | 1] -------
         float mU[MT][2];  // this warp's row maxima of S_U, log2 domain
-        if (tok) {
-            front_su_w<T, M, NCOL, NCH>(qbar, Ks, Vs, d, g, t, sl2, WPU == 1 ? mW : wpart, WS, mU);
-            if ((WPU > 1 || CW > 1) && t == 0) {
-                float* mdst = WPU > 1 ? wpart + MP * WS : gmu;
+        front_su_w<T, M, NCOL, NCH>(qbar, Ks, Vs, d, g, t, sl2, WPU == 1 ? mW : wpart, WS, mU);
+        if (WPU > 1 && t == 0) {
+            float* mdst = wpart + M * WS;
 #pragma unroll
-                for (int mt = 0; mt < MT; ++mt) {
-                    mdst[16 * mt + g] = mU[mt][0];
-                    mdst[16 * mt + g + 8] = mU[mt][1];
-                }
+            for (int mt = 0; mt < MT; ++mt) {
+                mdst[16 * mt + g] = mU[mt][0];
+                mdst[16 * mt + g + 8] = mU[mt][1];
             }
         }
 
         // ---------------- combine (WPU > 1) ----------------
         if constexpr (WPU > 1) {
             gsync();
-            if (tok)
-                combine_partials<MP, NCOL, WS, WPU>(
-                    reinterpret_cast<const float*>(smem_raw + (size_t)GROUPS * Lay::GROUP_BYTES +
-                                                   (size_t)(grp * WPU) * Lay::WARP_BYTES + Lay::WPART),
-                    Lay::WARP_BYTES / 4, mW, gmu, r, lane);
+            combine_partials<M, NCOL, WS, WPU>(
+                reinterpret_cast<const float*>(smem_raw + (size_t)GROUPS * Lay::GROUP_BYTES +
+                                               (size_t)(grp * WPU) * Lay::WARP_BYTES + Lay::WPART),
+                Lay::WARP_BYTES / 4, mW, gmu, r, lane);
         }
         if (gsync_or(failed)) break;
 
@@ -1474,7 +1457,7 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
         auto prefetch_qk = [&]() {
             fence_proxy_async_smem();  // this lane's reads of Q/K precede the async refill
             __syncwarp();
-            if (tok && un < n_units && !failed) {
+            if (un < n_units && !failed) {
                 if (lane == 0) {
                     arm_qk();
                     if constexpr (GLS) issue_q(un);
@@ -1487,39 +1470,26 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
 
         // ---------------- core: G_A^n, Z_0, iteration, Y ----------------
         if constexpr (CW == 1) {
-            if (r == 0) {
-                if constexpr (WPU > 1) {
-#pragma unroll
-                    for (int mt = 0; mt < MT; ++mt) {
-                        mU[mt][0] = gmu[16 * mt + g];
-                        mU[mt][1] = gmu[16 * mt + g + 8];
-                    }
-                }
-                core_warp<T, M, NCOL>(qbar, kbar, mU, mW, yT, iters, sl2, g, t);
-            }
+            core_warp<T, M, NCOL>(qbar, kbar, mU, mW, yT, iters, sl2, g, t);
         } else {
-            if (r < CW) {
-                float w[NCOL / 8][4];
-                sc_core<T, M, NCOL, false>(qbar, kbar, gmu[16 * r + g], gmu[16 * r + g + 8], w, yT, mat0, mat1, mW, aux,
-                                           iters, sl2, r, lane, 1 + GROUPS + grp);
-            }
+            float w[NCOL / 8][4];
+            sc_core<T, M, NCOL, false>(qbar, kbar, gmu[16 * r + g], gmu[16 * r + g + 8], w, yT, mat0, mat1, mW, aux,
+                                       iters, sl2, r, lane, 1 + GROUPS + grp);
         }
         gsync();
         if constexpr (CW > 1) prefetch_qk();
 
-        if (tok) {
-            // ---------------- output: O = (G_L^n Y_:d) / (G_L^n Y_d) ----------------
-            output_rows<T, M, NCOL, NCH, GLS>(glf, Qs, kbar, yT, Vs, d, g, t, lane, sl2);
+        // ---------------- output: O = (G_L^n Y_:d) / (G_L^n Y_d) ----------------
+        output_rows<T, M, NCOL, NCH, GLS>(glf, Qs, kbar, yT, Vs, d, g, t, lane, sl2);
 
-            // The output rows are staged in V's region: one bulk store, and once it
-            // has read shared memory, the next unit's V can land there.
-            fence_proxy_async_smem();  // this lane's staging writes precede the bulk store
-            __syncwarp();
-            if (lane == 0) {
-                bulk_s2g(out + unit_off(u), Vs, tile_bytes);
-                bulk_commit();
-                bulk_wait_read_all();
-            }
+        // The output rows are staged in V's region: one bulk store, and once it
+        // has read shared memory, the next unit's V can land there.
+        fence_proxy_async_smem();  // this lane's staging writes precede the bulk store
+        __syncwarp();
+        if (lane == 0) {
+            bulk_s2g(out + unit_off(u), Vs, tile_bytes);
+            bulk_commit();
+            bulk_wait_read_all();
         }
         // [P2] Q was needed until now: every warp of the group is done reading
         // the landmarks before anyone overwrites them.
@@ -1527,7 +1497,7 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
             fence_proxy_async_smem();  // reads of Q precede its refill
             gsync();
         }
-        if (tok && un < n_units && !failed) {
+        if (un < n_units && !failed) {
             if (lane == 0) {
                 if constexpr (!GLS) issue_q(un);
                 issue_v(un);
@@ -1536,19 +1506,19 @@ nystra_tc_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __re
         }
         __syncwarp();
     }
-    if (tok && lane == 0) bulk_wait_all();  // outstanding output stores complete before exit
+    if (lane == 0) bulk_wait_all();  // outstanding output stores complete before exit
     // Fault path only: copies still in flight land before the CTA's memory is released.
-    if (tok && pend_qk) (void)__all_sync(0xffffffffu, mbar_wait_bounded(barQK, phase_qk, kWaitNs));
-    if (tok && pend_v) (void)__all_sync(0xffffffffu, mbar_wait_bounded(barV, phase_v, kWaitNs));
+    if (pend_qk) (void)__all_sync(0xffffffffu, mbar_wait_bounded(barQK, phase_qk, kWaitNs));
+    if (pend_v) (void)__all_sync(0xffffffffu, mbar_wait_bounded(barV, phase_v, kWaitNs));
 }
 
 // Largest number of groups per CTA that fits the shared-memory and register
-// budgets (M <= 16 needs about 160 registers per thread, M = 32 about 255).
+// budgets (eight warps of up to 255 registers).
 template <typename T, int M, int NCOL, int TPW, int WPU, bool GLS, int CW>
 constexpr int groups_that_fit() {
     using Lay = Layout<T, M, NCOL, TPW, WPU, GLS, CW>;
     const int by_smem = (int)(kSmemLimit / Lay::PER_GROUP);
-    const int by_regs = ((M <= 16) ? 12 : 8) / Lay::GW;
+    const int by_regs = 8 / WPU;
     const int n = by_smem < by_regs ? by_smem : by_regs;
     const int cap = (CW > 1) ? 7 : 15;  // named barriers: 1 + group barriers + core barriers <= 16
     return n > cap ? cap : n;
@@ -1568,7 +1538,7 @@ cudaError_t launch_cfg(const void* q, const void* k, const void* v, void* out, l
     const size_t smem = (size_t)kGroups * Lay::PER_GROUP;
     static std::atomic<int> s_blocks[kMaxDevices];  // persistent grid size per device
     int blocks = 0;
-    if (cudaError_t e = persistent_grid(kern, kGroups * Lay::GW * 32, smem, s_blocks, &blocks); e != cudaSuccess)
+    if (cudaError_t e = persistent_grid(kern, kGroups * WPU * 32, smem, s_blocks, &blocks); e != cudaSuccess)
         return e;
     // Wave quantisation: every group processes ceil(units / groups) units, so
     // use the fewest groups per CTA that still reach the minimal number of
@@ -1579,7 +1549,7 @@ cudaError_t launch_cfg(const void* q, const void* k, const void* v, void* out, l
     const long long want = (n_units + active - 1) / active;
     const long long grid = want < blocks ? want : blocks;
     const float sl2 = 1.4426950408889634f / sqrtf((float)d);
-    kern<<<(unsigned)grid, kGroups * Lay::GW * 32, smem, stream>>>((const T*)q, (const T*)k, (const T*)v,
+    kern<<<(unsigned)grid, kGroups * WPU * 32, smem, stream>>>((const T*)q, (const T*)k, (const T*)v,
                                                                   (T*)out, n_units, d, iters, sl2, fault, active);
     return cudaGetLastError();
 }

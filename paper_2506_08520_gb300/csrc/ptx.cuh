@@ -198,12 +198,6 @@ __device__ __forceinline__ void ldsm_x2(uint32_t (&r)[2], const void* p) {
                  : "r"(smem_addr(p))
                  : "memory");
 }
-__device__ __forceinline__ void ldsm_x2_t(uint32_t (&r)[2], const void* p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
-                 : "=r"(r[0]), "=r"(r[1])
-                 : "r"(smem_addr(p))
-                 : "memory");
-}
 // Max over the warp of non-negative floats: their bit patterns order like
 // unsigned integers, so one redux.sync does it.
 __device__ __forceinline__ float warp_max_nonneg(float x) {
