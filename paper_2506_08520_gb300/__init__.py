@@ -10,7 +10,7 @@ layer's weight ``w_qkv`` ``[3 heads d_h, heads d_h]`` (16-bit)::
     pooled = pn.pool_bias(bias, m=16)                          # bias [heads, N, N] fp32, once
     o = pn.nystra_biased(q, k, v, pooled, m=16, iters=6)       # with a score bias
     e = pn.exact(q, k, v)                                      # exact window attention
-    o = pn.nystra_qkv(x, w_qkv, heads=6, b_qkv=b)              # fused Q/K/V projection
+    o = pn.nystra_qkv(x, w_qkv, heads=6, b_qkv=b)              # Q/K/V projection in front
     q, k, v = pn.project_qkv(x, w_qkv, heads=6, b_qkv=b)       # the projection alone (tcgen05)
 
 Every call goes through the C ABI of ``libnystra.so`` (``include/nystra.h``),

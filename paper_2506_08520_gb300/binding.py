@@ -1,7 +1,8 @@
-"""Thin ctypes binding of ``libnystra.so`` (C ABI in ``include/nystra.h``).
+"""ctypes binding of ``libnystra.so`` (C ABI in ``include/nystra.h``).
 
-Argument marshalling only: every step of the computation runs in the CUDA
-kernels behind the C ABI.  torch is used for device memory and streams.
+Argument marshalling, and for ``nystra_qkv`` the choice between two forms of the
+same computation; every step of it runs in the CUDA kernels behind the C ABI.
+torch is used for device memory and streams.
 There is no CPU fallback: if the library is missing, every call raises.
 """
 from __future__ import annotations
@@ -362,20 +363,21 @@ def _two_pass(nw, N, heads, d, m, iters, landmarks, x, w_qkv, b_qkv, pooled, bw,
     stream the workspace can be allocated for.
 
     The lines, from times of both forms (m = 16, bf16, fused / two-pass, us a call
-    among others; a call that is waited for pays about 10 more for the second form's
-    host work).  32x32 windows everywhere (1 x 16 features, 2048 tokens 48/33; 6 x
-    30, 262144 tokens 706/240).  16x16 windows from 128 token features on (4 x 32,
-    2048 tokens 50/34; 6 x 30, 262144 tokens 586/248) or 64 and 65536 tokens (2 x
-    32: 62/52, 3 x 32: 70/71, the one tie; but 1 x 32: 27/33, and at 2048 tokens 4 x
-    24: 33/29, waited for 42/48).  8x8 windows from 80 features and 65536 tokens on
-    (4 x 20: 61/56, 4 x 30: 74/57, 8 x 30: 177/149, 11 x 30: 313/308; but 2 x 32: 43/50,
-    and at 32768 tokens 4 x 20: 33/40, 8 x 28: 92/99, 11 x 30: 158/169), up to 180
-    features from 8e6 token features on (6 x 30, 45056 tokens 99/65, 5 x 30, 57344
-    tokens 98/81; at 24576 tokens 62/44, waited for 71/64, and 42/48).  There heads of 32 from 128 features and 98304 tokens on (4 x 32: 132/134 and, 131072 tokens,
-    173/164, 8 x 32: 337/305; but 3 x 32: 100/108, 223/233 at 262144 tokens, and 9 x 32,
-    65536 tokens: 264/274), and not where a CTA of the projection has room for the
-    weights of one head only and its rows of a multiple of 128 bytes for no
-    conflict-free read (10 x 32, 65536 tokens: 322/405, 20 x 16: 502/732)."""
+    among others; a call that is waited for pays about 10 more for the second
+    form's host work).  32x32 windows everywhere (1 x 16 features, 2048 tokens
+    48/33; 6 x 30, 262144 tokens 706/240).  16x16 windows from 128 token features on
+    (4 x 32, 2048 tokens 50/34; 6 x 30, 262144 tokens 586/248) or 64 and 65536 tokens
+    (2 x 32: 62/52, 3 x 32: 70/71, the one tie; but 1 x 32: 27/33, and at 2048 tokens
+    4 x 24: 33/29, waited for 42/48).  8x8 windows from 80 features and 65536 tokens
+    on (4 x 20: 61/56, 4 x 30: 74/57, 8 x 30: 177/149, 11 x 30: 313/308; but 2 x 32:
+    43/50, and at 32768 tokens 4 x 20: 33/40, 8 x 28: 92/99, 11 x 30: 158/169), up to
+    180 features from 8e6 token features on (6 x 30, 45056 tokens 99/65, 5 x 30, 57344
+    tokens 98/81; at 24576 tokens 62/44, waited for 71/64, and 42/48).  There heads of
+    32 from 128 features and 98304 tokens on (4 x 32: 132/134 and, 131072 tokens,
+    173/164, 8 x 32: 337/305; but 3 x 32: 100/108, 223/233 at 262144 tokens, and 9 x
+    32, 65536 tokens: 264/274), and not 320 features (10 x 32, 65536 tokens: 322/405, 20
+    x 16: 502/732): the projection's CTAs hold one head's weights there, so the tokens
+    are read once a head, from rows that all start in one bank."""
     C, T = heads * d, nw * N
     if N == 64:
         faster = C >= 80 and (T >= 65536 or (C <= 180 and C * T >= 8e6)) and not (C > 256 and C % 64 == 0)

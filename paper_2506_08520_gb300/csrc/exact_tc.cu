@@ -18,9 +18,9 @@
 // log2(e)/sqrt(d_h) so each exponential is half a packed FMA and one ex2.  This
 // is the computation PnP-Nystra replaces; it is the in-library comparator.
 //
-// What bounds it: at 32x32 windows the tensor pipe, 69% busy (32 MMAs and 32
-// ex2 per warp for 32 rows and 32 keys); at 16x16 windows also laying out K and
-// V, at 8x8 windows HBM.  The next unit's rows are brought to L2 meanwhile.
+// What bounds it: at 32x32 windows the tensor pipe, 61% busy (32 MMAs and 32
+// ex2 per warp for 32 rows and 32 keys); at 16x16 windows (53%) also laying out
+// K and V, at 8x8 windows HBM.  The next unit's rows are brought to L2 meanwhile.
 // Measured (d_h = 30, bf16) against fragments loaded from 60-byte rows by one
 // 16-row tile: 5520 units of 32x32 windows 3.34 -> 2.02 ms, 6144 of 16x16
 // 271 -> 176 us, 86400 of 8x8 269 -> 224 us; fp32, 2000 units of 16x16: 502 ->

@@ -27,8 +27,8 @@
 // one warp's (no CTA barriers); the other CTAs of the SM fill its wait.
 //
 // What bounds it: instruction issue and shared-memory latency (12x12 windows,
-// m = 16, fp16: 40,000 warp instructions per unit, 0.48 issued per cycle, 19
-// warps per SM, DRAM 5%), so chunks are as long as one score tile per thread
+// m = 16, fp16: 43,000 warp instructions per unit, 0.51 issued per cycle, 19
+// warps per SM, DRAM 6%), so chunks are as long as one score tile per thread
 // allows: chunks of 72 and 88 tokens with more CTAs per SM were 4-12% slower.
 // Measured: 6144 units of 16x16 windows, d_h = 30, m = 16, fp32 1.52 -> 0.62 ms
 // (1.2 TB/s of Q, K, V, O); 11094 units of 12x12, fp16 1.62 -> 0.76 ms; 1668

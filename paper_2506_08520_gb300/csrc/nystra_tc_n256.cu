@@ -1,7 +1,5 @@
 // Tensor-core PnP-Nystra kernels for windows of 256 tokens: the team kernel
-// (nystra_team.cuh) for m <= 32, the grouped kernel (nystra_tc.cuh, four
-// warps of 64 tokens per unit) for m = 32 with d_h = 32, the wide kernel
-// (nystra_wide.cuh) for m = 64.
+// (nystra_team.cuh) for m <= 32, the wide kernel (nystra_wide.cuh) for m = 64.
 #include "nystra_tc.cuh"
 #include "nystra_team.cuh"
 #include "nystra_wide.cuh"

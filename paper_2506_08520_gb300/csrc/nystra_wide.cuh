@@ -1,14 +1,15 @@
 // Wide-landmark PnP-Nystra kernel: m = 64 at 8x8 and 16x16 windows (N = 64,
-// 256 tokens), even d_h <= 32, 16-bit I/O, segment landmarks.  Included by the N = 64 and 256 translation units after
-// nystra_tc.cuh, whose per-phase device functions it reuses.
+// 256 tokens), even d_h <= 32, 16-bit I/O, segment landmarks.  Included by the N =
+// 64 and 256 translation units after nystra_tc.cuh, whose per-phase device
+// functions it reuses.
 //
 // With so many landmarks the m x m core dominates a unit, so a unit's group is
 // the core's CW = m/16 warps, and they share the token side too, by landmarks:
 //   stage    Q, K, V of the unit by three bulk copies on two mbarriers;
 //   front    landmark means, every warp a share; [sync]; warp c: S_U of its 16
-//            landmarks against all tokens, its rows of W stay in registers in
-//            the very layout the core takes (no partial W, no combine);
-//   core     sc_core; its scratch overlays K, V and Qbar, Y^T one of its
+//            landmarks against all tokens, its rows of W in registers (no partial
+//            W, no combine);
+//   core     sc_core; its scratch overlays K and V, W Qbar, Y^T one of its
 //            matrices; [sync]
 //   output   every warp a share of the 16-token tiles: S_L, G_L^n from the
 //            resident Q, O in place over Q; [sync]; one bulk store.
@@ -16,6 +17,8 @@
 // a group per SM, and the SM's other groups fill the wait.  Three groups of
 // four warps run per SM (73 KB each at N = 256), against two groups with 108 KB
 // and two token warps each on the grouped kernel.
+// What bounds it: dependent MMAs and the tensor pipe (63% busy at 16x16 windows,
+// 0.40 instructions issued per cycle, LSU data pipe 66%).
 // Measured (bf16): 4096 units of 16x16 windows, d_h = 32: 0.92 -> 0.45 ms; 8640
 // units of 8x8 windows, d_h = 30: 1.44 -> 0.72 ms.
 //
@@ -37,7 +40,7 @@ struct WideLayout {
     static constexpr size_t G_Q = 0;
     static constexpr size_t G_KV = ROWS;  // K, V; the core's two matrices
     static constexpr size_t KV = ((2 * ROWS > 2 * Sc::MAT ? 2 * ROWS : 2 * Sc::MAT) + 15) / 16 * 16;
-    static constexpr size_t G_QV = G_KV + KV;  // Qbar; the core's W
+    static constexpr size_t G_QV = G_KV + KV;  // Qbar; W
     static constexpr size_t WMAT = (size_t)M * (NCOL + 4) * 4;
     static constexpr size_t QV = LmS<T>::bytes(M) > WMAT ? LmS<T>::bytes(M) : WMAT;
     static constexpr size_t G_KBAR = G_QV + QV;

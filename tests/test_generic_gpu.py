@@ -59,8 +59,8 @@ def test_generic_score_bias(N, d, m, per_window):
 
 @pytest.mark.parametrize("N,d,m", [(5, 3, 5), (49, 30, 7), (36, 20, 4), (81, 16, 9)])
 def test_generic_few_and_many_units(N, d, m):
-    # up to 608 units a CTA has four warps at least, above only its tiles'
-    # threads: the sums are the same
+    # up to four units per SM (608 on 152 SMs) a CTA has four warps at least, above
+    # only its tiles' threads: the sums are the same
     q, k, v = workloads.random_qkv(609, N, d, "f32", seed=N + d)
     out = binding.nystra(q.cuda(), k.cuda(), v.cuda(), m, 5)
     few = binding.nystra(q[1:].cuda(), k[1:].cuda(), v[1:].cuda(), m, 5)

@@ -45,9 +45,9 @@ def _errors(q, k, v, m, iters, factors="pairs"):
 
 # Every tensor-core kernel family with 16-bit I/O: the stage-pool kernel
 # (8x8 windows), the team kernel (16x16), the streaming kernel (32x32), each
-# with the one-warp core (m <= 16) and, where it has one, the distributed core
-# (m = 32); the grouped kernel (m = 32 at 8x8 and, with d_h = 32, at 16x16;
-# every m = 64).
+# with the one-warp core (m <= 16) and, where it has one, the two-warp core (m =
+# 32); the grouped kernel (m = 32 at 8x8, m = 64 at 32x32) and the wide kernel (m =
+# 64 at 8x8 and 16x16).
 FAMILIES = [
     # N, d, m, dtype, units
     (64, 30, 16, "bf16", 48), (64, 32, 8, "f16", 48),
