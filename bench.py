@@ -39,17 +39,18 @@ METRIC = "Nystrom attention tokens*heads/s"
 # for the sources of the kernel they were taken with: reported as null once any
 # of those files changes.
 MEASURED_TRAFFIC = {
-    "sr720p-w16-m16-bf16": {"files": ["common.cuh", "nystra_team.cuh", "nystra_tc.cuh", "nystra_tc_n256.cu",
-                                      "ptx.cuh"],
-        "src_hash": "1b521d4f6ce92163", "bytes": 995_407_360 + 273_398_784},
-    "sr720p-w32-m16-bf16": {"files": ["common.cuh", "nystra_stream.cuh", "nystra_tc.cuh", "nystra_tc_n1024.cu",
-                                      "ptx.cuh"],
-        "src_hash": "e847d1950a7301d2", "bytes": 1_030_822_656 + 284_172_544},
-    "large-w16-m64": {"files": ["common.cuh", "nystra_tc.cuh", "nystra_tc_n256.cu", "nystra_team.cuh", "ptx.cuh"],
-        "src_hash": "8e80904b0aac3611", "bytes": 245_142_272},
+    "sr720p-w16-m16-bf16": {"files": ["common.cuh", "nystra_symcore.cuh", "nystra_tc.cuh", "nystra_tc_n256.cu",
+                                      "nystra_team.cuh", "ptx.cuh"],
+        "src_hash": "435f97ddcca932f7", "bytes": 995_405_568 + 272_768_256},
+    "sr720p-w32-m16-bf16": {"files": ["common.cuh", "nystra_stream.cuh", "nystra_symcore.cuh", "nystra_tc.cuh",
+                                      "nystra_tc_n1024.cu", "ptx.cuh"],
+        "src_hash": "496706704270e7cc", "bytes": 1_030_630_912 + 282_295_040},
+    "large-w16-m64": {"files": ["common.cuh", "nystra_symcore.cuh", "nystra_tc.cuh", "nystra_tc_n256.cu",
+                                "nystra_wide.cuh", "ptx.cuh"],
+        "src_hash": "2c0e782ac1785fcb", "bytes": 202_585_856 + 44_934_400},
     "sr720p-w32-m16-bf16-qkv": {"files": ["common.cuh", "nystra_pool.cuh", "nystra_qkv.cuh", "nystra_qkv_stream.cuh",
-                                          "nystra_qkvs_bf16.cu", "nystra_tc.cuh", "ptx.cuh"],
-        "src_hash": "0ecb2b5c71d59518", "bytes": 640_227_072},
+                                          "nystra_qkvs_bf16.cu", "nystra_symcore.cuh", "nystra_tc.cuh", "ptx.cuh"],
+        "src_hash": "8c957484c1085eaa", "bytes": 347_453_440 + 289_935_104},
 }
 
 
